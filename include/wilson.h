@@ -146,9 +146,8 @@ typedef struct {
                             hop D_eo x_o per rhs.  The odd half is the rounding of
                             the rebuild either way.                                  */
     int    outer_blocks_per_sm; /* FP64 outer loop: 0 (default) launches the residual
-                            hops with the autotuned full grid; 1 or 2 launches them as
-                            a grid-stride kernel of that many 128-thread blocks per SM.
-                            The FP64 hop is bound by the FP64 pipe and needs few warps;
+                            hops with the full grid; 1 or 2 launches them as
+                            a grid-stride kernel of that many 128-thread blocks per SM:
                             the small grid leaves the rest of each SM to work on other
                             streams, such as the inner solve of another batch of
                             sources solved at the same time on another handle.      */
@@ -240,7 +239,10 @@ int wilson_hop(wl_gauge *g, const void *in, void *out, const void *x, double coe
  * launch; rhs_block (1, 2 or 4) rhs are handled by one thread, which then
  * loads each link into registers once for all of them; rhs_block = 0 uses
  * the variant chosen by wl_autotune for (prec, n_rhs), or 1 if untuned; a
- * negative rhs_block selects the autotuner variant -rhs_block directly. */
+ * negative rhs_block selects the autotuner variant -rhs_block directly.
+ * FP64 hops run in block fixed point on the integer pipes (64-bit integers
+ * scaled per site, closer to the exact sum than FP64 arithmetic) for every
+ * rhs_block >= 0; the FP64-pipe hops stay selectable as variants. */
 int wilson_hop_multi(wl_gauge *g, const void *in, void *out, const void *x, double coef, int prec,
                      int out_parity, int dagger, int n_rhs, size_t rhs_stride, int rhs_block, void *stream);
 

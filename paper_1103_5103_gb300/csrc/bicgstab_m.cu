@@ -422,7 +422,7 @@ extern "C" int bicgstab_m_solve(wl_gauge *g, const void *b, void *const *x, cons
     MState *mst = reinterpret_cast<MState *>(static_cast<char *>(pst) + sizeof(BiState));
     ShiftState *sh = reinterpret_cast<ShiftState *>(static_cast<char *>(pst) + sizeof(BiState) + sizeof(MState));
     void *ppart;
-    WL_TRY(g->ws.get("bm_partials", sizeof(double) * 2 * nsb * kRedNV, &ppart));
+    WL_TRY(g->ws.get("bm_partials", sizeof(double) * 4 * nsb * kRedNV, &ppart));
     double *partials = static_cast<double *>(ppart);
     void *pn;
     WL_TRY(g->ws.get("bm_norm", sizeof(double) * 8 + sizeof(unsigned) * 4, &pn));
@@ -500,14 +500,14 @@ extern "C" int bicgstab_m_solve(wl_gauge *g, const void *b, void *const *x, cons
         Vec se = half_of(sv, 0), so = half_of(sv, 1), te = half_of(t, 0), to = half_of(t, 1);
         Vec rhe = half_of(rhat, 0), rho = half_of(rhat, 1);
         // v = A p, <rhat, v> -> alpha
-        WL_TRY(hop_reduce(g, 0, po, pe, a1, ve, rhe, -0.5, nullptr, WL_EVEN, 0, st, partials, 0, 2 * nsb, q));
-        WL_TRY(hop_reduce(g, 0, pe, po, a1, vo, rho, -0.5, nullptr, WL_ODD, 0, st, partials, nsb, 2 * nsb, q));
+        WL_TRY(hop_reduce(g, 0, po, pe, a1, ve, rhe, -0.5, nullptr, WL_EVEN, 0, st, partials, 0, 2, q));
+        WL_TRY(hop_reduce(g, 0, pe, po, a1, vo, rho, -0.5, nullptr, WL_ODD, 0, st, partials, 1, 2, q));
         if (P == WL_DF) k_m_s<WL_DF><<<2 * nsb, kBlock, 0, q>>>(geo, nsb, r, v, sv, st);
         else k_m_s<WL_F64><<<2 * nsb, kBlock, 0, q>>>(geo, nsb, r, v, sv, st);
         note_launch(q);
         // t = A s, <t,s>, <t,t> -> omega
-        WL_TRY(hop_reduce(g, 1, so, se, a1, te, rhe, -0.5, nullptr, WL_EVEN, 0, st, partials, 0, 2 * nsb, q));
-        WL_TRY(hop_reduce(g, 1, se, so, a1, to, rho, -0.5, nullptr, WL_ODD, 0, st, partials, nsb, 2 * nsb, q));
+        WL_TRY(hop_reduce(g, 1, so, se, a1, te, rhe, -0.5, nullptr, WL_EVEN, 0, st, partials, 0, 2, q));
+        WL_TRY(hop_reduce(g, 1, se, so, a1, to, rho, -0.5, nullptr, WL_ODD, 0, st, partials, 1, 2, q));
         if (ns) {
             k_shift_a<<<1, 32, 0, q>>>(sh, ns, st, mst);
             note_launch(q);

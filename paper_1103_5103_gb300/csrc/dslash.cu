@@ -44,6 +44,8 @@ int hop_ex(wl_gauge *g, const Vec &in, const Vec &out, const Vec *x1, double a1,
     a.rhs_bytes = in.rhs_bytes;
     a.links_out = links_of(g, in.prec, out_parity);
     a.links_in = links_of(g, in.prec, 1 - out_parity);
+    a.fix_out = g->fix_links[out_parity];
+    a.fix_in = g->fix_links[1 - out_parity];
     a.skip = skip;
     a.skip_stride = skip_stride;
     EpiStore e;
@@ -78,10 +80,18 @@ int hop(wl_gauge *g, const Vec &in, const Vec &out, const Vec *x, double coef, i
     return hop_ex(g, in, out, x, 1.0, nullptr, 0.0, coef, out_parity, dagger, rhs_block, nullptr, 0, s);
 }
 
+// Blocks of a reduction-fused hop over one parity: 128 sites each, 64 in the
+// fixed-point FP64 hop (two threads per site).
+static int reduce_blocks(const wl_gauge *g, int prec)
+{
+    const Geom &geo = g->lat->geom;
+    return prec == WL_F64 && g->fix_links[0] ? (geo.Vh + 63) / 64 : site_blocks(geo);
+}
+
 template <int KIND>
 static int hop_reduce_k(wl_gauge *g, const Vec &tmp, const Vec &xin, double a1, const Vec &out, const Vec &rhat,
                         double coef, const double *coef_dev, int out_parity, int dagger, BiState *state,
-                        double *partials, int blk_off, int blk_total, cudaStream_t s)
+                        double *partials, int part, int parts, cudaStream_t s)
 {
     WL_TRY(check_links(g, tmp.prec));
     HopArgs a;
@@ -93,6 +103,8 @@ static int hop_reduce_k(wl_gauge *g, const Vec &tmp, const Vec &xin, double a1, 
     a.rhs_bytes = tmp.rhs_bytes;
     a.links_out = links_of(g, tmp.prec, out_parity);
     a.links_in = links_of(g, tmp.prec, 1 - out_parity);
+    a.fix_out = g->fix_links[out_parity];
+    a.fix_in = g->fix_links[1 - out_parity];
     a.skip = &state[0].done;
     a.skip_stride = sizeof(BiState) / sizeof(int);
     EpiReduce<KIND> e;
@@ -102,8 +114,9 @@ static int hop_reduce_k(wl_gauge *g, const Vec &tmp, const Vec &xin, double a1, 
     e.a1 = a1;
     e.coef = coef;
     e.coef_dev = coef_dev;
-    e.blk_off = blk_off;
-    e.blk_total = blk_total;
+    const int nblk = reduce_blocks(g, tmp.prec);
+    e.blk_off = part * nblk;
+    e.blk_total = parts * nblk;
     e.rhs_bytes = out.rhs_bytes;
     e.st = state;
     e.partials = partials;
@@ -123,17 +136,17 @@ static int hop_reduce_k(wl_gauge *g, const Vec &tmp, const Vec &xin, double a1, 
 
 int hop_reduce(wl_gauge *g, int kind, const Vec &tmp, const Vec &xin, double a1, const Vec &out, const Vec &rhat,
                double coef, const double *coef_dev, int out_parity, int dagger, BiState *state, double *partials,
-               int blk_off, int blk_total, cudaStream_t s)
+               int part, int parts, cudaStream_t s)
 {
     switch (kind) {
     case 0: return hop_reduce_k<0>(g, tmp, xin, a1, out, rhat, coef, coef_dev, out_parity, dagger, state, partials,
-                                   blk_off, blk_total, s);
+                                   part, parts, s);
     case 1: return hop_reduce_k<1>(g, tmp, xin, a1, out, rhat, coef, coef_dev, out_parity, dagger, state, partials,
-                                   blk_off, blk_total, s);
+                                   part, parts, s);
     case 2: return hop_reduce_k<2>(g, tmp, xin, a1, out, rhat, coef, coef_dev, out_parity, dagger, state, partials,
-                                   blk_off, blk_total, s);
+                                   part, parts, s);
     case 3: return hop_reduce_k<3>(g, tmp, xin, a1, out, rhat, coef, coef_dev, out_parity, dagger, state, partials,
-                                   blk_off, blk_total, s);
+                                   part, parts, s);
     default: set_error("hop_reduce: bad kind"); return WL_ERR_ARG;
     }
 }

@@ -99,6 +99,8 @@ struct HopArgs {
     size_t rhs_bytes;
     const void *links_out;       // links at the output parity (forward links)
     const void *links_in;        // links at the input parity (backward links)
+    const void *fix_out;         // the same as integers for the fixed-point FP64 hop (or null)
+    const void *fix_in;
     const int *skip;             // optional per-rhs flags: skip rhs r when skip[r * skip_stride] != 0
     int skip_stride;
 };
@@ -967,6 +969,64 @@ void launch_k_hop_gs(HopArgs a, const EpiStore &e, cudaStream_t s)
     k_hop_gs<P, DAG, NB, MINB><<<MINB * sm_count(), 128, 0, s>>>(a, e);
 }
 
+// Last step of the reduction-fused hops: the block's partial sums red, and by
+// the last block the scalars they give.
+template <int KIND, typename RedT>
+__device__ __forceinline__ void hop_reduce_finish(const EpiReduce<KIND> &e, BiState &st, int r, int sb,
+                                                  RedT (&red)[EpiReduce<KIND>::NV])
+{
+    constexpr int NV = EpiReduce<KIND>::NV;
+    double tot[NV];
+    if (grid_sum<NV>(red, e.partials + (size_t)r * e.blk_total * kRedNV, &st.ticket[KIND], e.blk_off + sb,
+                     e.blk_total, tot) &&
+        threadIdx.x == 0) {
+        if constexpr (KIND == 0) {
+            const double dr = tot[0], di = tot[1];
+            const double den = dr * dr + di * di;
+            if (!(den > st.brk2 * st.rhat2 * tot[2]) || !isfinite(den)) {
+                st.breakdown = 1;
+                st.done = 1;
+            } else {  // alpha = rho / <rhat, v>
+                st.alpha_re = (st.rho_re * dr + st.rho_im * di) / den;
+                st.alpha_im = (st.rho_im * dr - st.rho_re * di) / den;
+            }
+        } else if constexpr (KIND == 1) {
+            const double tt = tot[2];
+            if (tt > 0.0 && isfinite(tt)) {
+                st.omega_re = tot[0] / tt;
+                st.omega_im = tot[1] / tt;
+            } else {
+                st.omega_re = 0.0;
+                st.omega_im = 0.0;
+            }
+        } else if constexpr (KIND == 2) {
+            // CG on the normal equations: w = M p, alpha = ||z||^2 / ||w||^2
+            const double ww = tot[2];
+            if (!(ww > 0.0) || !isfinite(ww)) {
+                st.breakdown = 1;
+                st.done = 1;
+            } else {
+                st.alpha_re = st.rho_re / ww;
+                st.alpha_im = 0.0;
+            }
+        } else {
+            // z = M^dag r, beta = ||z||^2 / ||z_old||^2 (0 on the first z
+            // after a restart), rho = ||z||^2
+            const double zz = tot[2];
+            if (!isfinite(zz)) {
+                st.breakdown = 1;
+                st.done = 1;
+            } else {
+                st.beta_re = (st.iters == 0 || !(st.rho_re > 0.0)) ? 0.0 : zz / st.rho_re;
+                st.beta_im = 0.0;
+                st.omega_re = st.omega_im = 0.0;
+                st.rho_re = zz;
+                st.rho_im = 0.0;
+            }
+        }
+    }
+}
+
 template <int P, bool DAG, int KIND>
 __device__ __forceinline__ void hop_reduce_body(const HopArgs &a, const EpiReduce<KIND> &e)
 {
@@ -1035,55 +1095,7 @@ __device__ __forceinline__ void hop_reduce_body(const HopArgs &a, const EpiReduc
             red[2] = red_cast<RedT>(n);
         }
     }
-    double tot[NV];
-    if (grid_sum<NV>(red, e.partials + (size_t)r * e.blk_total * kRedNV, &st.ticket[KIND], e.blk_off + sb,
-                     e.blk_total, tot) &&
-        threadIdx.x == 0) {
-        if constexpr (KIND == 0) {
-            const double dr = tot[0], di = tot[1];
-            const double den = dr * dr + di * di;
-            if (!(den > st.brk2 * st.rhat2 * tot[2]) || !isfinite(den)) {
-                st.breakdown = 1;
-                st.done = 1;
-            } else {  // alpha = rho / <rhat, v>
-                st.alpha_re = (st.rho_re * dr + st.rho_im * di) / den;
-                st.alpha_im = (st.rho_im * dr - st.rho_re * di) / den;
-            }
-        } else if constexpr (KIND == 1) {
-            const double tt = tot[2];
-            if (tt > 0.0 && isfinite(tt)) {
-                st.omega_re = tot[0] / tt;
-                st.omega_im = tot[1] / tt;
-            } else {
-                st.omega_re = 0.0;
-                st.omega_im = 0.0;
-            }
-        } else if constexpr (KIND == 2) {
-            // CG on the normal equations: w = M p, alpha = ||z||^2 / ||w||^2
-            const double ww = tot[2];
-            if (!(ww > 0.0) || !isfinite(ww)) {
-                st.breakdown = 1;
-                st.done = 1;
-            } else {
-                st.alpha_re = st.rho_re / ww;
-                st.alpha_im = 0.0;
-            }
-        } else {
-            // z = M^dag r, beta = ||z||^2 / ||z_old||^2 (0 on the first z
-            // after a restart), rho = ||z||^2
-            const double zz = tot[2];
-            if (!isfinite(zz)) {
-                st.breakdown = 1;
-                st.done = 1;
-            } else {
-                st.beta_re = (st.iters == 0 || !(st.rho_re > 0.0)) ? 0.0 : zz / st.rho_re;
-                st.beta_im = 0.0;
-                st.omega_re = st.omega_im = 0.0;
-                st.rho_re = zz;
-                st.rho_im = 0.0;
-            }
-        }
-    }
+    hop_reduce_finish<KIND>(e, st, r, sb, red);
 }
 
 // Resident blocks per SM the reduction-fused hop asks the register
@@ -1141,6 +1153,10 @@ constexpr int WL_VARIANT_NA = -100;
 
 // TMA-staged hop (hop_tma.cu), FP32 and FP16, variants 9000 + rhs per tile.
 int hop_launch_tma(int prec, int variant, int dagger, const HopArgs &a, const EpiStore &e, cudaStream_t s);
+
+// Fixed-point FP64 hop (hop_fix.cu).
+int hop_fix_launch(int dagger, const HopArgs &a, const EpiStore &e, int blocks_per_sm, cudaStream_t s);
+int hop_fix_reduce_launch(int kind, int dagger, const HopArgs &a, const void *epi, cudaStream_t s);
 
 // Per-precision entry points (hop_<prec>.cu).  variant: see hop_variants().
 template <int P> int hop_launch_prec(int variant, int dagger, const HopArgs &a, const EpiStore &e, cudaStream_t s);

@@ -1,7 +1,9 @@
 // Hop kernel instantiations for F64 (one translation unit per precision so the
 // library builds in parallel).  Variant v = 100 * (rhs per thread) + (minimum resident
 // blocks per SM requested from the register allocator); v = 7000 + 100 * (rhs per
-// thread) + B is the grid-stride form with B blocks per SM (k_hop_gs).
+// thread) + B is the grid-stride form with B blocks per SM (k_hop_gs); 6000 is the fixed-
+// point hop (hop_fix.cuh), which every FP64 hop takes unless one of the others is named,
+// 6000 + B the same with B looping blocks per SM.
 #include "hop.cuh"
 
 namespace wl {
@@ -10,6 +12,10 @@ namespace wl {
 template <>
 int hop_launch_prec<WL_F64>(int v, int dagger, const HopArgs &a, const EpiStore &e, cudaStream_t s)
 {
+    if (v >= 6000 && v <= 6002) {
+        if (!a.fix_out) return WL_VARIANT_NA;   // no integer links on this handle
+        return hop_fix_launch(dagger, a, e, v - 6000, s);
+    }
     if (dagger) {
         switch (v / 100) {
         case 1: launch_k_hop<WL_F64, true, 1, 1>(a, e, s); break;
@@ -40,6 +46,7 @@ int hop_launch_prec<WL_F64>(int v, int dagger, const HopArgs &a, const EpiStore 
 template <>
 int hop_reduce_launch_prec<WL_F64>(int kind, int dagger, const HopArgs &a, const void *epi, cudaStream_t s)
 {
+    if (a.fix_out) return hop_fix_reduce_launch(kind, dagger, a, epi, s);
     switch (kind) {
     case 0: launch_reduce_kind<WL_F64, 0>(dagger, a, epi, s); break;
     case 1: launch_reduce_kind<WL_F64, 1>(dagger, a, epi, s); break;

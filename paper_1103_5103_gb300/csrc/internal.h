@@ -81,6 +81,7 @@ struct wl_gauge {
     wl_lattice *lat;
     unsigned prec_mask;
     void *links[4][2];  // [prec index][parity] -> 4 directions of 12-real links
+    void *fix_links[2] = {nullptr, nullptr};  // [parity] FP64 links as integers (hop_fix.cuh); null without memory for them
     wl::Workspace ws;
     wl::HostPinned pinned;
     std::mutex mu;      // one solve at a time per handle (shared workspace)
@@ -119,14 +120,15 @@ int hop(wl_gauge *g, const Vec &in, const Vec &out, const Vec *x, double coef, i
         int rhs_block, cudaStream_t s);
 
 // Fused solver hops: second half of an operator application followed by the
-// BiCGstab reductions; blk_off / blk_total place this launch's blocks in a
-// reduction spread over several launches (full-lattice vectors).
+// BiCGstab reductions; this launch is part `part` of `parts` launches of one
+// reduction (full-lattice vectors: one launch per parity).  partials holds
+// parts * 2 * site_blocks * kRedNV doubles per rhs.
 //   kind 0:  v = a1 * xin + coef * D tmp;  <rhat, v>        -> alpha = rho / <rhat, v>
 //   kind 1:  t = a1 * xin + coef * D tmp;  <t, xin>, <t, t> -> omega
 // coef_dev (optional, device) overrides coef at run time.
 int hop_reduce(wl_gauge *g, int kind, const Vec &tmp, const Vec &xin, double a1, const Vec &out, const Vec &rhat,
                double coef, const double *coef_dev, int out_parity, int dagger, BiState *state, double *partials,
-               int blk_off, int blk_total, cudaStream_t s);
+               int part, int parts, cudaStream_t s);
 
 // ---- blas.cu (all on one parity; nrhs from the vectors)
 int blas_s_update(const Geom &g, const Vec &r, const Vec &v, const Vec &s_out, BiState *st, cudaStream_t s);

@@ -276,6 +276,27 @@ __global__ void k_pack_links(Geom g, const double2 *__restrict__ U, void *out, i
     }
 }
 
+// FP64 links as integers in units of 2^-62 for the fixed-point hop
+// (hop_fix.cuh): int4 [4][stride / 32][9][32], an entry as the balanced
+// 32-bit limbs re.lo, re.hi, im.lo, im.hi.
+__global__ void k_pack_fix(Geom g, const double2 *__restrict__ U, int4 *out, int parity)
+{
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    const int mu = blockIdx.y;
+    if (i >= g.Vh) return;
+    const Coord c = site_coord(g, i, parity);
+    const size_t V = (size_t)g.Vh * 2;
+    const size_t lex = c.x + (size_t)g.X * (c.y + (size_t)g.Y * (c.z + (size_t)g.Z * c.t));
+    const double2 *u = U + ((size_t)mu * V + lex) * 9;
+    int4 *p = out + (size_t)mu * 9 * g.stride + (size_t)(i >> 5) * (9 * 32) + (i & 31);
+    for (int k = 0; k < 9; ++k) {
+        const double2 z = u[k];
+        const long long re = __double2ll_rn(z.x * 0x1p62), im = __double2ll_rn(z.y * 0x1p62);
+        p[k * 32] =
+            make_int4((int)re, (int)((re + (1ll << 31)) >> 32), (int)im, (int)((im + (1ll << 31)) >> 32));
+    }
+}
+
 template <int P>
 static int launch_import(const Geom &g, const void *canon, void *out, int parity, cudaStream_t s)
 {
@@ -606,6 +627,28 @@ extern "C" int wl_gauge_create(wl_lattice *lat, const void *U, unsigned prec_mas
             note_launch(s);
         }
     }
+    if (prec_mask & WL_F64) {
+        // the integer links of the fixed-point FP64 hop; without the memory
+        // for them FP64 hops run on the FP64 pipe
+        const size_t bytes = (size_t)4 * 9 * sizeof(int4) * geo.stride;
+        for (int par = 0; par < 2; ++par)
+            if (cudaMalloc(&g->fix_links[par], bytes) != cudaSuccess) {
+                cudaGetLastError();
+                g->fix_links[par] = nullptr;
+            }
+        if (!g->fix_links[0] || !g->fix_links[1]) {
+            for (int par = 0; par < 2; ++par) {
+                if (g->fix_links[par]) cudaFree(g->fix_links[par]);
+                g->fix_links[par] = nullptr;
+            }
+        } else {
+            for (int par = 0; par < 2; ++par) {
+                k_pack_fix<<<dim3((geo.Vh + 127) / 128, 4), 128, 0, s>>>(
+                    geo, static_cast<const double2 *>(U), static_cast<int4 *>(g->fix_links[par]), par);
+                note_launch(s);
+            }
+        }
+    }
     cudaError_t e = cudaStreamSynchronize(s);
     if (e == cudaSuccess) e = cudaGetLastError();
     if (e != cudaSuccess) {
@@ -624,6 +667,8 @@ extern "C" int wl_gauge_destroy(wl_gauge *g)
     for (int pi = 0; pi < 4; ++pi)
         for (int par = 0; par < 2; ++par)
             if (g->links[pi][par]) cudaFree(g->links[pi][par]);
+    for (int par = 0; par < 2; ++par)
+        if (g->fix_links[par]) cudaFree(g->fix_links[par]);
     g->inner_graph.release();
     g->ws.release();
     g->pinned.release();

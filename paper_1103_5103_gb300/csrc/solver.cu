@@ -115,7 +115,7 @@ static int cg_normal_residual(Inner &in, int rhs_block, cudaStream_t s)
     const int ss = sizeof(BiState) / sizeof(int);
     WL_TRY(hop_ex(in.g, in.r, in.tmp, nullptr, 0.0, nullptr, 0.0, 1.0, WL_ODD, 1, rhs_block, skip, ss, s));
     WL_TRY(hop_reduce(in.g, 3, in.tmp, in.r, 1.0, in.s, in.rhat, 0.0, in.sc.kappa2, WL_EVEN, 1, in.sc.state,
-                      in.sc.partials, 0, site_blocks(geo), s));
+                      in.sc.partials, 0, 1, s));
     // omega = 0, so the BiCGstab p update reduces to p = z + beta p
     WL_TRY(blas_p_update(geo, in.s, in.p, in.p, in.sc.state, s));
     return WL_OK;
@@ -126,7 +126,6 @@ static int cg_normal_residual(Inner &in, int rhs_block, cudaStream_t s)
 static int inner_iteration(Inner &in, int rhs_block, cudaStream_t s, cudaEvent_t *ev = nullptr)
 {
     const Geom &geo = in.g->lat->geom;
-    const int nsb = site_blocks(geo);
     const int *skip = &in.sc.state[0].done;
     const int ss = sizeof(BiState) / sizeof(int);
     const double *k2 = in.sc.kappa2;  // -kappa^2, set per mass before the graph runs
@@ -143,11 +142,11 @@ static int inner_iteration(Inner &in, int rhs_block, cudaStream_t s, cudaEvent_t
     WL_TRY(hop_ex(in.g, in.p, in.tmp, nullptr, 0.0, nullptr, 0.0, 1.0, WL_ODD, 0, rhs_block, skip, ss, s));
     if (ev) WL_CUDA_TRY(cudaEventRecordWithFlags(ev[1], s, evflags));
     WL_TRY(hop_reduce(in.g, 0, in.tmp, in.p, 1.0, in.v, in.rhat, 0.0, k2, WL_EVEN, 0, in.sc.state, in.sc.partials,
-                      0, nsb, s));
+                      0, 1, s));
     WL_TRY(blas_s_update(geo, in.r, in.v, in.s, in.sc.state, s));
     WL_TRY(hop_ex(in.g, in.s, in.tmp, nullptr, 0.0, nullptr, 0.0, 1.0, WL_ODD, 0, rhs_block, skip, ss, s));
     WL_TRY(hop_reduce(in.g, 1, in.tmp, in.s, 1.0, in.t, in.rhat, 0.0, k2, WL_EVEN, 0, in.sc.state, in.sc.partials,
-                      0, nsb, s));
+                      0, 1, s));
     WL_TRY(blas_xr_update(geo, in.e, in.p, in.s, in.t, in.r, in.rhat, in.sc.state, in.sc.partials, s));
     WL_TRY(blas_p_update(geo, in.r, in.p, in.v, in.sc.state, s));
     return WL_OK;
@@ -162,7 +161,6 @@ static int inner_iteration(Inner &in, int rhs_block, cudaStream_t s, cudaEvent_t
 static int inner_iteration_cg(Inner &in, int rhs_block, cudaStream_t s, cudaEvent_t *ev = nullptr)
 {
     const Geom &geo = in.g->lat->geom;
-    const int nsb = site_blocks(geo);
     const int *skip = &in.sc.state[0].done;
     const int ss = sizeof(BiState) / sizeof(int);
     const double *k2 = in.sc.kappa2;
@@ -176,7 +174,7 @@ static int inner_iteration_cg(Inner &in, int rhs_block, cudaStream_t s, cudaEven
     WL_TRY(hop_ex(in.g, in.p, in.tmp, nullptr, 0.0, nullptr, 0.0, 1.0, WL_ODD, 0, rhs_block, skip, ss, s));
     if (ev) WL_CUDA_TRY(cudaEventRecordWithFlags(ev[1], s, evflags));
     WL_TRY(hop_reduce(in.g, 2, in.tmp, in.p, 1.0, in.v, in.rhat, 0.0, k2, WL_EVEN, 0, in.sc.state, in.sc.partials,
-                      0, nsb, s));
+                      0, 1, s));
     WL_TRY(blas_cg_xr(geo, in.e, in.p, in.v, in.r, in.sc.state, in.sc.partials, s));
     WL_TRY(cg_normal_residual(in, rhs_block, s));
     return WL_OK;
@@ -399,9 +397,9 @@ static int eo_defect_correction(wl_gauge *g, const Vec &bprec, const Vec &x64, d
     WL_CUDA_TRY(cudaMemsetAsync(in.sc.outer_done, 0, sizeof(int) * nrhs, s));
     int total_restarts = 0;
     bool lincomb_check = r0_given;
-    // outer residual hops: autotuned full grid, or the FP64 grid-stride form
+    // outer residual hops: full grid, or the FP64 grid-stride form
     const int ohop = (prm.outer_blocks_per_sm > 0 && x64.prec == WL_F64)
-                         ? -(7000 + 100 * (nrhs >= 2 ? 2 : 1) + prm.outer_blocks_per_sm)
+                         ? -((g->fix_links[0] ? 6000 : 7000 + 100 * (nrhs >= 2 ? 2 : 1)) + prm.outer_blocks_per_sm)
                          : 0;
     // Three levels for FP16 inner solves (prm.inner_refine): an FP16 BiCGstab
     // stops near 3e-4 of its starting residual, where the FP16 rounding of its

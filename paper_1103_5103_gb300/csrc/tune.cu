@@ -5,6 +5,7 @@
 // caches the fastest in the gauge handle.  With WL_AUTOTUNE_CACHE set to a
 // file path the choices are also read from / appended to that file, keyed by
 // lattice extents, precision, rhs count and device name.
+#include <algorithm>
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
@@ -22,7 +23,7 @@ const std::vector<int> &hop_variants(int prec)
                                          5006, 9001, 9002, 9004, 9102, 9104};
     static const std::vector<int> f16 = {101, 105, 106, 108, 110, 201, 204, 206, 401, 404, 5006,
                                          9001, 9002, 9004, 9102, 9104};
-    static const std::vector<int> f64 = {101, 103, 201, 7101, 7102, 7201, 7202};
+    static const std::vector<int> f64 = {101, 103, 201, 6000, 6001, 6002, 7101, 7102, 7201, 7202};
     static const std::vector<int> dfv = {101, 103, 104, 105, 106};
     static const std::vector<int> none;
     switch (prec) {
@@ -37,6 +38,10 @@ const std::vector<int> &hop_variants(int prec)
 int hop_variant_for(wl_gauge *g, int prec, int nrhs, int rhs_block)
 {
     if (rhs_block < 0) return -rhs_block;
+    // FP64: the fixed-point hop at every size (8^4 14 against 35 us, 24^3x64
+    // with three rhs 0.70 against 2.0 ms of the FP64-pipe hops); it shares the
+    // links of several rhs through L1 and has no rhs-per-thread form
+    if (prec == WL_F64 && g->fix_links[0]) return 6000;
     if (rhs_block > 0) return rhs_block * 100 + 1;
     auto it = g->tune.find(std::make_pair(prec, nrhs));
     return it == g->tune.end() ? 101 : it->second.variant;
@@ -63,7 +68,8 @@ int autotune_hop(wl_gauge *g, int prec, int nrhs, cudaStream_t s, TuneResult *ou
         if (out) *out = it->second;
         return WL_OK;
     }
-    const std::vector<int> &vs = hop_variants(prec);
+    static const std::vector<int> fix = {6000};   // the only FP64 candidate (hop_variant_for)
+    const std::vector<int> &vs = prec == WL_F64 && g->fix_links[0] ? fix : hop_variants(prec);
     if (vs.empty()) { set_error("autotune: bad precision"); return WL_ERR_ARG; }
     TuneResult best;
     const char *path = std::getenv("WL_AUTOTUNE_CACHE");
@@ -75,7 +81,7 @@ int autotune_hop(wl_gauge *g, int prec, int nrhs, cudaStream_t s, TuneResult *ou
             if (line.compare(0, fkey.size(), fkey) == 0 && line.size() > fkey.size() && line[fkey.size()] == ' ') {
                 std::istringstream is(line.substr(fkey.size() + 1));
                 TuneResult r;
-                if (is >> r.variant >> r.us) best = r;
+                if (is >> r.variant >> r.us && std::find(vs.begin(), vs.end(), r.variant) != vs.end()) best = r;
             }
         }
         if (best.variant > 0) {
