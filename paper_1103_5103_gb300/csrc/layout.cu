@@ -135,18 +135,39 @@ __global__ void k_import(Geom g, const double2 *__restrict__ canon, void *out, i
     SpinorIO<P>::store(out, g.stride, i, v);
 }
 
+// Export of one parity through shared memory: a block takes 128 consecutive
+// sites of the parity, whose canonical spinors are 192-byte pieces (12
+// complex) of a 48 KB stretch, and writes them piece by piece with 12
+// neighbouring lanes.  With one site per thread each 16-byte store of a warp
+// goes to 32 lines: 66 us against 27.5 us for 127 MB (FP32, 24^3x64).  The
+// import above keeps one site per thread: its loads hit L1 for the rest of
+// the line (27.6 us; 40 us when staged like this).  The staging buffer is
+// component-major with a stride of 129 (no bank conflicts).
+constexpr int kLayoutSites = 128;
+
 template <int P>
-__global__ void k_export(Geom g, const void *in, double2 *__restrict__ canon, int parity)
+__global__ void __launch_bounds__(kLayoutSites) k_export(Geom g, const void *in, double2 *__restrict__ canon,
+                                                         int parity)
 {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= g.Vh) return;
-    const Coord c = site_coord(g, i, parity);
-    const size_t lex = c.x + (size_t)g.X * (c.y + (size_t)g.Y * (c.z + (size_t)g.Z * c.t));
-    using R = typename PrecTraits<P>::R;
-    cx<R> v[12];
-    SpinorIO<P>::load(in, g.stride, i, v);
+    __shared__ double2 sm[12 * (kLayoutSites + 1)];
+    __shared__ unsigned off[kLayoutSites];
+    const int i0 = blockIdx.x * kLayoutSites, n = min(kLayoutSites, g.Vh - i0);
+    if ((int)threadIdx.x < n) {
+        // canonical offset in complex numbers (12 V < 2^31)
+        off[threadIdx.x] = 12u * (2u * (unsigned)(i0 + threadIdx.x) + (unsigned)(site_coord(g, i0 + threadIdx.x, parity).x & 1));
+        using R = typename PrecTraits<P>::R;
+        cx<R> v[12];
+        SpinorIO<P>::load(in, g.stride, i0 + threadIdx.x, v);
 #pragma unroll
-    for (int k = 0; k < 12; ++k) canon[lex * 12 + k] = make_double2(to_double(v[k].re), to_double(v[k].im));
+        for (int k = 0; k < 12; ++k)
+            sm[k * (kLayoutSites + 1) + threadIdx.x] = make_double2(to_double(v[k].re), to_double(v[k].im));
+    }
+    __syncthreads();
+#pragma unroll
+    for (int j = 0; j < 12; ++j) {
+        const int e = j * kLayoutSites + threadIdx.x;
+        if (e < 12 * n) canon[(size_t)off[e / 12] + e % 12] = sm[(e % 12) * (kLayoutSites + 1) + e / 12];
+    }
 }
 
 // Both parities at once, through shared memory, so that the canonical side
@@ -310,7 +331,7 @@ static int launch_import(const Geom &g, const void *canon, void *out, int parity
 template <int P>
 static int launch_export(const Geom &g, const void *in, void *canon, int parity, cudaStream_t s)
 {
-    const int th = 128, bl = (g.Vh + th - 1) / th;
+    const int th = kLayoutSites, bl = (g.Vh + th - 1) / th;
     k_export<P><<<bl, th, 0, s>>>(g, in, static_cast<double2 *>(canon), parity);
     WL_CUDA_TRY(cudaGetLastError());
     note_launch(s);
