@@ -268,7 +268,7 @@ __global__ void __launch_bounds__(kBlock) k_m_update(Geom g, int nsb, Vec x, Vec
         red[2] = to_double(n);
     }
     double tot[3];
-    if (grid_sum<3>(red, partials, &S.ticket[2], blockIdx.x, 2 * nsb, tot) && threadIdx.x == 0) {
+    if (site_sum<3>(red, g, partials, 0, &S.ticket[2], blockIdx.x, 2 * nsb, tot) && threadIdx.x == 0) {
         const double r1re = tot[0], r1im = tot[1], rr = tot[2];
         S.iters += 1;
         S.rr = rr;
@@ -422,7 +422,7 @@ extern "C" int bicgstab_m_solve(wl_gauge *g, const void *b, void *const *x, cons
     MState *mst = reinterpret_cast<MState *>(static_cast<char *>(pst) + sizeof(BiState));
     ShiftState *sh = reinterpret_cast<ShiftState *>(static_cast<char *>(pst) + sizeof(BiState) + sizeof(MState));
     void *ppart;
-    WL_TRY(g->ws.get("bm_partials", sizeof(double) * 4 * nsb * kRedNV, &ppart));
+    WL_TRY(red_buffer(g, "bm_partials", 1, &ppart, s));
     double *partials = static_cast<double *>(ppart);
     void *pn;
     WL_TRY(g->ws.get("bm_norm", sizeof(double) * 8 + sizeof(unsigned) * 4, &pn));

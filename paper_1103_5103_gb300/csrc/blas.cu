@@ -120,7 +120,7 @@ __global__ void __launch_bounds__(kBlock) k_xr_update(Geom g, Vec x, Vec p, Vec 
         red[2] = n;
     }
     double tot[3];
-    if (grid_sum<3>(red, partials + (size_t)q.r * q.nsb * kRedNV, &S.ticket[2], q.sb, q.nsb, tot) &&
+    if (site_sum<3>(red, g, partials, q.r, &S.ticket[2], q.sb, q.nsb, tot) &&
         threadIdx.x == 0) {
         const double r1re = tot[0], r1im = tot[1], rr = tot[2];
         S.iters += 1;
@@ -208,7 +208,7 @@ __global__ void __launch_bounds__(kBlock) k_cg_xr(Geom g, Vec x, Vec p, Vec w, V
         red[0] = n;
     }
     double tot[1];
-    if (grid_sum<1>(red, partials + (size_t)q.r * q.nsb * kRedNV, &S.ticket[1], q.sb, q.nsb, tot) &&
+    if (site_sum<1>(red, g, partials, q.r, &S.ticket[1], q.sb, q.nsb, tot) &&
         threadIdx.x == 0) {
         const double rr = tot[0];
         S.iters += 1;
@@ -333,7 +333,7 @@ __global__ void __launch_bounds__(kBlock) k_restart(Geom g, Vec r64, Vec r, Vec 
         red[2] = n;
     }
     double tot[3];
-    if (grid_sum<3>(red, partials + (size_t)q.r * q.nsb * kRedNV, &S.ticket[3], q.sb, q.nsb, tot) &&
+    if (site_sum<3>(red, g, partials, q.r, &S.ticket[3], q.sb, q.nsb, tot) &&
         threadIdx.x == 0) {
         const double rr = tot[2];
         double bre = 0.0, bim = 0.0, ore = 0.0, oim = 0.0;
@@ -479,7 +479,7 @@ __global__ void __launch_bounds__(kBlock) k_norm2(Geom g, Vec a, double *out, do
         red[0] = n;
     }
     double tot[1];
-    if (grid_sum<1>(red, partials + (size_t)q.r * q.nsb * kRedNV, &tickets[q.r], q.sb, q.nsb, tot) &&
+    if (site_sum<1>(red, g, partials, q.r, &tickets[q.r], q.sb, q.nsb, tot) &&
         threadIdx.x == 0)
         out[q.r] = tot[0];
 }
@@ -756,7 +756,7 @@ __global__ void __launch_bounds__(kBlock) k_recon(Geom g, Vec bo, Vec dx, double
         red[0] = (double)n;
     }
     double tot[1];
-    if (grid_sum<1>(red, partials + (size_t)q.r * q.nsb * kRedNV, &tickets[q.r], q.sb, q.nsb, tot) &&
+    if (site_sum<1>(red, g, partials, q.r, &tickets[q.r], q.sb, q.nsb, tot) &&
         threadIdx.x == 0)
         norm2[q.r] = tot[0];
 }

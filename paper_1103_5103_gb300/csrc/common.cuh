@@ -766,12 +766,92 @@ __device__ __forceinline__ bool grid_finish(double (&v)[NV], double *partials, u
     double acc[NV];
 #pragma unroll
     for (int k = 0; k < NV; ++k) acc[k] = 0.0;
+#pragma unroll 4
     for (int b = threadIdx.x; b < nblk; b += blockDim.x)
 #pragma unroll
         for (int k = 0; k < NV; ++k) acc[k] += __ldcg(partials + (size_t)b * NV + k);
     block_sum<NV>(acc);
 #pragma unroll
     for (int k = 0; k < NV; ++k) tot[k] = acc[k];
+    if (threadIdx.x == 0) *ticket = 0u;
+    return true;
+}
+
+// Reduction over the site blocks of a lattice, as grid_sum, in two levels:
+// with one, the last block of a 48^3x96 launch adds 41,472 partials in 324
+// dependent rounds while the GPU idles (k_xr_update FP16 1 rhs: 684 us for
+// 2.4 GB).  Blocks form groups of 128; the last block of a group adds its
+// partials, one per thread, and the last group adds the group sums.  Up to
+// 1024 blocks take one level: the second one costs 2.5 us (another ticket
+// and two more trips to L2), eight rounds of one level less.  Fixed order
+// either way (deterministic).
+//
+// Buffer per rhs, red_doubles(g) doubles, zeroed when allocated: group
+// tickets (one per double; each resets itself), group sums, block partials,
+// for the largest number of blocks of any launch (two parities of 64-site
+// blocks).  blockDim.x >= 128.
+constexpr int kRedNV = 4;
+constexpr int kRedGroup = 128;
+constexpr int kRedOneLevel = 1024;
+__host__ __device__ inline int red_max_blocks(const Geom &g) { return 4 * ((g.Vh + 127) / 128); }
+__host__ __device__ inline int red_groups(const Geom &g) { return (red_max_blocks(g) + kRedGroup - 1) / kRedGroup; }
+__host__ __device__ inline size_t red_doubles(const Geom &g)
+{
+    return (size_t)red_groups(g) * (1 + kRedNV) + (size_t)red_max_blocks(g) * kRedNV;
+}
+
+template <int NV, typename T>
+__device__ __forceinline__ bool site_sum(T (&red)[NV], const Geom &g, double *partials, int r, unsigned *ticket,
+                                         int blk, int nblk, double (&tot)[NV])
+{
+    static_assert(NV <= kRedNV, "partial slots");
+    double *base = partials + (size_t)r * red_doubles(g);
+    const int ng = red_groups(g);
+    double *gsum = base + ng, *part = gsum + (size_t)ng * kRedNV;
+    if (nblk <= kRedOneLevel) return grid_sum<NV>(red, part, ticket, blk, nblk, tot);
+    double v[NV];
+    if constexpr (sizeof(T) == sizeof(float)) {
+        block_sum<NV>(red, v);
+    } else {
+        block_sum<NV>(red);
+#pragma unroll
+        for (int k = 0; k < NV; ++k) v[k] = red[k];
+    }
+    const int grp = blk / kRedGroup, first = grp * kRedGroup;
+    const int in_grp = min(kRedGroup, nblk - first), ngrp = (nblk + kRedGroup - 1) / kRedGroup;
+    unsigned *gt = reinterpret_cast<unsigned *>(base + grp);
+    __shared__ bool last_blk, last_grp;
+    if (threadIdx.x == 0) {
+#pragma unroll
+        for (int k = 0; k < NV; ++k) part[(size_t)blk * NV + k] = v[k];
+        __threadfence();
+        last_blk = atomicAdd(gt, 1u) == (unsigned)in_grp - 1;
+    }
+    __syncthreads();
+    if (!last_blk) return false;
+    __threadfence();
+#pragma unroll
+    for (int k = 0; k < NV; ++k)
+        v[k] = (int)threadIdx.x < in_grp ? __ldcg(part + (size_t)(first + threadIdx.x) * NV + k) : 0.0;
+    block_sum<NV>(v);
+    if (threadIdx.x == 0) {
+        *gt = 0u;
+#pragma unroll
+        for (int k = 0; k < NV; ++k) gsum[(size_t)grp * NV + k] = v[k];
+        __threadfence();
+        last_grp = atomicAdd(ticket, 1u) == (unsigned)ngrp - 1;
+    }
+    __syncthreads();
+    if (!last_grp) return false;
+    __threadfence();
+#pragma unroll
+    for (int k = 0; k < NV; ++k) v[k] = 0.0;
+    for (int b = threadIdx.x; b < ngrp; b += blockDim.x)
+#pragma unroll
+        for (int k = 0; k < NV; ++k) v[k] += __ldcg(gsum + (size_t)b * NV + k);
+    block_sum<NV>(v);
+#pragma unroll
+    for (int k = 0; k < NV; ++k) tot[k] = v[k];
     if (threadIdx.x == 0) *ticket = 0u;
     return true;
 }
@@ -799,8 +879,6 @@ struct BiState {
     unsigned ticket[4];         // last-block tickets, one per reduction site
 };
 
-// Reduction scratch: partials[(rhs * nblocks + block) * kRedNV + k].
-constexpr int kRedNV = 4;
 constexpr int kBlock = 128;  // threads per block of every site kernel
 inline int site_blocks(const Geom &g) { return (g.Vh + kBlock - 1) / kBlock; }
 

@@ -239,7 +239,7 @@ struct EpiReduce {
     int blk_off, blk_total;
     size_t rhs_bytes;
     BiState *st;
-    double *partials;   // [rhs][block][kRedNV]
+    double *partials;   // site_sum's buffer
     static constexpr int NV = 3;
 };
 
@@ -972,13 +972,12 @@ void launch_k_hop_gs(HopArgs a, const EpiStore &e, cudaStream_t s)
 // Last step of the reduction-fused hops: the block's partial sums red, and by
 // the last block the scalars they give.
 template <int KIND, typename RedT>
-__device__ __forceinline__ void hop_reduce_finish(const EpiReduce<KIND> &e, BiState &st, int r, int sb,
+__device__ __forceinline__ void hop_reduce_finish(const Geom &g, const EpiReduce<KIND> &e, BiState &st, int r, int sb,
                                                   RedT (&red)[EpiReduce<KIND>::NV])
 {
     constexpr int NV = EpiReduce<KIND>::NV;
     double tot[NV];
-    if (grid_sum<NV>(red, e.partials + (size_t)r * e.blk_total * kRedNV, &st.ticket[KIND], e.blk_off + sb,
-                     e.blk_total, tot) &&
+    if (site_sum<NV>(red, g, e.partials, r, &st.ticket[KIND], e.blk_off + sb, e.blk_total, tot) &&
         threadIdx.x == 0) {
         if constexpr (KIND == 0) {
             const double dr = tot[0], di = tot[1];
@@ -1095,15 +1094,15 @@ __device__ __forceinline__ void hop_reduce_body(const HopArgs &a, const EpiReduc
             red[2] = red_cast<RedT>(n);
         }
     }
-    hop_reduce_finish<KIND>(e, st, r, sb, red);
+    hop_reduce_finish<KIND>(a.g, e, st, r, sb, red);
 }
 
 // Resident blocks per SM the reduction-fused hop asks the register
 // allocator for: six (80 registers, no spills) for FP16 storage, where
-// occupancy hides the load latency; the other precisions need more
-// registers than that (FP32 would spill at 80).
+// occupancy hides the load latency, four (128) for FP32; the other
+// precisions need more registers than that.
 template <int P> struct ReduceMinBlocks {
-    static constexpr int value = P == WL_F16 ? 6 : 1;
+    static constexpr int value = P == WL_F16 ? 6 : P == WL_F32 ? 4 : 1;
 };
 
 template <int P, bool DAG, int KIND>

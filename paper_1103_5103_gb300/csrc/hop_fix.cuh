@@ -447,7 +447,7 @@ __global__ void __launch_bounds__(128, 4) k_hop_fix_reduce(HopArgs a, EpiReduce<
             red[2] = n;
         }
     }
-    hop_reduce_finish<KIND>(e, st, r, sb, red);
+    hop_reduce_finish<KIND>(a.g, e, st, r, sb, red);
 }
 
 template <bool DAG, int KIND>

@@ -121,14 +121,17 @@ int hop(wl_gauge *g, const Vec &in, const Vec &out, const Vec *x, double coef, i
 
 // Fused solver hops: second half of an operator application followed by the
 // BiCGstab reductions; this launch is part `part` of `parts` launches of one
-// reduction (full-lattice vectors: one launch per parity).  partials holds
-// parts * 2 * site_blocks * kRedNV doubles per rhs.
+// reduction (full-lattice vectors: one launch per parity); partials from
+// red_buffer.
 //   kind 0:  v = a1 * xin + coef * D tmp;  <rhat, v>        -> alpha = rho / <rhat, v>
 //   kind 1:  t = a1 * xin + coef * D tmp;  <t, xin>, <t, t> -> omega
 // coef_dev (optional, device) overrides coef at run time.
 int hop_reduce(wl_gauge *g, int kind, const Vec &tmp, const Vec &xin, double a1, const Vec &out, const Vec &rhat,
                double coef, const double *coef_dev, int out_parity, int dagger, BiState *state, double *partials,
                int part, int parts, cudaStream_t s);
+
+// Workspace of site_sum for nrhs right-hand sides (group tickets at zero).
+int red_buffer(wl_gauge *g, const std::string &name, int nrhs, void **out, cudaStream_t s);
 
 // ---- blas.cu (all on one parity; nrhs from the vectors)
 int blas_s_update(const Geom &g, const Vec &r, const Vec &v, const Vec &s_out, BiState *st, cudaStream_t s);

@@ -29,7 +29,7 @@ namespace wl {
 // Scratch of one batched solve: per-rhs state, reduction partials, flags.
 struct Scratch {
     BiState *state = nullptr;    // [nrhs]
-    double *partials = nullptr;  // [nrhs][2 * site_blocks][kRedNV]
+    double *partials = nullptr;  // site_sum's buffer, nrhs of them
     double *norms = nullptr;     // [nrhs * 4]
     unsigned *tickets = nullptr; // [nrhs * 4]
     int *active = nullptr;       // [nrhs]
@@ -39,13 +39,21 @@ struct Scratch {
     int *outer_done = nullptr;   // [nrhs] 1 once the outer residual of rhs r has converged
 };
 
+int red_buffer(wl_gauge *g, const std::string &name, int nrhs, void **out, cudaStream_t s)
+{
+    const size_t bytes = sizeof(double) * nrhs * red_doubles(g->lat->geom);
+    const bool fresh = g->ws.bufs[name].bytes < bytes;
+    WL_TRY(g->ws.get(name, bytes, out));
+    if (fresh) WL_CUDA_TRY(cudaMemsetAsync(*out, 0, bytes, s));
+    return WL_OK;
+}
+
 static int get_scratch(wl_gauge *g, int nrhs, Scratch *sc, cudaStream_t s)
 {
-    const Geom &geo = g->lat->geom;
     void *p;
     WL_TRY(g->ws.get("state", sizeof(BiState) * nrhs, &p));
     sc->state = static_cast<BiState *>(p);
-    WL_TRY(g->ws.get("partials", sizeof(double) * nrhs * 2 * site_blocks(geo) * kRedNV, &p));
+    WL_TRY(red_buffer(g, "partials", nrhs, &p, s));
     sc->partials = static_cast<double *>(p);
     WL_TRY(g->ws.get("norms", sizeof(double) * nrhs * 4, &p));
     sc->norms = static_cast<double *>(p);
