@@ -382,8 +382,9 @@ int wl_profile_enable(wl_gauge *g, int on);
  * site_rhs counting only the rhs that the launch processed. */
 int wl_profile_read(wl_gauge *g, wl_kernel_profile out[4]);
 
-/* Autotune the hop for (prec, n_rhs) on this gauge handle: every variant
- * (right-hand sides per thread, minimum resident blocks per SM) is timed
+/* Autotune the hop for (prec, n_rhs) on this gauge handle: the variants
+ * (right-hand sides per thread, minimum resident blocks per SM, load order)
+ * that are the fastest for some lattice and n_rhs are timed
  * with CUDA events on the stream and the fastest is cached in the handle;
  * solvers and wilson_hop_multi with rhs_block = 0 use it.  With the
  * environment variable WL_AUTOTUNE_CACHE naming a file, results are read

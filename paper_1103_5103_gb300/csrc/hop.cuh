@@ -1026,6 +1026,10 @@ __device__ __forceinline__ void hop_reduce_finish(const Geom &g, const EpiReduce
     }
 }
 
+// hop_batch.cuh
+template <int P, bool DAG>
+__device__ __forceinline__ void hop_accumulate_batch(const HopArgs &a, const void *in, int i, cx<float> (&acc)[12]);
+
 template <int P, bool DAG, int KIND>
 __device__ __forceinline__ void hop_reduce_body(const HopArgs &a, const EpiReduce<KIND> &e)
 {
@@ -1052,6 +1056,8 @@ __device__ __forceinline__ void hop_reduce_body(const HopArgs &a, const EpiReduc
             HopArgs b = a;
             b.in = static_cast<const char *>(a.in) + (size_t)r * a.rhs_bytes;
             hop_accumulate_rolled<P, DAG>(b, i, acc[0]);
+        } else if constexpr (P == WL_F16 || P == WL_F32) {
+            hop_accumulate_batch<P, DAG>(a, static_cast<const char *>(a.in) + (size_t)r * a.rhs_bytes, i, acc[0]);
         } else {
             hop_accumulate<P, DAG, 1>(a, i, r, acc);
         }
@@ -1097,12 +1103,14 @@ __device__ __forceinline__ void hop_reduce_body(const HopArgs &a, const EpiReduc
     hop_reduce_finish<KIND>(a.g, e, st, r, sb, red);
 }
 
-// Resident blocks per SM the reduction-fused hop asks the register
-// allocator for: six (80 registers, no spills) for FP16 storage, where
-// occupancy hides the load latency, four (128) for FP32; the other
-// precisions need more registers than that.
+// The reduction-fused hops of FP32 and FP16 data issue their loads a
+// transporter ahead (hop_batch.cuh) at 96 registers, five blocks per SM: on
+// 24^3x64, 12 rhs, FP32 the two kinds average 317 and 296 us over a solve
+// (370 and 359 with the compiler's 167 registers and three blocks; 329 and
+// 313 at four), FP16 3 rhs 32^3x64 167 and 155 us (173 and 163 with loads at
+// their uses and six blocks).
 template <int P> struct ReduceMinBlocks {
-    static constexpr int value = P == WL_F16 ? 6 : P == WL_F32 ? 4 : 1;
+    static constexpr int value = P == WL_F16 || P == WL_F32 ? 5 : 1;
 };
 
 template <int P, bool DAG, int KIND>

@@ -2,9 +2,10 @@
 // library builds in parallel).  Variant v = 100 * (rhs per thread) + (minimum resident
 // blocks per SM requested from the register allocator); 5006 is the paired-site hop
 // (two sites per thread in packed FP32 arithmetic, 64-thread blocks, six resident per
-// SM: 168 registers; a tighter budget spills); 9000 + 100 b + R is the TMA-staged hop with R rhs per tile and
+// SM: 168 registers; a tighter budget spills); 8100 + B issues its loads a transporter ahead, B
+// blocks per SM (hop_batch.cuh); 9000 + 100 b + R is the TMA-staged hop with R rhs per tile and
 // register budget b (hop_tma.cu).
-#include "hop.cuh"
+#include "hop_batch.cuh"
 
 namespace wl {
 
@@ -26,6 +27,7 @@ int hop_launch_prec<WL_F32>(int v, int dagger, const HopArgs &a, const EpiStore 
         }
     } else {
         switch (v) {
+        case 8104: launch_k_hop_batch<WL_F32, false, 4>(a, e, s); break;
         case 1104: launch_k_hop_async<false, 1, 4>(a, e, s); break;
         case 1106: launch_k_hop_async<false, 1, 6>(a, e, s); break;
         case 1202: launch_k_hop_async<false, 2, 2>(a, e, s); break;

@@ -20,8 +20,8 @@ namespace wl {
 const std::vector<int> &hop_variants(int prec)
 {
     static const std::vector<int> f32 = {101, 105, 106, 108, 201, 204, 205, 401, 404, 301, 304, 305, 1104, 1106, 1202, 1203,
-                                         5006, 9001, 9002, 9004, 9102, 9104};
-    static const std::vector<int> f16 = {101, 105, 106, 108, 110, 201, 204, 206, 401, 404, 5006,
+                                         5006, 8104, 9001, 9002, 9004, 9102, 9104};
+    static const std::vector<int> f16 = {101, 105, 106, 108, 110, 201, 204, 206, 401, 404, 5006, 8105,
                                          9001, 9002, 9004, 9102, 9104};
     static const std::vector<int> f64 = {101, 103, 201, 6000, 6001, 6002, 7101, 7102, 7201, 7202};
     static const std::vector<int> dfv = {101, 103, 104, 105, 106};
@@ -47,6 +47,23 @@ int hop_variant_for(wl_gauge *g, int prec, int nrhs, int rhs_block)
     return it == g->tune.end() ? 101 : it->second.variant;
 }
 
+// The variants that tuning times: those that were the fastest of
+// hop_variants() on some lattice and rhs count.  The others (cp.async and TMA
+// staging, paired sites, prefetch, four rhs per thread) never were, some won
+// a noisy timing and then lost in the solve (TMA-staged 304 us per hop where
+// 205 takes 247, 12 rhs on 24^3x64), and each costs seven launches per handle.
+static const std::vector<int> &tune_candidates(const wl_gauge *g, int prec)
+{
+    static const std::vector<int> f32 = {8104, 105, 106, 205}, f16 = {105, 106, 8105}, fix = {6000},
+                                  dfv = {101, 103, 104};
+    switch (prec) {
+    case WL_F32: return f32;
+    case WL_F16: return f16;
+    case WL_DF: return dfv;
+    default: return g->fix_links[0] ? fix : hop_variants(prec);   // (hop_variant_for)
+    }
+}
+
 static std::string tune_key(const wl_gauge *g, int prec, int nrhs)
 {
     cudaDeviceProp prop;
@@ -68,8 +85,7 @@ int autotune_hop(wl_gauge *g, int prec, int nrhs, cudaStream_t s, TuneResult *ou
         if (out) *out = it->second;
         return WL_OK;
     }
-    static const std::vector<int> fix = {6000};   // the only FP64 candidate (hop_variant_for)
-    const std::vector<int> &vs = prec == WL_F64 && g->fix_links[0] ? fix : hop_variants(prec);
+    const std::vector<int> &vs = tune_candidates(g, prec);
     if (vs.empty()) { set_error("autotune: bad precision"); return WL_ERR_ARG; }
     TuneResult best;
     const char *path = std::getenv("WL_AUTOTUNE_CACHE");
