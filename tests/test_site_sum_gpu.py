@@ -44,9 +44,10 @@ def test_sums_at_the_edge_of_two_levels(dims, prec, tol):
         for r in range(nrhs):
             want = float((av[r].abs() ** 2).sum())
             assert abs(got[r] - want) <= tol * want
-    # x += 0, r = s - 0: <rhat, s> and ||s||^2
-    (x, _), (p, _), (s, sv), (t, _), (r_, _), (rh, hv) = (batch() for _ in range(6))
-    dots = api.vector_op(g, api.VEC_XR, prec, nrhs, stride, [x, p, s, t, r_, rh], [(0, 0, 0)] * nrhs)
+    # omega = 1 and t = 0, so r = s: <rhat, s> and ||s||^2
+    (x, _), (p, _), (s, sv), (r_, _), (rh, hv) = (batch() for _ in range(5))
+    t = torch.zeros_like(s)
+    dots = api.vector_op(g, api.VEC_XR, prec, nrhs, stride, [x, p, s, t, r_, rh], [(0, 1, 0)] * nrhs)
     for r in range(nrhs):
         d = complex(torch.vdot(hv[r].reshape(-1), sv[r].reshape(-1)))
         n = float((sv[r].abs() ** 2).sum())
