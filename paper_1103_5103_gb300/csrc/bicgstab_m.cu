@@ -70,7 +70,7 @@ __device__ __forceinline__ cx<double> cdiv(cx<double> a, cx<double> b)
 // After alpha_n and omega_n: pi_{n+1}, alpha^s, omega^s and the x/q coefficients.
 __global__ void k_shift_a(ShiftState *sh, int ns, const BiState *bs, const MState *ms)
 {
-    const int k = threadIdx.x;
+    const int k = threadIdx.x + chain_begin();
     if (k >= ns || bs->done || !sh[k].active) return;
     ShiftState &S = sh[k];
     const cx<double> al = dc(bs->alpha_re, bs->alpha_im), om = dc(bs->omega_re, bs->omega_im);
@@ -98,7 +98,7 @@ __global__ void k_shift_a(ShiftState *sh, int ns, const BiState *bs, const MStat
 // then roll pi and the previous alpha/beta forward.
 __global__ void k_shift_b(ShiftState *sh, int ns, const BiState *bs, MState *ms)
 {
-    const int k = threadIdx.x;
+    const int k = threadIdx.x + chain_begin();
     if (ms->finished) return;     // uniform: no shift updates after the last iteration
     __syncthreads();
     if (bs->breakdown) {
@@ -192,6 +192,7 @@ __global__ void __launch_bounds__(kBlock) k_m_s(Geom g, int nsb, Vec r, Vec v, V
 {
     using C = CompIO<P>;
     using R = typename PrecTraits<P>::R;
+    st += chain_begin();
     const FullIdx f = full_idx(nsb);
     if (__ldcg(&st->done) || f.i >= g.Vh) return;
     const cx<R> al = cs<R>(__ldcg(&st->alpha_re), __ldcg(&st->alpha_im));
@@ -212,6 +213,7 @@ __global__ void __launch_bounds__(kBlock) k_m_update(Geom g, int nsb, Vec x, Vec
     using C = CompIO<P>;
     using R = typename PrecTraits<P>::R;
     static_assert(sizeof(cx<R>) == 16, "coefficient staging assumes 16-byte complex scalars");
+    st += chain_begin();
     const FullIdx f = full_idx(nsb);
     BiState &S = *st;
     if (__ldcg(&S.done)) return;
@@ -305,6 +307,7 @@ __global__ void __launch_bounds__(kBlock) k_m_p(Geom g, int nsb, Vec r, Vec p, V
 {
     using C = CompIO<P>;
     using R = typename PrecTraits<P>::R;
+    st += chain_begin();
     const FullIdx f = full_idx(nsb);
     if (f.i >= g.Vh || __ldcg(&st->done)) return;
     const int h = f.half, i = f.i, str = g.stride;
@@ -322,6 +325,7 @@ __global__ void k_m_dots(const double2 *a, const double2 *b, size_t n, double *p
                          double *out)
 {
     double v[3] = {0.0, 0.0, 0.0};
+    chain_begin();
     for (size_t k = (size_t)blockIdx.x * blockDim.x + threadIdx.x; k < n; k += (size_t)gridDim.x * blockDim.x) {
         const double2 x = a[k], y = b[k];
         v[0] += x.x * y.x + x.y * y.y;
@@ -337,6 +341,7 @@ __global__ void k_m_dots(const double2 *a, const double2 *b, size_t n, double *p
 // residual (dots = {Re <rhat, b>, Im <rhat, b>, ||rhat||^2}).
 __global__ void k_m_init(BiState *st, double bn2, const double *dots, double target2, double brk2)
 {
+    chain_begin();
     st->rho_re = dots ? dots[0] : bn2;
     st->rho_im = dots ? dots[1] : 0.0;
     st->rhat2 = dots ? dots[2] : bn2;
@@ -453,7 +458,7 @@ extern "C" int bicgstab_m_solve(wl_gauge *g, const void *b, void *const *x, cons
         void *pd;
         WL_TRY(g->ws.get("bm_dots_partials", sizeof(double) * 3 * 1024, &pd));
         d_dots = d_norm + 4;
-        k_m_dots<<<1024, 256, 0, s>>>(static_cast<const double2 *>(p->shadow), static_cast<const double2 *>(b),
+        launch_chained(k_m_dots, 1024, 256, s, static_cast<const double2 *>(p->shadow), static_cast<const double2 *>(b),
                                       (size_t)geo.Vh * 2 * 12, static_cast<double *>(pd), d_ticket + 2, d_dots);
         WL_CUDA_TRY(cudaGetLastError());
         note_launch(s);
@@ -490,7 +495,7 @@ extern "C" int bicgstab_m_solve(wl_gauge *g, const void *b, void *const *x, cons
     WL_CUDA_TRY(cudaMemcpyAsync(mst, &hm, sizeof(MState), cudaMemcpyHostToDevice, s));
     if (ns) WL_CUDA_TRY(cudaMemcpyAsync(sh, hsh.data(), sizeof(ShiftState) * ns, cudaMemcpyHostToDevice, s));
     // iterate the unshifted system to half the tolerance (iterated/true gap)
-    k_m_init<<<1, 1, 0, s>>>(st, bn2, d_dots, 0.25 * hm.target2, kBreakdown2);
+    launch_chained(k_m_init, 1, 1, s, st, bn2, d_dots, 0.25 * hm.target2, kBreakdown2);
     note_launch(s);
     WL_CUDA_TRY(cudaStreamSynchronize(s));
 
@@ -502,23 +507,23 @@ extern "C" int bicgstab_m_solve(wl_gauge *g, const void *b, void *const *x, cons
         // v = A p, <rhat, v> -> alpha
         WL_TRY(hop_reduce(g, 0, po, pe, a1, ve, rhe, -0.5, nullptr, WL_EVEN, 0, st, partials, 0, 2, q));
         WL_TRY(hop_reduce(g, 0, pe, po, a1, vo, rho, -0.5, nullptr, WL_ODD, 0, st, partials, 1, 2, q));
-        if (P == WL_DF) k_m_s<WL_DF><<<2 * nsb, kBlock, 0, q>>>(geo, nsb, r, v, sv, st);
-        else k_m_s<WL_F64><<<2 * nsb, kBlock, 0, q>>>(geo, nsb, r, v, sv, st);
+        if (P == WL_DF) launch_chained(k_m_s<WL_DF>, 2 * nsb, kBlock, q, geo, nsb, r, v, sv, st);
+        else launch_chained(k_m_s<WL_F64>, 2 * nsb, kBlock, q, geo, nsb, r, v, sv, st);
         note_launch(q);
         // t = A s, <t,s>, <t,t> -> omega
         WL_TRY(hop_reduce(g, 1, so, se, a1, te, rhe, -0.5, nullptr, WL_EVEN, 0, st, partials, 0, 2, q));
         WL_TRY(hop_reduce(g, 1, se, so, a1, to, rho, -0.5, nullptr, WL_ODD, 0, st, partials, 1, 2, q));
         if (ns) {
-            k_shift_a<<<1, 32, 0, q>>>(sh, ns, st, mst);
+            launch_chained(k_shift_a, 1, 32, q, sh, ns, st, mst);
             note_launch(q);
         }
         if (P == WL_DF)
-            k_m_update<WL_DF><<<2 * nsb, kBlock, 0, q>>>(geo, nsb, xv, pv, sv, t, r, rhat, shv, sh, ns, st, partials);
+            launch_chained(k_m_update<WL_DF>, 2 * nsb, kBlock, q, geo, nsb, xv, pv, sv, t, r, rhat, shv, sh, ns, st, partials);
         else
-            k_m_update<WL_F64><<<2 * nsb, kBlock, 0, q>>>(geo, nsb, xv, pv, sv, t, r, rhat, shv, sh, ns, st, partials);
-        k_shift_b<<<1, 32, 0, q>>>(sh, ns, st, mst);
-        if (P == WL_DF) k_m_p<WL_DF><<<2 * nsb, kBlock, 0, q>>>(geo, nsb, r, pv, v, st);
-        else k_m_p<WL_F64><<<2 * nsb, kBlock, 0, q>>>(geo, nsb, r, pv, v, st);
+            launch_chained(k_m_update<WL_F64>, 2 * nsb, kBlock, q, geo, nsb, xv, pv, sv, t, r, rhat, shv, sh, ns, st, partials);
+        launch_chained(k_shift_b, 1, 32, q, sh, ns, st, mst);
+        if (P == WL_DF) launch_chained(k_m_p<WL_DF>, 2 * nsb, kBlock, q, geo, nsb, r, pv, v, st);
+        else launch_chained(k_m_p<WL_F64>, 2 * nsb, kBlock, q, geo, nsb, r, pv, v, st);
         note_launch(q);
         note_launch(q);
         note_launch(q);

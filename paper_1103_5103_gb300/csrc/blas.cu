@@ -19,8 +19,9 @@ struct SiteIdx {
 __device__ __forceinline__ SiteIdx site_idx(int nrhs)
 {
     SiteIdx s;
-    s.r = blockIdx.x % nrhs;
-    s.sb = blockIdx.x / nrhs;
+    const int z = chain_begin();
+    s.r = blockIdx.x % nrhs + z;
+    s.sb = blockIdx.x / nrhs + z;
     s.nsb = gridDim.x / nrhs;
     s.i = s.sb * blockDim.x + threadIdx.x;
     return s;
@@ -60,9 +61,9 @@ __global__ void __launch_bounds__(kBlock) k_s_update(Geom g, Vec r, Vec v, Vec s
 int blas_s_update(const Geom &g, const Vec &r, const Vec &v, const Vec &s_out, BiState *state, cudaStream_t s)
 {
     switch (r.prec) {
-    case WL_F64: k_s_update<WL_F64><<<grid_of(g, r.nrhs), kBlock, 0, s>>>(g, r, v, s_out, state); break;
-    case WL_F32: k_s_update<WL_F32><<<grid_of(g, r.nrhs), kBlock, 0, s>>>(g, r, v, s_out, state); break;
-    case WL_F16: k_s_update<WL_F16><<<grid_of(g, r.nrhs), kBlock, 0, s>>>(g, r, v, s_out, state); break;
+    case WL_F64: launch_chained(k_s_update<WL_F64>, grid_of(g, r.nrhs), kBlock, s, g, r, v, s_out, state); break;
+    case WL_F32: launch_chained(k_s_update<WL_F32>, grid_of(g, r.nrhs), kBlock, s, g, r, v, s_out, state); break;
+    case WL_F16: launch_chained(k_s_update<WL_F16>, grid_of(g, r.nrhs), kBlock, s, g, r, v, s_out, state); break;
     }
     WL_CUDA_TRY(cudaGetLastError());
     note_launch(s);
@@ -158,11 +159,11 @@ int blas_xr_update(const Geom &g, const Vec &x, const Vec &p, const Vec &sv, con
 {
     const int gr = grid_of(g, r.nrhs);
     if (r.prec == WL_F64 && x.prec == WL_F64)
-        k_xr_update<WL_F64, WL_F64><<<gr, kBlock, 0, s>>>(g, x, p, sv, t, r, rhat, state, partials);
+        launch_chained(k_xr_update<WL_F64, WL_F64>, gr, kBlock, s, g, x, p, sv, t, r, rhat, state, partials);
     else if (r.prec == WL_F32 && x.prec == WL_F32)
-        k_xr_update<WL_F32, WL_F32><<<gr, kBlock, 0, s>>>(g, x, p, sv, t, r, rhat, state, partials);
+        launch_chained(k_xr_update<WL_F32, WL_F32>, gr, kBlock, s, g, x, p, sv, t, r, rhat, state, partials);
     else if (r.prec == WL_F16 && x.prec == WL_F32)
-        k_xr_update<WL_F16, WL_F32><<<gr, kBlock, 0, s>>>(g, x, p, sv, t, r, rhat, state, partials);
+        launch_chained(k_xr_update<WL_F16, WL_F32>, gr, kBlock, s, g, x, p, sv, t, r, rhat, state, partials);
     else {
         set_error("blas_xr_update: unsupported precision pair");
         return WL_ERR_ARG;
@@ -227,11 +228,11 @@ int blas_cg_xr(const Geom &g, const Vec &x, const Vec &p, const Vec &w, const Ve
 {
     const int gr = grid_of(g, r.nrhs);
     if (r.prec == WL_F64 && x.prec == WL_F64)
-        k_cg_xr<WL_F64, WL_F64><<<gr, kBlock, 0, s>>>(g, x, p, w, r, state, partials);
+        launch_chained(k_cg_xr<WL_F64, WL_F64>, gr, kBlock, s, g, x, p, w, r, state, partials);
     else if (r.prec == WL_F32 && x.prec == WL_F32)
-        k_cg_xr<WL_F32, WL_F32><<<gr, kBlock, 0, s>>>(g, x, p, w, r, state, partials);
+        launch_chained(k_cg_xr<WL_F32, WL_F32>, gr, kBlock, s, g, x, p, w, r, state, partials);
     else if (r.prec == WL_F16 && x.prec == WL_F32)
-        k_cg_xr<WL_F16, WL_F32><<<gr, kBlock, 0, s>>>(g, x, p, w, r, state, partials);
+        launch_chained(k_cg_xr<WL_F16, WL_F32>, gr, kBlock, s, g, x, p, w, r, state, partials);
     else {
         set_error("blas_cg_xr: unsupported precision pair");
         return WL_ERR_ARG;
@@ -263,9 +264,9 @@ __global__ void __launch_bounds__(kBlock) k_p_update(Geom g, Vec r, Vec p, Vec v
 int blas_p_update(const Geom &g, const Vec &r, const Vec &p, const Vec &v, BiState *state, cudaStream_t s)
 {
     switch (r.prec) {
-    case WL_F64: k_p_update<WL_F64><<<grid_of(g, r.nrhs), kBlock, 0, s>>>(g, r, p, v, state); break;
-    case WL_F32: k_p_update<WL_F32><<<grid_of(g, r.nrhs), kBlock, 0, s>>>(g, r, p, v, state); break;
-    case WL_F16: k_p_update<WL_F16><<<grid_of(g, r.nrhs), kBlock, 0, s>>>(g, r, p, v, state); break;
+    case WL_F64: launch_chained(k_p_update<WL_F64>, grid_of(g, r.nrhs), kBlock, s, g, r, p, v, state); break;
+    case WL_F32: launch_chained(k_p_update<WL_F32>, grid_of(g, r.nrhs), kBlock, s, g, r, p, v, state); break;
+    case WL_F16: launch_chained(k_p_update<WL_F16>, grid_of(g, r.nrhs), kBlock, s, g, r, p, v, state); break;
     }
     WL_CUDA_TRY(cudaGetLastError());
     note_launch(s);
@@ -377,11 +378,11 @@ static int restart_po(const Geom &g, const Vec &r64, const Vec &r, const Vec &rh
 {
     const int gr = grid_of(g, r.nrhs);
     if (r.prec == WL_F64 && x.prec == WL_F64)
-        k_restart<PO, WL_F64, WL_F64><<<gr, kBlock, 0, s>>>(g, r64, r, rhat, p, x, state, partials, active, delta2);
+        launch_chained(k_restart<PO, WL_F64, WL_F64>, gr, kBlock, s, g, r64, r, rhat, p, x, state, partials, active, delta2);
     else if (r.prec == WL_F32 && x.prec == WL_F32)
-        k_restart<PO, WL_F32, WL_F32><<<gr, kBlock, 0, s>>>(g, r64, r, rhat, p, x, state, partials, active, delta2);
+        launch_chained(k_restart<PO, WL_F32, WL_F32>, gr, kBlock, s, g, r64, r, rhat, p, x, state, partials, active, delta2);
     else if (r.prec == WL_F16 && x.prec == WL_F32)
-        k_restart<PO, WL_F16, WL_F32><<<gr, kBlock, 0, s>>>(g, r64, r, rhat, p, x, state, partials, active, delta2);
+        launch_chained(k_restart<PO, WL_F16, WL_F32>, gr, kBlock, s, g, r64, r, rhat, p, x, state, partials, active, delta2);
     else {
         set_error("blas_restart: unsupported precision pair");
         return WL_ERR_ARG;
@@ -419,11 +420,11 @@ int blas_accum(const Geom &g, const Vec &e, const Vec &x64, const int *active, c
 {
     const int gr = grid_of(g, x64.nrhs);
     if (x64.prec == WL_DF) {
-        if (e.prec == WL_F64) k_accum<WL_DF, WL_F64><<<gr, kBlock, 0, s>>>(g, e, x64, active);
-        else k_accum<WL_DF, WL_F32><<<gr, kBlock, 0, s>>>(g, e, x64, active);
+        if (e.prec == WL_F64) launch_chained(k_accum<WL_DF, WL_F64>, gr, kBlock, s, g, e, x64, active);
+        else launch_chained(k_accum<WL_DF, WL_F32>, gr, kBlock, s, g, e, x64, active);
     } else {
-        if (e.prec == WL_F64) k_accum<WL_F64, WL_F64><<<gr, kBlock, 0, s>>>(g, e, x64, active);
-        else k_accum<WL_F64, WL_F32><<<gr, kBlock, 0, s>>>(g, e, x64, active);
+        if (e.prec == WL_F64) launch_chained(k_accum<WL_F64, WL_F64>, gr, kBlock, s, g, e, x64, active);
+        else launch_chained(k_accum<WL_F64, WL_F32>, gr, kBlock, s, g, e, x64, active);
     }
     WL_CUDA_TRY(cudaGetLastError());
     note_launch(s);
@@ -450,8 +451,8 @@ __global__ void __launch_bounds__(kBlock) k_xpay(Geom g, Vec x, double a, Vec y,
 int blas_xpay(const Geom &g, const Vec &x, double a, const Vec &y, const Vec &out, cudaStream_t s)
 {
     const int gr = grid_of(g, out.nrhs);
-    if (out.prec == WL_DF) k_xpay<WL_DF><<<gr, kBlock, 0, s>>>(g, x, a, y, out);
-    else if (out.prec == WL_F64) k_xpay<WL_F64><<<gr, kBlock, 0, s>>>(g, x, a, y, out);
+    if (out.prec == WL_DF) launch_chained(k_xpay<WL_DF>, gr, kBlock, s, g, x, a, y, out);
+    else if (out.prec == WL_F64) launch_chained(k_xpay<WL_F64>, gr, kBlock, s, g, x, a, y, out);
     else { set_error("blas_xpay: outer precision only"); return WL_ERR_ARG; }
     WL_CUDA_TRY(cudaGetLastError());
     note_launch(s);
@@ -488,10 +489,10 @@ int blas_norm2(const Geom &g, const Vec &a, double *out_dev, double *partials, u
 {
     const int gr = grid_of(g, a.nrhs);
     switch (a.prec) {
-    case WL_F64: k_norm2<WL_F64><<<gr, kBlock, 0, s>>>(g, a, out_dev, partials, tickets); break;
-    case WL_F32: k_norm2<WL_F32><<<gr, kBlock, 0, s>>>(g, a, out_dev, partials, tickets); break;
-    case WL_F16: k_norm2<WL_F16><<<gr, kBlock, 0, s>>>(g, a, out_dev, partials, tickets); break;
-    case WL_DF: k_norm2<WL_DF><<<gr, kBlock, 0, s>>>(g, a, out_dev, partials, tickets); break;
+    case WL_F64: launch_chained(k_norm2<WL_F64>, gr, kBlock, s, g, a, out_dev, partials, tickets); break;
+    case WL_F32: launch_chained(k_norm2<WL_F32>, gr, kBlock, s, g, a, out_dev, partials, tickets); break;
+    case WL_F16: launch_chained(k_norm2<WL_F16>, gr, kBlock, s, g, a, out_dev, partials, tickets); break;
+    case WL_DF: launch_chained(k_norm2<WL_DF>, gr, kBlock, s, g, a, out_dev, partials, tickets); break;
     }
     WL_CUDA_TRY(cudaGetLastError());
     note_launch(s);
@@ -564,13 +565,13 @@ int blas_lincomb2(const Geom &g, const double *c1_dev, const Vec *const *in, int
     const Vec o1 = k > 0 ? *out : o2;
     const int grid = grid_of(g, o.nrhs);
     if (o.prec == WL_DF && complex_coef)
-        k_lincomb<WL_DF, true><<<grid, kBlock, 0, s>>>(g, li, k, k2, o.rhs_bytes, o.nrhs, c1_dev, c2_dev, o1, o2);
+        launch_chained(k_lincomb<WL_DF, true>, grid, kBlock, s, g, li, k, k2, o.rhs_bytes, o.nrhs, c1_dev, c2_dev, o1, o2);
     else if (o.prec == WL_DF)
-        k_lincomb<WL_DF, false><<<grid, kBlock, 0, s>>>(g, li, k, k2, o.rhs_bytes, o.nrhs, c1_dev, c2_dev, o1, o2);
+        launch_chained(k_lincomb<WL_DF, false>, grid, kBlock, s, g, li, k, k2, o.rhs_bytes, o.nrhs, c1_dev, c2_dev, o1, o2);
     else if (o.prec == WL_F64 && complex_coef)
-        k_lincomb<WL_F64, true><<<grid, kBlock, 0, s>>>(g, li, k, k2, o.rhs_bytes, o.nrhs, c1_dev, c2_dev, o1, o2);
+        launch_chained(k_lincomb<WL_F64, true>, grid, kBlock, s, g, li, k, k2, o.rhs_bytes, o.nrhs, c1_dev, c2_dev, o1, o2);
     else if (o.prec == WL_F64)
-        k_lincomb<WL_F64, false><<<grid, kBlock, 0, s>>>(g, li, k, k2, o.rhs_bytes, o.nrhs, c1_dev, c2_dev, o1, o2);
+        launch_chained(k_lincomb<WL_F64, false>, grid, kBlock, s, g, li, k, k2, o.rhs_bytes, o.nrhs, c1_dev, c2_dev, o1, o2);
     else { set_error("blas_lincomb: outer precision only"); return WL_ERR_ARG; }
     WL_CUDA_TRY(cudaGetLastError());
     note_launch(s);
@@ -637,7 +638,7 @@ int blas_guess_residual(const Geom &g, const double *c_dev, const double *d_dev,
     LinIn li;
     for (int j = 0; j < 2 * k + 1; ++j) li.p[j] = in[j]->ptr;
     const int grid = grid_of(g, x.nrhs);
-#define WL_GR(PO, CP) k_guess_residual<PO, CP><<<grid, kBlock, 0, s>>>(g, li, k, x.rhs_bytes, x.nrhs, c_dev, d_dev, x, r)
+#define WL_GR(PO, CP) launch_chained(k_guess_residual<PO, CP>, grid, kBlock, s, g, li, k, x.rhs_bytes, x.nrhs, c_dev, d_dev, x, r)
     if (x.prec == WL_DF && complex_coef) WL_GR(WL_DF, true);
     else if (x.prec == WL_DF) WL_GR(WL_DF, false);
     else if (x.prec == WL_F64 && complex_coef) WL_GR(WL_F64, true);
@@ -669,6 +670,7 @@ __global__ void __launch_bounds__(256) k_canon_dots(const double2 *a, DotIn in, 
                                                     unsigned *ticket, double *out)
 {
     double v[2 * N];
+    chain_begin();
 #pragma unroll
     for (int j = 0; j < 2 * N; ++j) v[j] = 0.0;
     for (size_t k = (size_t)blockIdx.x * blockDim.x + threadIdx.x; k < n; k += (size_t)gridDim.x * blockDim.x) {
@@ -689,7 +691,7 @@ template <int N>
 static void launch_canon_dots(const double2 *a, const DotIn &in, size_t n, double *partials, unsigned *ticket,
                               double *out, cudaStream_t s)
 {
-    k_canon_dots<N><<<1024, 256, 0, s>>>(a, in, n, partials, ticket, out);
+    launch_chained(k_canon_dots<N>, 1024, 256, s, a, in, n, partials, ticket, out);
 }
 
 int canon_dots(const void *const *a, const void *const *in, int n, int nrhs, size_t n_complex, double *dots_dev,
@@ -765,8 +767,8 @@ int blas_recon(const Geom &g, const Vec &bo, const Vec &dx, double kappa, const 
                double *partials, unsigned *tickets, cudaStream_t s)
 {
     const int gr = grid_of(g, xo.nrhs);
-    if (xo.prec == WL_DF) k_recon<WL_DF><<<gr, kBlock, 0, s>>>(g, bo, dx, kappa, xo, norm2_dev, partials, tickets);
-    else if (xo.prec == WL_F64) k_recon<WL_F64><<<gr, kBlock, 0, s>>>(g, bo, dx, kappa, xo, norm2_dev, partials, tickets);
+    if (xo.prec == WL_DF) launch_chained(k_recon<WL_DF>, gr, kBlock, s, g, bo, dx, kappa, xo, norm2_dev, partials, tickets);
+    else if (xo.prec == WL_F64) launch_chained(k_recon<WL_F64>, gr, kBlock, s, g, bo, dx, kappa, xo, norm2_dev, partials, tickets);
     else { set_error("blas_recon: outer precision only"); return WL_ERR_ARG; }
     WL_CUDA_TRY(cudaGetLastError());
     note_launch(s);
@@ -792,7 +794,7 @@ int blas_convert(const Geom &g, const Vec &in, const Vec &out, cudaStream_t s)
 {
     const int gr = grid_of(g, out.nrhs);
 #define WL_CONV(A, B) \
-    if (in.prec == A && out.prec == B) { k_convert<A, B><<<gr, kBlock, 0, s>>>(g, in, out); WL_CUDA_TRY(cudaGetLastError()); note_launch(s); return WL_OK; }
+    if (in.prec == A && out.prec == B) { launch_chained(k_convert<A, B>, gr, kBlock, s, g, in, out); WL_CUDA_TRY(cudaGetLastError()); note_launch(s); return WL_OK; }
     WL_CONV(WL_F64, WL_F64) WL_CONV(WL_F64, WL_F32) WL_CONV(WL_F64, WL_F16)
     WL_CONV(WL_F32, WL_F64) WL_CONV(WL_F32, WL_F32) WL_CONV(WL_F32, WL_F16)
     WL_CONV(WL_F16, WL_F64) WL_CONV(WL_F16, WL_F32) WL_CONV(WL_F16, WL_F16)

@@ -481,8 +481,9 @@ __device__ __forceinline__ void hop_accumulate_prefetch_f32(const HopArgs &a, in
 template <bool DAG, int MINB>
 __global__ void __launch_bounds__(128, MINB) k_hop_prefetch_f32(HopArgs a, EpiStore epi)
 {
-    const int r = blockIdx.x % a.ngroups;
-    const int sb = blockIdx.x / a.ngroups;
+    const int z = chain_begin();
+    const int r = blockIdx.x % a.ngroups + z;
+    const int sb = blockIdx.x / a.ngroups + z;
     if (rhs_done(a, r)) return;
     const int i = sb * blockDim.x + threadIdx.x;
     if (i >= a.g.Vh) return;
@@ -500,7 +501,7 @@ void launch_k_hop_prefetch_f32(HopArgs a, const EpiStore &e, cudaStream_t s)
 {
     a.ngroups = a.nrhs;
     const int nsb = (a.g.Vh + 127) / 128;
-    k_hop_prefetch_f32<DAG, MINB><<<nsb * a.nrhs, 128, 0, s>>>(a, e);
+    launch_chained(k_hop_prefetch_f32<DAG, MINB>, nsb * a.nrhs, 128, s, a, e);
 }
 
 // ------------------------------------------ asynchronous-copy FP32 variant
@@ -675,8 +676,9 @@ template <int P, bool DAG, int MINB>
 __global__ void __launch_bounds__(128, MINB) k_hop_rolled(HopArgs a, EpiStore epi)
 {
     using R = typename PrecTraits<P>::R;
-    const int r = blockIdx.x % a.ngroups;
-    const int sb = blockIdx.x / a.ngroups;
+    const int z = chain_begin();
+    const int r = blockIdx.x % a.ngroups + z;
+    const int sb = blockIdx.x / a.ngroups + z;
     if (rhs_done(a, r)) return;
     const int i = sb * blockDim.x + threadIdx.x;
     if (i >= a.g.Vh) return;
@@ -693,8 +695,9 @@ template <int P, bool DAG, int NB, int MINB>
 __global__ void __launch_bounds__(128, MINB) k_hop(HopArgs a, EpiStore epi)
 {
     using R = typename PrecTraits<P>::R;
-    const int grp = blockIdx.x % a.ngroups;
-    const int sb = blockIdx.x / a.ngroups;
+    const int z = chain_begin();
+    const int grp = blockIdx.x % a.ngroups + z;
+    const int sb = blockIdx.x / a.ngroups + z;
     const int r0 = grp * NB;
     if (a.skip) {
         bool all_done = true;
@@ -725,7 +728,7 @@ __global__ void __launch_bounds__(128, MINB) k_hop_gs(HopArgs a, EpiStore epi)
     using R = typename PrecTraits<P>::R;
     const int nsb = (a.g.Vh + 127) / 128;
     const int ntiles = nsb * a.ngroups;
-    for (int t = blockIdx.x; t < ntiles; t += gridDim.x) {
+    for (int t = blockIdx.x + chain_begin(); t < ntiles; t += gridDim.x) {
         const int grp = t % a.ngroups;
         const int sb = t / a.ngroups;
         const int r0 = grp * NB;
@@ -936,8 +939,9 @@ constexpr int kPairThreads = 64;   // threads per block; 2 x 64 = 128 sites per 
 template <int P, bool DAG, int MINB>
 __global__ void __launch_bounds__(kPairThreads, MINB) k_hop_pair(HopArgs a, EpiStore epi)
 {
-    const int r = blockIdx.x % a.ngroups;
-    const int sb = blockIdx.x / a.ngroups;
+    const int z = chain_begin();
+    const int r = blockIdx.x % a.ngroups + z;
+    const int sb = blockIdx.x / a.ngroups + z;
     if (rhs_done(a, r)) return;
     const int ia = sb * (2 * kPairThreads) + threadIdx.x;
     if (ia >= a.g.Vh) return;
@@ -957,7 +961,7 @@ void launch_k_hop_pair(HopArgs a, const EpiStore &e, cudaStream_t s)
 {
     a.ngroups = a.nrhs;
     const int nsb = (a.g.Vh + 2 * kPairThreads - 1) / (2 * kPairThreads);
-    k_hop_pair<P, DAG, MINB><<<nsb * a.nrhs, kPairThreads, 0, s>>>(a, e);
+    launch_chained(k_hop_pair<P, DAG, MINB>, nsb * a.nrhs, kPairThreads, s, a, e);
 }
 
 int sm_count();
@@ -966,7 +970,7 @@ template <int P, bool DAG, int NB, int MINB>
 void launch_k_hop_gs(HopArgs a, const EpiStore &e, cudaStream_t s)
 {
     a.ngroups = (a.nrhs + NB - 1) / NB;
-    k_hop_gs<P, DAG, NB, MINB><<<MINB * sm_count(), 128, 0, s>>>(a, e);
+    launch_chained(k_hop_gs<P, DAG, NB, MINB>, MINB * sm_count(), 128, s, a, e);
 }
 
 // Last step of the reduction-fused hops: the block's partial sums red, and by
@@ -1035,8 +1039,9 @@ __device__ __forceinline__ void hop_reduce_body(const HopArgs &a, const EpiReduc
 {
     using R = typename PrecTraits<P>::R;
     constexpr int NV = EpiReduce<KIND>::NV;
-    const int r = blockIdx.x % a.nrhs;
-    const int sb = blockIdx.x / a.nrhs;
+    const int z = chain_begin();
+    const int r = blockIdx.x % a.nrhs + z;
+    const int sb = blockIdx.x / a.nrhs + z;
     BiState &st = e.st[r];
     if (__ldcg(&st.done)) return;   // uniform over every block of this rhs
     const int i = sb * blockDim.x + threadIdx.x;
@@ -1127,7 +1132,7 @@ void launch_k_hop(HopArgs a, const EpiStore &e, cudaStream_t s)
 {
     a.ngroups = (a.nrhs + NB - 1) / NB;
     const int nsb = (a.g.Vh + 127) / 128;
-    k_hop<P, DAG, NB, MINB><<<nsb * a.ngroups, 128, 0, s>>>(a, e);
+    launch_chained(k_hop<P, DAG, NB, MINB>, nsb * a.ngroups, 128, s, a, e);
 }
 
 template <int P, bool DAG, int MINB>
@@ -1135,14 +1140,14 @@ void launch_k_hop_rolled(HopArgs a, const EpiStore &e, cudaStream_t s)
 {
     a.ngroups = a.nrhs;
     const int nsb = (a.g.Vh + 127) / 128;
-    k_hop_rolled<P, DAG, MINB><<<nsb * a.nrhs, 128, 0, s>>>(a, e);
+    launch_chained(k_hop_rolled<P, DAG, MINB>, nsb * a.nrhs, 128, s, a, e);
 }
 
 template <int P, bool DAG, int KIND>
 void launch_k_hop_reduce(const HopArgs &a, const EpiReduce<KIND> &e, cudaStream_t s)
 {
     const int nsb = (a.g.Vh + 127) / 128;
-    k_hop_reduce<P, DAG, KIND><<<nsb * a.nrhs, 128, 0, s>>>(a, e);
+    launch_chained(k_hop_reduce<P, DAG, KIND>, nsb * a.nrhs, 128, s, a, e);
 }
 
 template <int P, int KIND>

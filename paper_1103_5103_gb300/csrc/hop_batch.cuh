@@ -166,8 +166,9 @@ __device__ __forceinline__ void hop_accumulate_batch(const HopArgs &a, const voi
 template <int P, bool DAG, int MINB>
 __global__ void __launch_bounds__(128, MINB) k_hop_batch(HopArgs a, EpiStore epi)
 {
-    const int r = blockIdx.x % a.nrhs;
-    const int i = (blockIdx.x / a.nrhs) * 128 + threadIdx.x;
+    const int z = chain_begin();
+    const int r = blockIdx.x % a.nrhs + z;
+    const int i = (blockIdx.x / a.nrhs) * 128 + threadIdx.x + z;
     if (i >= a.g.Vh || rhs_done(a, r)) return;
     cx<float> acc[1][12];
 #pragma unroll
@@ -179,7 +180,7 @@ __global__ void __launch_bounds__(128, MINB) k_hop_batch(HopArgs a, EpiStore epi
 template <int P, bool DAG, int MINB>
 void launch_k_hop_batch(const HopArgs &a, const EpiStore &e, cudaStream_t s)
 {
-    k_hop_batch<P, DAG, MINB><<<(a.g.Vh + 127) / 128 * a.nrhs, 128, 0, s>>>(a, e);
+    launch_chained(k_hop_batch<P, DAG, MINB>, (a.g.Vh + 127) / 128 * a.nrhs, 128, s, a, e);
 }
 
 }  // namespace wl

@@ -383,7 +383,7 @@ inline __host__ __device__ unsigned fix_tasks(const HopArgs &a)
 template <bool DAG>
 __global__ void __launch_bounds__(128, 4) k_hop_fix(HopArgs a, EpiStore e)
 {
-    hop_fix_task<DAG>(a, e, blockIdx.x * 4 + (threadIdx.x >> 5), threadIdx.x & 31);
+    hop_fix_task<DAG>(a, e, blockIdx.x * 4 + (threadIdx.x >> 5) + chain_begin(), threadIdx.x & 31);
 }
 
 // The same with a fixed number of blocks that loop over the tasks: leaves
@@ -392,7 +392,7 @@ template <bool DAG>
 __global__ void __launch_bounds__(128, 4) k_hop_fix_gs(HopArgs a, EpiStore e)
 {
     const unsigned n = fix_tasks(a);
-    for (unsigned t = blockIdx.x * 4 + (threadIdx.x >> 5); t < n; t += gridDim.x * 4) {
+    for (unsigned t = blockIdx.x * 4 + (threadIdx.x >> 5) + chain_begin(); t < n; t += gridDim.x * 4) {
         hop_fix_task<DAG>(a, e, t, threadIdx.x & 31);
         __syncwarp();   // lanes past the last site rejoin
     }
@@ -402,15 +402,16 @@ __global__ void __launch_bounds__(128, 4) k_hop_fix_gs(HopArgs a, EpiStore e)
 template <bool DAG>
 void launch_k_hop_fix(const HopArgs &a, const EpiStore &e, int blocks_per_sm, cudaStream_t s)
 {
-    if (blocks_per_sm > 0) k_hop_fix_gs<DAG><<<blocks_per_sm * sm_count(), 128, 0, s>>>(a, e);
-    else k_hop_fix<DAG><<<(fix_tasks(a) + 3) / 4, 128, 0, s>>>(a, e);
+    if (blocks_per_sm > 0) launch_chained(k_hop_fix_gs<DAG>, blocks_per_sm * sm_count(), 128, s, a, e);
+    else launch_chained(k_hop_fix<DAG>, (fix_tasks(a) + 3) / 4, 128, s, a, e);
 }
 
 // The reduction-fused hop (EpiReduce): blocks of 64 sites of one rhs.
 template <bool DAG, int KIND>
 __global__ void __launch_bounds__(128, 4) k_hop_fix_reduce(HopArgs a, EpiReduce<KIND> e)
 {
-    const int r = blockIdx.x % a.nrhs, sb = blockIdx.x / a.nrhs;
+    const int z = chain_begin();
+    const int r = blockIdx.x % a.nrhs + z, sb = blockIdx.x / a.nrhs + z;
     BiState &st = e.st[r];
     if (__ldcg(&st.done)) return;   // uniform over every block of this rhs
     const int lane = threadIdx.x & 31, s = lane >> 4;
@@ -453,7 +454,7 @@ __global__ void __launch_bounds__(128, 4) k_hop_fix_reduce(HopArgs a, EpiReduce<
 template <bool DAG, int KIND>
 void launch_k_hop_fix_reduce(const HopArgs &a, const EpiReduce<KIND> &e, cudaStream_t s)
 {
-    k_hop_fix_reduce<DAG, KIND><<<(a.g.Vh + 63) / 64 * a.nrhs, 128, 0, s>>>(a, e);
+    launch_chained(k_hop_fix_reduce<DAG, KIND>, (a.g.Vh + 63) / 64 * a.nrhs, 128, s, a, e);
 }
 
 }  // namespace wl

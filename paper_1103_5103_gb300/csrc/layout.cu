@@ -121,7 +121,7 @@ int make_vec(wl_gauge *g, const std::string &name, int prec, int nrhs, Vec *v)
 template <int P>
 __global__ void k_import(Geom g, const double2 *__restrict__ canon, void *out, int parity)
 {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    const int i = blockIdx.x * blockDim.x + threadIdx.x + chain_begin();
     if (i >= g.Vh) return;
     const Coord c = site_coord(g, i, parity);
     const size_t lex = c.x + (size_t)g.X * (c.y + (size_t)g.Y * (c.z + (size_t)g.Z * c.t));
@@ -151,7 +151,7 @@ __global__ void __launch_bounds__(kLayoutSites) k_export(Geom g, const void *in,
 {
     __shared__ double2 sm[12 * (kLayoutSites + 1)];
     __shared__ unsigned off[kLayoutSites];
-    const int i0 = blockIdx.x * kLayoutSites, n = min(kLayoutSites, g.Vh - i0);
+    const int i0 = blockIdx.x * kLayoutSites + chain_begin(), n = min(kLayoutSites, g.Vh - i0);
     if ((int)threadIdx.x < n) {
         // canonical offset in complex numbers (12 V < 2^31)
         off[threadIdx.x] = 12u * (2u * (unsigned)(i0 + threadIdx.x) + (unsigned)(site_coord(g, i0 + threadIdx.x, parity).x & 1));
@@ -197,7 +197,7 @@ __global__ void __launch_bounds__(kFullSites) k_export_full(Geom g, const void *
     const size_t ntiles = (V + kFullSites - 1) / kFullSites;
     // tiles strided by the grid: a reduced grid (the overlapped export of
     // the multi-mass solver) occupies a few SMs while other work runs
-    for (size_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+    for (size_t tile = blockIdx.x + chain_begin(); tile < ntiles; tile += gridDim.x) {
         const size_t n0 = tile * kFullSites;
         const size_t n = n0 + threadIdx.x;
         if (n < V) {
@@ -225,7 +225,7 @@ __global__ void __launch_bounds__(kFullSites) k_import_full(Geom g, const double
 {
     __shared__ double2 sm[12 * (kFullSites + 1)];
     const size_t V = (size_t)g.Vh * 2;
-    const size_t n0 = (size_t)blockIdx.x * kFullSites;
+    const size_t n0 = (size_t)(blockIdx.x + chain_begin()) * kFullSites;
     const size_t e0 = n0 * 12, e_end = V * 12;
 #pragma unroll
     for (int j = 0; j < 12; ++j) {
@@ -322,7 +322,7 @@ template <int P>
 static int launch_import(const Geom &g, const void *canon, void *out, int parity, cudaStream_t s)
 {
     const int th = 128, bl = (g.Vh + th - 1) / th;
-    k_import<P><<<bl, th, 0, s>>>(g, static_cast<const double2 *>(canon), out, parity);
+    launch_chained(k_import<P>, bl, th, s, g, static_cast<const double2 *>(canon), out, parity);
     WL_CUDA_TRY(cudaGetLastError());
     note_launch(s);
     return WL_OK;
@@ -332,7 +332,7 @@ template <int P>
 static int launch_export(const Geom &g, const void *in, void *canon, int parity, cudaStream_t s)
 {
     const int th = kLayoutSites, bl = (g.Vh + th - 1) / th;
-    k_export<P><<<bl, th, 0, s>>>(g, in, static_cast<double2 *>(canon), parity);
+    launch_chained(k_export<P>, bl, th, s, g, in, static_cast<double2 *>(canon), parity);
     WL_CUDA_TRY(cudaGetLastError());
     note_launch(s);
     return WL_OK;
@@ -345,9 +345,9 @@ static int launch_full(const Geom &g, const void *canon_in, void *canon_out, con
     unsigned bl = (unsigned)(((size_t)g.Vh * 2 + kFullSites - 1) / kFullSites);
     if (max_blocks > 0 && canon_out && bl > (unsigned)max_blocks) bl = (unsigned)max_blocks;
     if (canon_out)
-        k_export_full<P><<<bl, kFullSites, 0, s>>>(g, even_in, odd_in, static_cast<double2 *>(canon_out));
+        launch_chained(k_export_full<P>, bl, kFullSites, s, g, even_in, odd_in, static_cast<double2 *>(canon_out));
     else
-        k_import_full<P><<<bl, kFullSites, 0, s>>>(g, static_cast<const double2 *>(canon_in), even_out, odd_out);
+        launch_chained(k_import_full<P>, bl, kFullSites, s, g, static_cast<const double2 *>(canon_in), even_out, odd_out);
     WL_CUDA_TRY(cudaGetLastError());
     note_launch(s);
     return WL_OK;
