@@ -256,6 +256,14 @@ __device__ __forceinline__ void hop_accumulate(const HopArgs &a, int i, int r0,
     hop_dir<P, DAG, NB, 3, CG>(a, i, c, rowbase, r0, acc);
 }
 
+// Canonical (lexicographic) site of the neighbour with even-odd index j in
+// direction mu of the site at c, of parity p: 2 j plus the parity bit of the
+// neighbour's row (the x neighbours share the site's row, the others do not).
+__device__ __forceinline__ size_t canon_site(const Coord &c, int p, int mu, int j)
+{
+    return 2 * (size_t)j + ((p + c.y + c.z + c.t + (mu == 0 ? 1 : 0)) & 1);
+}
+
 // ------------------------------------------------------- rolled variant
 // The same stencil with the eight transporters in a loop that is not
 // unrolled: projector, link orientation and neighbour are selected per trip
@@ -274,7 +282,8 @@ __device__ __forceinline__ cx<R> uphase_rt(int c, cx<R> z)
     return {re, im};
 }
 
-template <int P, bool DAG>
+// CANON (FP64 only): a.in is a canonical full-lattice field.
+template <int P, bool DAG, bool CANON = false>
 __device__ __forceinline__ void hop_accumulate_rolled(const HopArgs &a, int i, cx<typename PrecTraits<P>::R> (&acc)[12])
 {
     using R = typename PrecTraits<P>::R;
@@ -310,7 +319,13 @@ __device__ __forceinline__ void hop_accumulate_rolled(const HopArgs &a, int i, c
         const size_t dir_off = (size_t)mu * link_dir_bytes(P, g.stride);
         LinkIO<P>::load(static_cast<const char *>(fwd ? a.links_out : a.links_in) + dir_off, g.stride, fwd ? i : j, u);
         cx<R> psi[12];
-        SpinorIO<P>::load(a.in, g.stride, j, psi);
+        if constexpr (CANON) {
+            const double2 *q = static_cast<const double2 *>(a.in) + 12 * canon_site(c, a.out_parity, mu, j);
+#pragma unroll
+            for (int k = 0; k < 12; ++k) psi[k] = {q[k].x, q[k].y};
+        } else {
+            SpinorIO<P>::load(a.in, g.stride, j, psi);
+        }
         cx<R> h1[3], h2[3];
 #pragma unroll
         for (int k = 0; k < 3; ++k) {

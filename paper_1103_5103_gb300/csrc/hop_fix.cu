@@ -31,4 +31,43 @@ int hop_fix_reduce_launch(int kind, int dagger, const HopArgs &a, const void *ep
     return WL_OK;
 }
 
+// Canonical operator application; tmp: one internal FP64 spinor (M_prec).
+int dslash_fix(wl_gauge *g, const void *in, void *out, double kappa, int op, int dagger, void *tmp, cudaStream_t s)
+{
+    DslashArgs d;
+    for (int p = 0; p < 2; ++p) {
+        HopArgs &a = d.a[p];
+        a = HopArgs{};
+        a.g = g->lat->geom;
+        a.out_parity = p;
+        a.nrhs = a.ngroups = 1;
+        a.links_out = g->links[prec_index(WL_F64)][p];
+        a.links_in = g->links[prec_index(WL_F64)][1 - p];
+        a.fix_out = g->fix_links[p];
+        a.fix_in = g->fix_links[1 - p];
+    }
+    d.in = static_cast<const double2 *>(in);
+    d.out = static_cast<double2 *>(out);
+    d.tmp = tmp;
+    // four warps per 16 sites while the chunks do not fill the SMs: 8^4 8.9
+    // against 12.6 us (M), 12.7 against 23.1 (M_prec), 20x12x6x14 M_prec 29.9
+    // against 32.2; from two waves on the extra pass through shared memory
+    // costs more (16^4 59 against 44)
+    const unsigned chunks = (unsigned)((g->lat->geom.Vh + 15) / 16) * (op == WL_OP_MPREC ? 1u : 2u);
+    const bool split = chunks <= 5u * (unsigned)sm_count();
+    if (op == WL_OP_MPREC) {
+        d.coef = -kappa * kappa;
+        d.add = 1;
+        WL_CUDA_TRY((dagger ? launch_dslash_fix<true, 1>(d, split, s) : launch_dslash_fix<false, 1>(d, split, s)));
+        note_launch(s);
+        WL_CUDA_TRY((dagger ? launch_dslash_fix<true, 2>(d, split, s) : launch_dslash_fix<false, 2>(d, split, s)));
+    } else {
+        d.add = op == WL_OP_M;
+        d.coef = d.add ? -kappa : 1.0;
+        WL_CUDA_TRY((dagger ? launch_dslash_fix<true, 0>(d, split, s) : launch_dslash_fix<false, 0>(d, split, s)));
+    }
+    note_launch(s);
+    return WL_OK;
+}
+
 }  // namespace wl

@@ -120,7 +120,7 @@ struct FixRaw {
     double2 a[3], b[3];
 };
 
-__device__ __forceinline__ void fix_load(FixRaw &x, const void *in, int j, unsigned off_u, unsigned off_l, int stride)
+__device__ __forceinline__ void fix_load(FixRaw &x, const void *in, size_t j, unsigned off_u, unsigned off_l, int stride)
 {
     const double2 *q = static_cast<const double2 *>(in) + j;
 #pragma unroll
@@ -234,73 +234,83 @@ __device__ __forceinline__ double fix_out(i64 v, double scale)
     return ((hi - (0x1p84 + 0x1p63 + 0x1p52)) + lo) * scale;
 }
 
-// D in at site i by its two threads: thread s gets spin s in acc[0..2] and
-// spin 3 - s in acc[3..5].  Every lane of the warp takes part.
-template <bool DAG>
-__device__ __forceinline__ void hop_half(const HopArgs &a, const void *in, int i, int s, cx<double> (&acc)[6])
+// The thread's accumulators and their scale.
+struct FixAcc {
+    i64 up[6], low[6];   // spin s; the spin that the direction couples to it
+    int E;
+    bool special;
+    __device__ __forceinline__ void clear()
+    {
+#pragma unroll
+        for (int k = 0; k < 6; ++k) up[k] = low[k] = 0;
+        E = kFixMinExp;
+        special = false;
+    }
+};
+
+// What the transporters need of the output site.
+struct FixSite {
+    Coord c;
+    int i;            // even-odd index (links)
+    int nb[8];        // neighbours: forward, backward in x, y, z, t
+    bool nf, nbk;     // time boundary
+};
+
+__device__ __forceinline__ FixSite fix_site(const HopArgs &a, int i)
 {
     const Geom &g = a.g;
-    const Coord q = site_coord(g, i, a.out_parity);
-    const int rowbase = i - (q.x >> 1);
-    int nb[8];
-    bool f0, f1, nf, nbk;
-    neighbours<0>(g, i, q, rowbase, nb[0], nb[1], f0, f1);
-    neighbours<1>(g, i, q, rowbase, nb[2], nb[3], f0, f1);
-    neighbours<2>(g, i, q, rowbase, nb[4], nb[5], f0, f1);
-    neighbours<3>(g, i, q, rowbase, nb[6], nb[7], nf, nbk);
+    FixSite q;
+    q.c = site_coord(g, i, a.out_parity);
+    const int rowbase = i - (q.c.x >> 1);
+    bool f0, f1;
+    neighbours<0>(g, i, q.c, rowbase, q.nb[0], q.nb[1], f0, f1);
+    neighbours<1>(g, i, q.c, rowbase, q.nb[2], q.nb[3], f0, f1);
+    neighbours<2>(g, i, q.c, rowbase, q.nb[4], q.nb[5], f0, f1);
+    neighbours<3>(g, i, q.c, rowbase, q.nb[6], q.nb[7], q.nf, q.nbk);
 #pragma unroll
-    for (int k = 0; k < 8; ++k) nb[k] = WL_LOAD_IDX(nb[k], g.stride, 1);
-    const int il = WL_LOAD_IDX(i, g.stride, 3);
-    bool special = false;
-    int E = kFixMinExp;
-    // spin s, and the spin coupled to it: 3 - s in x and y, 2 + s in z and t
-    i64 up[6], low[6];
-#pragma unroll
-    for (int k = 0; k < 6; ++k) up[k] = low[k] = 0;
-    const int4 *lo = static_cast<const int4 *>(a.fix_out), *li = static_cast<const int4 *>(a.fix_in);
+    for (int k = 0; k < 8; ++k) q.nb[k] = WL_LOAD_IDX(q.nb[k], g.stride, 1);
+    q.i = WL_LOAD_IDX(i, g.stride, 3);
+    return q;
+}
+
+// Both transporters of directions x, z (SWAP) or y, t, by m = 0, 1.  CANON:
+// the input is a canonical field ([site][12]) instead of an internal one.
+template <bool DAG, bool CANON, bool SWAP>
+__device__ __forceinline__ void fix_direction(const HopArgs &a, const void *in, const FixSite &q, int m, int s,
+                                              FixAcc &A)
+{
+    const Geom &g = a.g;
+    const int mu = (SWAP ? 0 : 1) + 2 * m;
+    // signs of the phase of spin s in 1 - gamma: x (+, +), z (+, -); y (-, +), t (+, +)
     constexpr int PF = DAG ? -1 : 0;   // 1 + gamma in the forward hops of the adjoint
-    const unsigned off_u = (unsigned)(3 * s * g.stride);
-    unsigned off_l = (unsigned)(3 * (3 - s) * g.stride);
+    const int f = (SWAP ? (m ? -s : 0) : (m ? 0 : s - 1)) ^ PF;
+    const int cs = CANON ? 1 : g.stride;
+    const unsigned off_u = (unsigned)(3 * s * cs), off_l = (unsigned)(3 * (m ? 2 + s : 3 - s) * cs);
+    const int4 *lo = static_cast<const int4 *>(a.fix_out), *li = static_cast<const int4 *>(a.fix_in);
+    FixRaw x;
+    int4 u[9];
 #pragma unroll 1
-    for (int m = 0; m < 2; ++m) {   // x, y, then z, t
-        // signs of the phase of spin s in 1 - gamma: x (+, +), z (+, -); y (-, +), t (+, +)
-        const int fx = (m ? -s : 0) ^ PF, fy = (m ? 0 : s - 1) ^ PF;
-        FixRaw x;
-        int4 u[9];
-#pragma unroll 1
-        for (int cj = 0; cj >= -1; --cj) {   // forward, backward
-            const int j = m ? (cj ? nb[5] : nb[4]) : (cj ? nb[1] : nb[0]);
-            fix_load(x, in, j, off_u, off_l, g.stride);
-            fix_load_link(u, (cj ? li : lo) + fix_link(g, 2 * m, cj ? j : il), cj);
-            fix_transport<true>(x, u, fx ^ cj, cj, false, E, special, up, low);
-        }
-#pragma unroll 1
-        for (int cj = 0; cj >= -1; --cj) {
-            const int j = m ? (cj ? nb[7] : nb[6]) : (cj ? nb[3] : nb[2]);
-            fix_load(x, in, j, off_u, off_l, g.stride);
-            fix_load_link(u, (cj ? li : lo) + fix_link(g, 1 + 2 * m, cj ? j : il), cj);
-            fix_transport<false>(x, u, fy ^ cj, cj, m && (cj ? nbk : nf), E, special, up, low);
-        }
-        off_l = (unsigned)(3 * (2 + s) * g.stride);
-        // the pair moves to the larger of its two scales and exchanges the
-        // lower spins: after x, y thread s holds spin 3 - s and goes on with
-        // 2 + s; after z, t it gets 3 - s back
-        const int Eo = __shfl_xor_sync(0xffffffffu, E, 16);
-        const int sh = max(0, Eo - E);
-        E = max(E, Eo);
-#pragma unroll
-        for (int k = 0; k < 6; ++k) {
-            up[k] = fix_sar(up[k], sh);
-            low[k] = __shfl_xor_sync(0xffffffffu, fix_sar(low[k], sh), 16);
-        }
+    for (int cj = 0; cj >= -1; --cj) {   // forward, backward
+        const int j = m ? (cj ? (SWAP ? q.nb[5] : q.nb[7]) : (SWAP ? q.nb[4] : q.nb[6]))
+                        : (cj ? (SWAP ? q.nb[1] : q.nb[3]) : (SWAP ? q.nb[0] : q.nb[2]));
+        fix_load(x, in, CANON ? 12 * canon_site(q.c, a.out_parity, mu, j) : (size_t)j, off_u, off_l, cs);
+        fix_load_link(u, (cj ? li : lo) + fix_link(g, mu, cj ? j : q.i), cj);
+        fix_transport<SWAP>(x, u, f ^ cj, cj, !SWAP && m && (cj ? q.nbk : q.nf), A.E, A.special, A.up, A.low);
     }
-    special = __shfl_xor_sync(0xffffffffu, special ? 1 : 0, 16) || special;
-    if (!special) {
-        const double scale = __hiloint2double((E + 2 - kFixFrac) << 20, 0);   // 2^(E - 1023 - 56)
+}
+
+// FP64 values of the accumulators (acc[0..2] spin s, acc[3..5] spin 3 - s),
+// or those of the FP64 transporters for a special site.
+template <bool DAG, bool CANON>
+__device__ __forceinline__ void fix_values(const HopArgs &a, const void *in, int i, int s, const FixAcc &A,
+                                           cx<double> (&acc)[6])
+{
+    if (!A.special) {
+        const double scale = __hiloint2double((A.E + 2 - kFixFrac) << 20, 0);   // 2^(E - 1023 - 56)
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
-            acc[k] = {fix_out(up[2 * k], scale), fix_out(up[2 * k + 1], scale)};
-            acc[3 + k] = {fix_out(low[2 * k], scale), fix_out(low[2 * k + 1], scale)};
+            acc[k] = {fix_out(A.up[2 * k], scale), fix_out(A.up[2 * k + 1], scale)};
+            acc[3 + k] = {fix_out(A.low[2 * k], scale), fix_out(A.low[2 * k + 1], scale)};
         }
     } else {
         HopArgs b = a;
@@ -308,13 +318,41 @@ __device__ __forceinline__ void hop_half(const HopArgs &a, const void *in, int i
         cx<double> full[12];
 #pragma unroll
         for (int k = 0; k < 12; ++k) full[k] = acc_zero<double>();
-        hop_accumulate_rolled<WL_F64, DAG>(b, i, full);
+        hop_accumulate_rolled<WL_F64, DAG, CANON>(b, i, full);
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
             acc[k] = s ? full[3 + k] : full[k];
             acc[3 + k] = s ? full[6 + k] : full[9 + k];
         }
     }
+}
+
+// D in at site i by its two threads: thread s gets spin s in acc[0..2] and
+// spin 3 - s in acc[3..5].  Every lane of the warp takes part.
+template <bool DAG, bool CANON>
+__device__ __forceinline__ void hop_half(const HopArgs &a, const void *in, int i, int s, cx<double> (&acc)[6])
+{
+    const FixSite q = fix_site(a, i);
+    FixAcc A;
+    A.clear();
+#pragma unroll 1
+    for (int m = 0; m < 2; ++m) {   // x, y, then z, t
+        fix_direction<DAG, CANON, true>(a, in, q, m, s, A);
+        fix_direction<DAG, CANON, false>(a, in, q, m, s, A);
+        // the pair moves to the larger of its two scales and exchanges the
+        // lower spins: after x, y thread s holds spin 3 - s and goes on with
+        // 2 + s; after z, t it gets 3 - s back
+        const int Eo = __shfl_xor_sync(0xffffffffu, A.E, 16);
+        const int sh = max(0, Eo - A.E);
+        A.E = max(A.E, Eo);
+#pragma unroll
+        for (int k = 0; k < 6; ++k) {
+            A.up[k] = fix_sar(A.up[k], sh);
+            A.low[k] = __shfl_xor_sync(0xffffffffu, fix_sar(A.low[k], sh), 16);
+        }
+    }
+    A.special = __shfl_xor_sync(0xffffffffu, A.special ? 1 : 0, 16) || A.special;
+    fix_values<DAG, CANON>(a, in, i, s, A, acc);
 }
 
 // Load and store of a thread's half of a site: spins s and 3 - s.
@@ -353,7 +391,7 @@ __device__ __forceinline__ void hop_fix_task(const HopArgs &a, const EpiStore &e
     const bool active = i0 < a.g.Vh;
     const int i = active ? i0 : a.g.Vh - 1;
     cx<double> acc[6];
-    hop_half<DAG>(a, static_cast<const char *>(a.in) + (size_t)r * a.rhs_bytes, i, s, acc);
+    hop_half<DAG, false>(a, static_cast<const char *>(a.in) + (size_t)r * a.rhs_bytes, i, s, acc);
     if (!active) return;
     const size_t off = (size_t)r * e.rhs_bytes;
     if (e.out_raw) half_store(static_cast<char *>(e.out_raw) + off, a.g.stride, s, i, acc);
@@ -422,7 +460,7 @@ __global__ void __launch_bounds__(128, 4) k_hop_fix_reduce(HopArgs a, EpiReduce<
     if (i0 - (lane & 15) < a.g.Vh) {   // the whole warp
         const int i = active ? i0 : a.g.Vh - 1;
         cx<double> acc[6];
-        hop_half<DAG>(a, static_cast<const char *>(a.in) + (size_t)r * a.rhs_bytes, i, s, acc);
+        hop_half<DAG, false>(a, static_cast<const char *>(a.in) + (size_t)r * a.rhs_bytes, i, s, acc);
         if (active) {
             const size_t off = (size_t)r * e.rhs_bytes;
             cx<double> x[6], o[6];
@@ -455,6 +493,125 @@ template <bool DAG, int KIND>
 void launch_k_hop_fix_reduce(const HopArgs &a, const EpiReduce<KIND> &e, cudaStream_t s)
 {
     launch_chained(k_hop_fix_reduce<DAG, KIND>, (a.g.Vh + 63) / 64 * a.nrhs, 128, s, a, e);
+}
+
+// ------------------------------------------- canonical operator application
+// wilson_dslash in FP64 without the layout passes: the hops read and write
+// the canonical fields.
+//   STAGE 0: out = add in + coef D in on both parities in one launch
+//   STAGE 1: tmp_o = D_oe in_e (internal);  STAGE 2: out_e = in_e + coef D_eo
+//   tmp_o, out_o = 0  (M_prec)
+struct DslashArgs {
+    HopArgs a[2];         // by output parity
+    const double2 *in;    // canonical
+    double2 *out;         // canonical
+    void *tmp;            // internal, odd sites (stages 1, 2)
+    double coef;
+    int add;
+};
+
+// Store of a thread's half of a site, by stage.  active threads only.
+template <int STAGE>
+__device__ __forceinline__ void dslash_finish(const DslashArgs &d, const HopArgs &a, int i, int s, cx<double> (&acc)[6])
+{
+    if constexpr (STAGE == 1) {
+        half_store(d.tmp, a.g.stride, s, i, acc);
+    } else {
+        const Coord c = site_coord(a.g, i, a.out_parity);
+        const size_t bit = c.x & 1, n = 2 * (size_t)i + bit;
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+                const size_t e = 12 * n + 3 * (h ? 3 - s : s) + k;
+                // product, then sum, each rounded: the internal hops' epilogue
+                cx<double> o = {__dmul_rn(d.coef, acc[3 * h + k].re), __dmul_rn(d.coef, acc[3 * h + k].im)};
+                if (STAGE == 2 || d.add) {
+                    const double2 x = d.in[e];
+                    o = {__dadd_rn(o.re, x.x), __dadd_rn(o.im, x.y)};
+                }
+                d.out[e] = make_double2(o.re, o.im);
+                if (STAGE == 2) d.out[12 * (n ^ 1) + 3 * (h ? 3 - s : s) + k] = make_double2(0.0, 0.0);
+            }
+    }
+}
+
+template <bool DAG, int STAGE>
+__global__ void __launch_bounds__(128, 4) k_dslash_fix(DslashArgs d)
+{
+    const int lane = threadIdx.x & 31, s = lane >> 4;
+    const unsigned task = blockIdx.x * 4 + (threadIdx.x >> 5) + chain_begin();
+    const int p = STAGE == 0 ? (int)(task & 1) : STAGE == 1 ? 1 : 0;
+    const HopArgs &a = d.a[p];
+    const int i0 = (int)(STAGE == 0 ? task >> 1 : task) * 16 + (lane & 15);
+    if (i0 - (lane & 15) >= a.g.Vh) return;   // the whole warp
+    const int i = min(i0, a.g.Vh - 1);
+    cx<double> acc[6];
+    hop_half<DAG, STAGE != 2>(a, STAGE == 2 ? d.tmp : static_cast<const void *>(d.in), i, s, acc);
+    if (i0 < a.g.Vh) dslash_finish<STAGE>(d, a, i, s, acc);
+}
+
+// The same with the four directions of 16 sites on the four warps of a
+// block: a quarter of the serial work per thread, for lattices that do not
+// fill the GPU.  The warps' sums meet in shared memory.
+template <bool DAG, int STAGE>
+__global__ void __launch_bounds__(128, 4) k_dslash_fix_split(DslashArgs d)
+{
+    __shared__ i64 sum[4][12][32];
+    __shared__ int exps[4][32];
+    const int lane = threadIdx.x & 31, s = lane >> 4, w = threadIdx.x >> 5;
+    const unsigned task = blockIdx.x + chain_begin();
+    const int p = STAGE == 0 ? (int)(task & 1) : STAGE == 1 ? 1 : 0;
+    const HopArgs &a = d.a[p];
+    const int i0 = (int)(STAGE == 0 ? task >> 1 : task) * 16 + (lane & 15);
+    const int i = min(i0, a.g.Vh - 1);
+    const void *in = STAGE == 2 ? d.tmp : static_cast<const void *>(d.in);
+    const FixSite q = fix_site(a, i);
+    FixAcc A;
+    A.clear();
+    if (w & 1) fix_direction<DAG, STAGE != 2, false>(a, in, q, w >> 1, s, A);   // y, t
+    else fix_direction<DAG, STAGE != 2, true>(a, in, q, w >> 1, s, A);          // x, z
+#pragma unroll
+    for (int k = 0; k < 6; ++k) {
+        sum[w][k][lane] = A.up[k];
+        sum[w][6 + k][lane] = A.low[k];
+    }
+    exps[w][lane] = A.special ? -1 : A.E;
+    __syncthreads();
+    if (w != 0) return;
+    // thread s: spin s from its own sums, spin 3 - s from its own in x, y and
+    // from its partner's in z, t
+    A.special = false;
+    int Ew[4], Eo[4];
+    A.E = kFixMinExp;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        Ew[k] = exps[k][lane];
+        Eo[k] = exps[k][lane ^ 16];
+        A.special |= Ew[k] < 0 || Eo[k] < 0;
+        A.E = max(A.E, max(Ew[k], Eo[k]));
+    }
+#pragma unroll
+    for (int k = 0; k < 6; ++k) {
+        A.up[k] = A.low[k] = 0;
+#pragma unroll
+        for (int v = 0; v < 4; ++v) {
+            A.up[k] += fix_sar(sum[v][k][lane], A.E - Ew[v]);
+            A.low[k] += fix_sar(sum[v][6 + k][v < 2 ? lane : lane ^ 16], A.E - (v < 2 ? Ew[v] : Eo[v]));
+        }
+    }
+    if (i0 >= a.g.Vh) return;
+    cx<double> acc[6];
+    fix_values<DAG, STAGE != 2>(a, in, i, s, A, acc);
+    dslash_finish<STAGE>(d, a, i, s, acc);
+}
+
+template <bool DAG, int STAGE>
+cudaError_t launch_dslash_fix(const DslashArgs &d, bool split, cudaStream_t s)
+{
+    const unsigned chunks = (unsigned)((d.a[0].g.Vh + 15) / 16) * (STAGE == 0 ? 2u : 1u);
+    return split ? launch_chained(k_dslash_fix_split<DAG, STAGE>, chunks, 128, s, d)
+                 : launch_chained(k_dslash_fix<DAG, STAGE>, (chunks + 3) / 4, 128, s, d);
 }
 
 }  // namespace wl

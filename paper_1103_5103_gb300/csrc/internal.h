@@ -133,6 +133,12 @@ int hop_reduce(wl_gauge *g, int kind, const Vec &tmp, const Vec &xin, double a1,
 // Workspace of site_sum for nrhs right-hand sides (group tickets at zero).
 int red_buffer(wl_gauge *g, const std::string &name, int nrhs, void **out, cudaStream_t s);
 
+// ---- hop_fix.cu: FP64 operator application (wilson_dslash) on canonical
+// device fields, where dslash_direct (dslash.cu) allows it; tmp: one internal
+// FP64 spinor, for WL_OP_MPREC
+bool dslash_direct(const wl_gauge *g, const void *in, const void *out, int prec);
+int dslash_fix(wl_gauge *g, const void *in, void *out, double kappa, int op, int dagger, void *tmp, cudaStream_t s);
+
 // ---- blas.cu (all on one parity; nrhs from the vectors)
 int blas_s_update(const Geom &g, const Vec &r, const Vec &v, const Vec &s_out, BiState *st, cudaStream_t s);
 // CG on the normal equations: x += alpha p, r -= alpha w, ||r||^2 -> stop

@@ -94,6 +94,7 @@ extern "C" int wilson_dslash_noalloc(wl_gauge *g, const void *in, void *out, dou
     const int dag = dagger ? 1 : 0;
     const void *cin[1] = {in};
     void *cout[1] = {out};
+    if (dslash_direct(g, in, out, prec)) return dslash_fix(g, in, out, kappa, op, dag, base, s);
     // every scratch buffer is fully written below before it is read, except
     // the odd output of M_prec, which is defined as zero
     WL_TRY(import_full(geo, cin, ie, io, s));

@@ -169,3 +169,36 @@ def test_out_of_range_sites_take_the_fp64_path(api, value):
     assert np.abs(got[ok] - ref[ok]).max() <= 2.0 ** -50 * scale + 1e-323
     if value == 0.0:
         assert np.array_equal(got == 0, ref == 0)
+
+
+@pytest.mark.parametrize("dims", [(2, 2, 2, 2), (6, 4, 2, 10), (8, 8, 8, 8), (10, 14, 12, 16), (12, 14, 12, 16)])
+@pytest.mark.parametrize("kind", ["gauss", "sites", "special"])
+def test_canonical_application_is_the_internal_one(api, dims, kind):
+    """wilson_dslash in FP64 reads and writes the canonical fields, with the
+    directions of a site on four warps up to 760 chunks of 16 sites (10x14x12x16:
+    840 chunks per parity, 2^4: one ragged chunk) and in one thread above.  It
+    agrees with the same application from page-locked host fields, which goes
+    through the layout passes and the internal hops: the sums differ by the
+    order of their rescaling, four units of 2^(E-56) per hop."""
+    U = synth.gauge_field(dims, 0.5, seed=31)
+    lat = api.Lattice(dims)
+    g = api.Gauge(lat, torch.from_numpy(U).cuda(), precs=("f64",))
+    psi = _source(dims, "gauss" if kind == "special" else kind)
+    if kind == "special":
+        psi[3, 2, 1], psi[5 % len(psi), 0, 0] = np.nan, 1e300
+    dev = torch.from_numpy(np.ascontiguousarray(psi)).cuda()
+    host = torch.from_numpy(np.ascontiguousarray(psi)).pin_memory()
+    for op in (api.OP_HOP, api.OP_M, api.OP_MPREC):
+        for f in (api.wilson_dslash, api.wilson_dslash_dag):
+            a = torch.full_like(dev, float("nan"))
+            b = torch.full_like(host, float("nan")).pin_memory()
+            f(g, dev, a, 0.13, "f64", op)
+            f(g, host, b, 0.13, "f64", op)
+            torch.cuda.synchronize()
+            a, b = a.cpu().numpy(), b.numpy()
+            assert np.array_equal(np.isnan(a), np.isnan(b))
+            ok = np.isfinite(b) & (np.abs(b) < 1e290)
+            big = np.abs(b[ok]).max()
+            assert np.abs(a[ok] - b[ok]).max() <= 2.0 ** -50 * big
+            if op == api.OP_MPREC:
+                assert np.all(a[synth.parity(dims) == 1] == 0)
