@@ -26,15 +26,9 @@ static int check_links(wl_gauge *g, int prec)
     return WL_OK;
 }
 
-int hop_ex(wl_gauge *g, const Vec &in, const Vec &out, const Vec *x1, double a1, const Vec *x2, double a2,
-           double coef, int out_parity, int dagger, int rhs_block, const int *skip, int skip_stride, cudaStream_t s,
-           const Vec *out_raw)
+// Arguments of a hop from in to sites of parity out_parity.
+static HopArgs hop_args(wl_gauge *g, const Vec &in, int out_parity)
 {
-    WL_TRY(check_links(g, in.prec));
-    if (in.prec != out.prec || (x1 && x1->prec != in.prec) || (x2 && x2->prec != in.prec)) {
-        set_error("hop: precision mismatch");
-        return WL_ERR_ARG;
-    }
     HopArgs a;
     a.g = g->lat->geom;
     a.out_parity = out_parity;
@@ -46,6 +40,21 @@ int hop_ex(wl_gauge *g, const Vec &in, const Vec &out, const Vec *x1, double a1,
     a.links_in = links_of(g, in.prec, 1 - out_parity);
     a.fix_out = g->fix_links[out_parity];
     a.fix_in = g->fix_links[1 - out_parity];
+    a.skip = nullptr;
+    a.skip_stride = 0;
+    return a;
+}
+
+int hop_ex(wl_gauge *g, const Vec &in, const Vec &out, const Vec *x1, double a1, const Vec *x2, double a2,
+           double coef, int out_parity, int dagger, int rhs_block, const int *skip, int skip_stride, cudaStream_t s,
+           const Vec *out_raw)
+{
+    WL_TRY(check_links(g, in.prec));
+    if (in.prec != out.prec || (x1 && x1->prec != in.prec) || (x2 && x2->prec != in.prec)) {
+        set_error("hop: precision mismatch");
+        return WL_ERR_ARG;
+    }
+    HopArgs a = hop_args(g, in, out_parity);
     a.skip = skip;
     a.skip_stride = skip_stride;
     EpiStore e;
@@ -94,17 +103,7 @@ static int hop_reduce_k(wl_gauge *g, const Vec &tmp, const Vec &xin, double a1, 
                         double *partials, int part, int parts, cudaStream_t s)
 {
     WL_TRY(check_links(g, tmp.prec));
-    HopArgs a;
-    a.g = g->lat->geom;
-    a.out_parity = out_parity;
-    a.nrhs = tmp.nrhs;
-    a.ngroups = tmp.nrhs;
-    a.in = tmp.ptr;
-    a.rhs_bytes = tmp.rhs_bytes;
-    a.links_out = links_of(g, tmp.prec, out_parity);
-    a.links_in = links_of(g, tmp.prec, 1 - out_parity);
-    a.fix_out = g->fix_links[out_parity];
-    a.fix_in = g->fix_links[1 - out_parity];
+    HopArgs a = hop_args(g, tmp, out_parity);
     a.skip = &state[0].done;
     a.skip_stride = sizeof(BiState) / sizeof(int);
     EpiReduce<KIND> e;
@@ -213,12 +212,18 @@ extern "C" int wilson_hop_multi(wl_gauge *g, const void *in, void *out, const vo
 
 namespace wl {
 
+static bool device_fields(const void *in, const void *out);
+
 // FP64 operator applications read and write the canonical fields in the hop
 // itself (8^4 28.5 -> 8.9 us, 24^3x64 612 -> 499 us).  Page-locked host fields
 // keep the layout passes, which read each site over the host link once.
 bool dslash_direct(const wl_gauge *g, const void *in, const void *out, int prec)
 {
-    if (prec != WL_F64 || !g->fix_links[0]) return false;
+    return prec == WL_F64 && g->fix_links[0] && device_fields(in, out);
+}
+
+static bool device_fields(const void *in, const void *out)
+{
     for (const void *p : {in, out}) {
         cudaPointerAttributes pa{};
         if (cudaPointerGetAttributes(&pa, p) != cudaSuccess || pa.type != cudaMemoryTypeDevice) {
@@ -230,6 +235,13 @@ bool dslash_direct(const wl_gauge *g, const void *in, const void *out, int prec)
 }
 
 }  // namespace wl
+
+// FP32, FP16 and double-float: whether the last hop stores to the canonical
+// field (device memory).  D and M, both parities in one launch, gain at every
+// size (FP32 8^4 15.2 -> 12.0 us, 16^4 28.7 -> 18.0, 24^3x64 211 -> 167; DF
+// 24^3x64 786 -> 619); M_prec, one parity after another, up to 16384 sites of
+// one (20x12x6x14 18.6 -> 16.8; 16^4 26.6 -> 29.8 us).
+constexpr int kCanonPrecSites = 16384;
 
 static int dslash_common(wl_gauge *g, const void *in, void *out, double kappa, int prec, int op, int dagger,
                          void *stream)
@@ -255,6 +267,23 @@ static int dslash_common(wl_gauge *g, const void *in, void *out, double kappa, i
     const void *cin[1] = {in};
     void *cout[1] = {out};
     WL_TRY(import_full(geo, cin, ie, io, s));
+    if (prec != WL_F64 && (op != WL_OP_MPREC || geo.Vh <= kCanonPrecSites) && device_fields(in, out)) {
+        CanonHop h{};
+        for (int p = 0; p < 2; ++p) {
+            h.a[p] = hop_args(g, op == WL_OP_MPREC ? oo : p ? ie : io, p);
+            if (op != WL_OP_HOP) h.x[p] = p ? io.ptr : ie.ptr;
+        }
+        h.a1 = 1.0;
+        h.coef = op == WL_OP_HOP ? 1.0 : op == WL_OP_M ? -kappa : -kappa * kappa;
+        h.out = static_cast<double2 *>(out);
+        h.both = op != WL_OP_MPREC;
+        if (op == WL_OP_MPREC) WL_TRY(hop(g, ie, oo, nullptr, 1.0, WL_ODD, dagger, 1, s));
+        switch (prec) {
+        case WL_F32: return hop_canon_launch_prec<WL_F32>(dagger, h, s);
+        case WL_F16: return hop_canon_launch_prec<WL_F16>(dagger, h, s);
+        default: return hop_canon_launch_prec<WL_DF>(dagger, h, s);
+        }
+    }
     if (op == WL_OP_HOP) {
         WL_TRY(hop(g, io, oe, nullptr, 1.0, WL_EVEN, dagger, 1, s));
         WL_TRY(hop(g, ie, oo, nullptr, 1.0, WL_ODD, dagger, 1, s));

@@ -1139,6 +1139,69 @@ __global__ void __launch_bounds__(128, ReduceMinBlocks<P>::value) k_hop_reduce(H
     hop_reduce_body<P, DAG, KIND>(a, e);
 }
 
+// Last hop of an operator application (FP32, FP16 and double-float), storing to the canonical field: saves the export pass and,
+// with both parities in one launch, a hop.  Values as if stored internally
+// and exported.
+//   both = 1: out = a1 x + coef D in on both parities (in, x: [parity])
+//   both = 0: the even parity; the odd output sites are set to zero
+struct CanonHop {
+    HopArgs a[2];        // by output parity; a[p].in: the other parity's spinor
+    const void *x[2];    // null: no a1 x term
+    double a1, coef;
+    double2 *out;
+    int both;
+};
+
+template <int P, bool DAG>
+__global__ void __launch_bounds__(128) k_hop_canon(CanonHop h)
+{
+    using R = typename PrecTraits<P>::R;
+    const int z = chain_begin();
+    const int p = h.both ? (int)(blockIdx.x & 1) + z : z;
+    const HopArgs &a = h.a[p];
+    const int i = (int)(h.both ? blockIdx.x >> 1 : blockIdx.x) * 128 + threadIdx.x + z;
+    if (i >= a.g.Vh) return;
+    cx<R> acc[1][12];
+#pragma unroll
+    for (int k = 0; k < 12; ++k) acc[0][k] = acc_zero<R>();
+    if constexpr (P == WL_DF) hop_accumulate_rolled<P, DAG>(a, i, acc[0]);
+    else hop_accumulate_batch<P, DAG>(a, a.in, i, acc[0]);
+    cx<R> o[12];
+    const R c = Conv<R>::from(h.coef);
+#pragma unroll
+    for (int k = 0; k < 12; ++k) o[k] = c * acc[0][k];
+    if (h.x[p]) {
+        cx<R> v[12];
+        SpinorIO<P>::load(h.x[p], a.g.stride, i, v);
+#pragma unroll
+        for (int k = 0; k < 12; ++k) o[k] = o[k] + Conv<R>::from(h.a1) * v[k];
+    }
+    SpinorIO<P>::roundtrip(o);
+    const size_t n = 2 * (size_t)i + (site_coord(a.g, i, a.out_parity).x & 1);
+#pragma unroll
+    for (int k = 0; k < 12; ++k) {
+        if constexpr (P == WL_DF) {
+            const df re = df_normalize(o[k].re), im = df_normalize(o[k].im);
+            h.out[12 * n + k] = make_double2(to_double(re), to_double(im));
+        } else {
+            h.out[12 * n + k] = make_double2(to_double(o[k].re), to_double(o[k].im));
+        }
+        if (!h.both) h.out[12 * (n ^ 1) + k] = make_double2(0.0, 0.0);
+    }
+}
+
+template <int P>
+int hop_canon_launch(int dagger, const CanonHop &h, cudaStream_t s)
+{
+    const unsigned blocks = (unsigned)((h.a[0].g.Vh + 127) / 128) * (h.both ? 2u : 1u);
+    WL_CUDA_TRY(dagger ? launch_chained(k_hop_canon<P, true>, blocks, 128, s, h)
+                       : launch_chained(k_hop_canon<P, false>, blocks, 128, s, h));
+    note_launch(s);
+    return WL_OK;
+}
+// Instantiated in hop_<prec>.cu for FP32, FP16 and double-float.
+template <int P> int hop_canon_launch_prec(int dagger, const CanonHop &h, cudaStream_t s);
+
 // ------------------------------------------------------------ launchers
 // Instantiated per precision in hop_<prec>.cu.
 

@@ -1,7 +1,7 @@
 // Hop kernel instantiations for DF (one translation unit per precision so the
 // library builds in parallel).  Variant v = 100 * (rhs per thread) + (minimum resident
 // blocks per SM requested from the register allocator).
-#include "hop.cuh"
+#include "hop_batch.cuh"
 
 namespace wl {
 
@@ -35,6 +35,12 @@ int hop_reduce_launch_prec<WL_DF>(int kind, int dagger, const HopArgs &a, const 
     }
     WL_CUDA_TRY(cudaGetLastError());
     return WL_OK;
+}
+
+template <>
+int hop_canon_launch_prec<WL_DF>(int dagger, const CanonHop &h, cudaStream_t s)
+{
+    return hop_canon_launch<WL_DF>(dagger, h, s);
 }
 
 }  // namespace wl

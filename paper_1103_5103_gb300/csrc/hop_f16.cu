@@ -65,4 +65,10 @@ int hop_reduce_launch_prec<WL_F16>(int kind, int dagger, const HopArgs &a, const
     return WL_OK;
 }
 
+template <>
+int hop_canon_launch_prec<WL_F16>(int dagger, const CanonHop &h, cudaStream_t s)
+{
+    return hop_canon_launch<WL_F16>(dagger, h, s);
+}
+
 }  // namespace wl

@@ -71,4 +71,10 @@ int hop_reduce_launch_prec<WL_F32>(int kind, int dagger, const HopArgs &a, const
     return WL_OK;
 }
 
+template <>
+int hop_canon_launch_prec<WL_F32>(int dagger, const CanonHop &h, cudaStream_t s)
+{
+    return hop_canon_launch<WL_F32>(dagger, h, s);
+}
+
 }  // namespace wl
