@@ -723,7 +723,9 @@ int canon_dots(const void *const *a, const void *const *in, int n, int nrhs, siz
 // r_o = b_o - x_o + kappa * Dx, the odd part of the full-lattice residual,
 // reduced to norm2[r] = ||r_o||^2.
 
-template <int PO>
+// HAS_B = false: b_o = 0 (a source without an odd part): x_o = kappa Dx, one
+// read and a quarter of the FP64 operations less.
+template <int PO, bool HAS_B>
 __global__ void __launch_bounds__(kBlock) k_recon(Geom g, Vec bo, Vec dx, double kappa, Vec xo, double *norm2,
                                                   double *partials, unsigned *tickets)
 {
@@ -732,24 +734,27 @@ __global__ void __launch_bounds__(kBlock) k_recon(Geom g, Vec bo, Vec dx, double
     double red[1] = {0.0};
     if (q.i < g.Vh) {
         cx<R> b[12], d[12], x[12];
-        SpinorIO<PO>::load(bo.rhs(q.r), g.stride, q.i, b);
+        if constexpr (HAS_B) SpinorIO<PO>::load(bo.rhs(q.r), g.stride, q.i, b);
         SpinorIO<PO>::load(dx.rhs(q.r), g.stride, q.i, d);
         const R k = Conv<R>::from(kappa);
         typename NormT<R>::T n = 0;
 #pragma unroll
         for (int c = 0; c < 12; ++c) {
             cx<R> ro;
-            if constexpr (PO == WL_F64) {
+            if constexpr (PO == WL_F64 && HAS_B) {
                 // x = b + kappa d in one rounding; its rounding error
                 // ro = (b - x) + kappa d, with the product fused again
                 // (the FP64 pipe bounds this pass: 4 operations per real
                 // instead of 5)
                 x[c] = {fma(k, d[c].re, b[c].re), fma(k, d[c].im, b[c].im)};
                 ro = {fma(k, d[c].re, b[c].re - x[c].re), fma(k, d[c].im, b[c].im - x[c].im)};
+            } else if constexpr (PO == WL_F64) {
+                x[c] = {k * d[c].re, k * d[c].im};
+                ro = {fma(k, d[c].re, -x[c].re), fma(k, d[c].im, -x[c].im)};
             } else {
                 const cx<R> kd = k * d[c];
-                x[c] = b[c] + kd;
-                ro = (b[c] - x[c]) + kd;
+                x[c] = HAS_B ? b[c] + kd : kd;
+                ro = HAS_B ? (b[c] - x[c]) + kd : kd - x[c];
             }
             norm_acc(n, ro.re);
             norm_acc(n, ro.im);
@@ -763,13 +768,18 @@ __global__ void __launch_bounds__(kBlock) k_recon(Geom g, Vec bo, Vec dx, double
         norm2[q.r] = tot[0];
 }
 
-int blas_recon(const Geom &g, const Vec &bo, const Vec &dx, double kappa, const Vec &xo, double *norm2_dev,
+int blas_recon(const Geom &g, const Vec *bo, const Vec &dx, double kappa, const Vec &xo, double *norm2_dev,
                double *partials, unsigned *tickets, cudaStream_t s)
 {
     const int gr = grid_of(g, xo.nrhs);
-    if (xo.prec == WL_DF) launch_chained(k_recon<WL_DF>, gr, kBlock, s, g, bo, dx, kappa, xo, norm2_dev, partials, tickets);
-    else if (xo.prec == WL_F64) launch_chained(k_recon<WL_F64>, gr, kBlock, s, g, bo, dx, kappa, xo, norm2_dev, partials, tickets);
+    const Vec b = bo ? *bo : dx;
+#define WL_RECON(PO, HB) launch_chained(k_recon<PO, HB>, gr, kBlock, s, g, b, dx, kappa, xo, norm2_dev, partials, tickets)
+    if (xo.prec == WL_DF && bo) WL_RECON(WL_DF, true);
+    else if (xo.prec == WL_DF) WL_RECON(WL_DF, false);
+    else if (xo.prec == WL_F64 && bo) WL_RECON(WL_F64, true);
+    else if (xo.prec == WL_F64) WL_RECON(WL_F64, false);
     else { set_error("blas_recon: outer precision only"); return WL_ERR_ARG; }
+#undef WL_RECON
     WL_CUDA_TRY(cudaGetLastError());
     note_launch(s);
     return WL_OK;

@@ -47,7 +47,7 @@ static HopArgs hop_args(wl_gauge *g, const Vec &in, int out_parity)
 
 int hop_ex(wl_gauge *g, const Vec &in, const Vec &out, const Vec *x1, double a1, const Vec *x2, double a2,
            double coef, int out_parity, int dagger, int rhs_block, const int *skip, int skip_stride, cudaStream_t s,
-           const Vec *out_raw)
+           const Vec *out_raw, const NormOut *norm)
 {
     WL_TRY(check_links(g, in.prec));
     if (in.prec != out.prec || (x1 && x1->prec != in.prec) || (x2 && x2->prec != in.prec)) {
@@ -68,6 +68,11 @@ int hop_ex(wl_gauge *g, const Vec &in, const Vec &out, const Vec *x1, double a1,
     e.rhs_bytes = out.rhs_bytes;
     if (out.rhs_bytes != in.rhs_bytes) { set_error("hop: rhs stride mismatch"); return WL_ERR_ARG; }
     const int variant = hop_variant_for(g, in.prec, in.nrhs, rhs_block);
+    if (norm && variant == 6000 && !dagger) {
+        WL_TRY(hop_fix_norm_launch(a, e, norm->norms, norm->partials, norm->tickets, s));
+        note_launch(s);
+        return WL_OK;
+    }
     int st = WL_ERR_ARG;
     switch (in.prec) {
     case WL_F64: st = hop_launch_prec<WL_F64>(variant, dagger, a, e, s); break;
@@ -80,6 +85,7 @@ int hop_ex(wl_gauge *g, const Vec &in, const Vec &out, const Vec *x1, double a1,
     WL_TRY(st);
     WL_CUDA_TRY(cudaGetLastError());
     note_launch(s);
+    if (norm) return blas_norm2(a.g, out, norm->norms, norm->partials, norm->tickets, s);
     return WL_OK;
 }
 

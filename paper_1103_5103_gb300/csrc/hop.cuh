@@ -1246,6 +1246,8 @@ int hop_launch_tma(int prec, int variant, int dagger, const HopArgs &a, const Ep
 
 // Fixed-point FP64 hop (hop_fix.cu).
 int hop_fix_launch(int dagger, const HopArgs &a, const EpiStore &e, int blocks_per_sm, cudaStream_t s);
+int hop_fix_norm_launch(const HopArgs &a, const EpiStore &e, double *norms, double *partials, unsigned *tickets,
+                        cudaStream_t s);
 int hop_fix_reduce_launch(int kind, int dagger, const HopArgs &a, const void *epi, cudaStream_t s);
 
 // Per-precision entry points (hop_<prec>.cu).  variant: see hop_variants().

@@ -11,6 +11,14 @@ int hop_fix_launch(int dagger, const HopArgs &a, const EpiStore &e, int blocks_p
     return WL_OK;
 }
 
+int hop_fix_norm_launch(const HopArgs &a, const EpiStore &e, double *norms, double *partials, unsigned *tickets,
+                        cudaStream_t s)
+{
+    WL_CUDA_TRY(launch_chained(k_hop_fix_norm<false>, (unsigned)((a.g.Vh + 63) / 64 * a.nrhs), 128, s, a, e, norms,
+                               partials, tickets));
+    return WL_OK;
+}
+
 template <int KIND>
 static void reduce_kind(int dagger, const HopArgs &a, const void *epi, cudaStream_t s)
 {

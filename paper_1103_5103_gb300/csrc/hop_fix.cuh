@@ -378,6 +378,29 @@ __device__ __forceinline__ void half_store(void *base, int stride, int s, int i,
     }
 }
 
+// o = a1 x1 + a2 x2 + coef acc, stored, as EpiStore on the other hops.
+__device__ __forceinline__ void half_epilogue(const EpiStore &e, int stride, int r, int s, int i,
+                                              const cx<double> (&acc)[6], cx<double> (&o)[6])
+{
+    const size_t off = (size_t)r * e.rhs_bytes;
+    if (e.out_raw) half_store(static_cast<char *>(e.out_raw) + off, stride, s, i, acc);
+#pragma unroll
+    for (int k = 0; k < 6; ++k) o[k] = e.coef * acc[k];
+    if (e.x1) {
+        cx<double> x[6];
+        half_load(static_cast<const char *>(e.x1) + off, stride, s, i, x);
+#pragma unroll
+        for (int k = 0; k < 6; ++k) o[k] = o[k] + e.a1 * x[k];
+    }
+    if (e.x2) {
+        cx<double> x[6];
+        half_load(static_cast<const char *>(e.x2) + off, stride, s, i, x);
+#pragma unroll
+        for (int k = 0; k < 6; ++k) o[k] = o[k] + e.a2 * x[k];
+    }
+    half_store(static_cast<char *>(e.out) + off, stride, s, i, o);
+}
+
 // out = a1 x1 + a2 x2 + coef D in, as EpiStore on the other hops, for task
 // `task`: 16 sites of one rhs.  The rhs of the same sites are consecutive
 // tasks, taken by neighbouring warps, which share the links through L1.
@@ -390,27 +413,9 @@ __device__ __forceinline__ void hop_fix_task(const HopArgs &a, const EpiStore &e
     if (i0 - (lane & 15) >= a.g.Vh || rhs_done(a, r)) return;   // the whole warp
     const bool active = i0 < a.g.Vh;
     const int i = active ? i0 : a.g.Vh - 1;
-    cx<double> acc[6];
+    cx<double> acc[6], o[6];
     hop_half<DAG, false>(a, static_cast<const char *>(a.in) + (size_t)r * a.rhs_bytes, i, s, acc);
-    if (!active) return;
-    const size_t off = (size_t)r * e.rhs_bytes;
-    if (e.out_raw) half_store(static_cast<char *>(e.out_raw) + off, a.g.stride, s, i, acc);
-    cx<double> o[6];
-#pragma unroll
-    for (int k = 0; k < 6; ++k) o[k] = e.coef * acc[k];
-    if (e.x1) {
-        cx<double> x[6];
-        half_load(static_cast<const char *>(e.x1) + off, a.g.stride, s, i, x);
-#pragma unroll
-        for (int k = 0; k < 6; ++k) o[k] = o[k] + e.a1 * x[k];
-    }
-    if (e.x2) {
-        cx<double> x[6];
-        half_load(static_cast<const char *>(e.x2) + off, a.g.stride, s, i, x);
-#pragma unroll
-        for (int k = 0; k < 6; ++k) o[k] = o[k] + e.a2 * x[k];
-    }
-    half_store(static_cast<char *>(e.out) + off, a.g.stride, s, i, o);
+    if (active) half_epilogue(e, a.g.stride, r, s, i, acc, o);
 }
 
 inline __host__ __device__ unsigned fix_tasks(const HopArgs &a)
@@ -442,6 +447,35 @@ void launch_k_hop_fix(const HopArgs &a, const EpiStore &e, int blocks_per_sm, cu
 {
     if (blocks_per_sm > 0) launch_chained(k_hop_fix_gs<DAG>, blocks_per_sm * sm_count(), 128, s, a, e);
     else launch_chained(k_hop_fix<DAG>, (fix_tasks(a) + 3) / 4, 128, s, a, e);
+}
+
+// The same with ||out_r||^2 into norms[r] for the rhs that are not skipped:
+// the residual hop of an outer check and its norm in one pass (the norm's own
+// pass reads the residual again: 294 us of 3.2 ms, 12 rhs on 24^3x64).  Blocks of
+// 64 sites of one rhs.
+template <bool DAG>
+__global__ void __launch_bounds__(128, 4) k_hop_fix_norm(HopArgs a, EpiStore e, double *norms, double *partials,
+                                                         unsigned *tickets)
+{
+    const int z = chain_begin();
+    const int r = blockIdx.x % a.nrhs + z, sb = blockIdx.x / a.nrhs + z;
+    if (rhs_done(a, r)) return;   // uniform over every block of this rhs
+    const int lane = threadIdx.x & 31, s = lane >> 4;
+    const int i0 = sb * 64 + (threadIdx.x >> 5) * 16 + (lane & 15);
+    double red[1] = {0.0};
+    if (i0 - (lane & 15) < a.g.Vh) {   // the whole warp
+        const int i = min(i0, a.g.Vh - 1);
+        cx<double> acc[6], o[6];
+        hop_half<DAG, false>(a, static_cast<const char *>(a.in) + (size_t)r * a.rhs_bytes, i, s, acc);
+        if (i0 < a.g.Vh) {
+            half_epilogue(e, a.g.stride, r, s, i, acc, o);
+#pragma unroll
+            for (int k = 0; k < 6; ++k) red[0] = fma(o[k].re, o[k].re, fma(o[k].im, o[k].im, red[0]));
+        }
+    }
+    double tot[1];
+    if (site_sum<1>(red, a.g, partials, r, &tickets[r], sb, gridDim.x / a.nrhs, tot) && threadIdx.x == 0)
+        norms[r] = tot[0];
 }
 
 // The reduction-fused hop (EpiReduce): blocks of 64 sites of one rhs.

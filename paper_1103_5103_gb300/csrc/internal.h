@@ -112,10 +112,17 @@ int export_full(const Geom &g, const Vec &even, const Vec &odd, void *const *can
 // ---- dslash.cu
 // out[r] = a1 * x1[r] + a2 * x2[r] + coef * D_{p,1-p} in[r] for r < nrhs (x1, x2
 // optional).  rhs_block = rhs per thread (1, 2 or 4).  skip (optional, device)
-// skips rhs r when skip[r * skip_stride] != 0.
+// skips rhs r when skip[r * skip_stride] != 0.  norm (optional) also receives
+// ||out_r||^2, in the same launch for the fixed-point FP64 hop (skipped rhs
+// then keep their entries).
+struct NormOut {
+    double *norms;       // [nrhs], device
+    double *partials;    // red_buffer
+    unsigned *tickets;   // [nrhs]
+};
 int hop_ex(wl_gauge *g, const Vec &in, const Vec &out, const Vec *x1, double a1, const Vec *x2, double a2,
            double coef, int out_parity, int dagger, int rhs_block, const int *skip, int skip_stride, cudaStream_t s,
-           const Vec *out_raw = nullptr);
+           const Vec *out_raw = nullptr, const NormOut *norm = nullptr);
 int hop(wl_gauge *g, const Vec &in, const Vec &out, const Vec *x, double coef, int out_parity, int dagger,
         int rhs_block, cudaStream_t s);
 
@@ -170,8 +177,9 @@ int canon_dots(const void *const *a, const void *const *in, int n, int nrhs, siz
                double *partials, unsigned *tickets, cudaStream_t s);
 int blas_convert(const Geom &g, const Vec &in, const Vec &out, cudaStream_t s);
 int blas_xpay(const Geom &g, const Vec &x, double a, const Vec &y, const Vec &out, cudaStream_t s);  // out = x + a y
-// x_o = b_o + kappa Dx and ||b_o - x_o + kappa Dx||^2 per rhs into norm2_dev
-int blas_recon(const Geom &g, const Vec &bo, const Vec &dx, double kappa, const Vec &xo, double *norm2_dev,
+// x_o = b_o + kappa Dx and ||b_o - x_o + kappa Dx||^2 per rhs into norm2_dev;
+// bo null: b_o = 0
+int blas_recon(const Geom &g, const Vec *bo, const Vec &dx, double kappa, const Vec &xo, double *norm2_dev,
                double *partials, unsigned *tickets, cudaStream_t s);
 
 

@@ -387,6 +387,10 @@ static int eo_defect_correction(wl_gauge *g, const Vec &bprec, const Vec &x64, d
     Vec r64, tmp64;  // outer precision (FP64 or double-float)
     WL_TRY(make_vec(g, "dc_r64", x64.prec, nrhs, &r64));
     WL_TRY(make_vec(g, "dc_tmp64", x64.prec, nrhs, &tmp64));
+    // ||r||^2 per rhs, in an array of its own: those of finished rhs stay
+    void *pnorm = nullptr;
+    WL_TRY(g->ws.get("dc_norms", sizeof(double) * nrhs, &pnorm));
+    const NormOut norm{static_cast<double *>(pnorm), in.sc.partials, in.sc.tickets};
     void *pin = nullptr;
     WL_TRY(g->pinned.get("dc_scalars", nrhs * (sizeof(double) * 2 + sizeof(int) * 2), &pin));
     double *h_rn2 = static_cast<double *>(pin);
@@ -458,10 +462,11 @@ static int eo_defect_correction(wl_gauge *g, const Vec &bprec, const Vec &x64, d
             WL_TRY(hop_ex(g, x64, tmp64, nullptr, 0.0, nullptr, 0.0, 1.0, WL_ODD, 0, ohop, in.sc.outer_done, 1, s));
             if (ev.e[1]) WL_CUDA_TRY(cudaEventRecord(ev.e[1], s));
             WL_TRY(hop_ex(g, tmp64, r64, &bprec, 1.0, &x64, -1.0, k2, WL_EVEN, 0, ohop, in.sc.outer_done, 1, s,
-                          y_out));
+                          y_out, &norm));
+        } else {
+            WL_TRY(blas_norm2(geo, r64, norm.norms, norm.partials, norm.tickets, s));
         }
-        WL_TRY(blas_norm2(geo, r64, in.sc.norms, in.sc.partials, in.sc.tickets, s));
-        WL_CUDA_TRY(cudaMemcpyAsync(h_rn2, in.sc.norms, sizeof(double) * nrhs, cudaMemcpyDeviceToHost, s));
+        WL_CUDA_TRY(cudaMemcpyAsync(h_rn2, norm.norms, sizeof(double) * nrhs, cudaMemcpyDeviceToHost, s));
         WL_CUDA_TRY(cudaStreamSynchronize(s));
         if (ev.e[0] && n_hop > 0) {
             float ms = 0.f;
@@ -723,7 +728,8 @@ struct AsyncExport {
 static int solve_one_mass(wl_gauge *g, const Vec &be, const Vec &bo, const Vec &bprec, const Vec &xe, double m0,
                           const wl_solver_params &prm, const std::vector<double> &bnorm2, void *const *x_out,
                           int x_out_stride, std::vector<wl_solver_stats> &stats, cudaStream_t s,
-                          const Vec *y_out = nullptr, bool r0_given = false, AsyncExport *ax = nullptr)
+                          const Vec *y_out = nullptr, bool r0_given = false, AsyncExport *ax = nullptr,
+                          bool odd_zero = false)
 {
     const Geom &geo = g->lat->geom;
     const int nrhs = be.nrhs;
@@ -742,7 +748,7 @@ static int solve_one_mass(wl_gauge *g, const Vec &be, const Vec &bo, const Vec &
     Scratch sc;
     WL_TRY(get_scratch(g, nrhs, &sc, s));
     if (ax && ax->pending[slot]) WL_CUDA_TRY(cudaStreamWaitEvent(s, ax->done[slot], 0));
-    WL_TRY(blas_recon(geo, bo, dx, kappa, xo, sc.norms, sc.partials, sc.tickets, s));
+    WL_TRY(blas_recon(geo, odd_zero ? nullptr : &bo, dx, kappa, xo, sc.norms, sc.partials, sc.tickets, s));
     std::vector<double> ro2(nrhs);
     WL_CUDA_TRY(cudaMemcpyAsync(ro2.data(), sc.norms, sizeof(double) * nrhs, cudaMemcpyDeviceToHost, s));
     WL_CUDA_TRY(cudaStreamSynchronize(s));
@@ -1027,8 +1033,6 @@ extern "C" int multimass_solve(wl_gauge *g, const void *const *b, void *const *x
     Vec be, bo, dbo, bprec;
     WL_TRY(make_vec(g, "b_e", PO, n_rhs, &be));
     WL_TRY(make_vec(g, "b_o", PO, n_rhs, &bo));
-    WL_TRY(make_vec(g, "mm_Dbo", PO, n_rhs, &dbo));
-    WL_TRY(make_vec(g, "mm_bprec", PO, n_rhs, &bprec));
     WL_TRY(import_full(geo, b, be, bo, s));
     Scratch sc;
     WL_TRY(get_scratch(g, n_rhs, &sc, s));
@@ -1039,8 +1043,15 @@ extern "C" int multimass_solve(wl_gauge *g, const void *const *b, void *const *x
     // D_eo b_o once for all masses; b_prec(m) = b_e + kappa(m) D_eo b_o.  A
     // source without an odd part (a point source on an even site) needs no
     // hop: its D_eo b_o is zero.  ||b_o||^2 is exactly zero only if every odd
-    // entry is below 2.2e-162, whose hop would be as negligible.
-    {
+    // entry is below 2.2e-162, whose hop would be as negligible.  If no source
+    // of the call has one, b_prec is b_e for every mass.
+    bool odd_zero = true;
+    for (int r = 0; r < n_rhs; ++r) odd_zero &= no[r] == 0.0;
+    if (odd_zero) {
+        bprec = be;
+    } else {
+        WL_TRY(make_vec(g, "mm_Dbo", PO, n_rhs, &dbo));
+        WL_TRY(make_vec(g, "mm_bprec", PO, n_rhs, &bprec));
         void *pp = nullptr;
         WL_TRY(g->pinned.get("mm_skip", sizeof(int) * n_rhs, &pp));
         int *h_zero = static_cast<int *>(pp);
@@ -1116,7 +1127,7 @@ extern "C" int multimass_solve(wl_gauge *g, const void *const *b, void *const *x
         const int slot = k % ring;
         WL_TRY(make_vec(g, "mm_sol" + std::to_string(slot), PO, n_rhs, &sol[k]));
         WL_TRY(make_vec(g, "mm_y" + std::to_string(slot), PO, n_rhs, &ys[k]));
-        WL_TRY(blas_xpay(geo, be, 1.0 / (2.0 * m + 8.0), dbo, bprec, s));
+        if (!odd_zero) WL_TRY(blas_xpay(geo, be, 1.0 / (2.0 * m + 8.0), dbo, bprec, s));
         Vec r0;
         WL_TRY(make_vec(g, "dc_r64", PO, n_rhs, &r0));
         const double k2 = 1.0 / ((2.0 * m + 8.0) * (2.0 * m + 8.0));
@@ -1177,7 +1188,8 @@ extern "C" int multimass_solve(wl_gauge *g, const void *const *b, void *const *x
         for (int r = 0; r < n_rhs; ++r) std::memset(&st[r], 0, sizeof(wl_solver_stats));
         // nothing overlaps the last mass's export: give it the whole GPU
         if (axp && k == n_mass - 1) ax.blocks = ax.full_blocks;
-        WL_TRY(solve_one_mass(g, be, bo, bprec, sol[k], m, *p, bn2, x + im, n_mass, st, s, &ys[k], true, axp));
+        WL_TRY(solve_one_mass(g, be, bo, bprec, sol[k], m, *p, bn2, x + im, n_mass, st, s, &ys[k], true, axp,
+                              odd_zero));
         if (p->guess == WL_GUESS_SSM && k + 1 < n_mass) {
             // the Gram products read the canonical solutions: wait for their export
             WL_TRY(ax.join(s));
