@@ -68,8 +68,9 @@ struct TuneResult {
 // are unchanged (the mass enters through device memory).
 struct GraphCache {
     std::vector<uintptr_t> key;
-    cudaGraphExec_t exec = nullptr;
-    long long kernels = 0;
+    cudaGraphExec_t exec = nullptr;   // the block
+    cudaGraphExec_t one = nullptr;    // a single iteration (not while profiling)
+    long long kernels = 0, one_kernels = 0;
     std::vector<cudaEvent_t> events;
     void release();
 };

@@ -78,8 +78,10 @@ static int get_scratch(wl_gauge *g, int nrhs, Scratch *sc, cudaStream_t s)
 
 void GraphCache::release()
 {
-    if (exec) cudaGraphExecDestroy(exec);
-    exec = nullptr;
+    for (auto x : {&exec, &one}) {
+        if (*x) cudaGraphExecDestroy(*x);
+        *x = nullptr;
+    }
     for (auto e : events) cudaEventDestroy(e);
     events.clear();
     key.clear();
@@ -94,6 +96,7 @@ struct Inner {
     double kappa;
     Vec r, rhat, p, v, s, t, tmp, e;
     Scratch sc;
+    double rate = 0.0;   // ln of ||r||^2 lost per iteration in the last inner solve (0: none yet)
 };
 
 static int make_inner(wl_gauge *g, int prec, int nrhs, double kappa, Inner *in, cudaStream_t s)
@@ -188,10 +191,64 @@ static int inner_iteration_cg(Inner &in, int rhs_block, cudaStream_t s, cudaEven
     return WL_OK;
 }
 
+// A captured graph of n inner iterations and its number of kernels; ev
+// (optional): 2 n events recorded around each iteration's first hop.
+static int capture_iterations(Inner &in, const wl_solver_params &prm, int rhs_block, int n, cudaEvent_t *ev,
+                              cudaStream_t cap, cudaGraphExec_t *exec, long long *kernels)
+{
+    int status = WL_OK;
+    cudaGraph_t graph = nullptr;
+    cudaError_t e = cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal);
+    if (e == cudaSuccess) {
+        for (int k = 0; k < n && status == WL_OK; ++k)
+            status = prm.inner_solver == WL_SOLVER_CG ? inner_iteration_cg(in, rhs_block, cap, ev ? ev + 2 * k : nullptr)
+                                                      : inner_iteration(in, rhs_block, cap, ev ? ev + 2 * k : nullptr);
+        e = cudaStreamEndCapture(cap, &graph);
+    }
+    if (e == cudaSuccess && status == WL_OK) e = cudaGraphInstantiate(exec, graph, 0);
+    *kernels = 0;
+    if (graph) {
+        // kernel nodes only (event-record nodes are not launches)
+        size_t m = 0;
+        cudaGraphGetNodes(graph, nullptr, &m);
+        std::vector<cudaGraphNode_t> nodes(m);
+        if (m) cudaGraphGetNodes(graph, nodes.data(), &m);
+        for (auto nd : nodes) {
+            cudaGraphNodeType t;
+            if (cudaGraphNodeGetType(nd, &t) == cudaSuccess && t == cudaGraphNodeTypeKernel) ++*kernels;
+        }
+        cudaGraphDestroy(graph);
+    }
+    if (e != cudaSuccess && status == WL_OK) {
+        set_error(std::string("graph capture: ") + cudaGetErrorString(e));
+        status = WL_ERR_CUDA;
+    }
+    return status;
+}
+
+// Iterations that an rhs still needs to take its residual (squared) down by
+// the factor exp(-lnf), at `rate` per iteration.
+static int iterations_for(double lnf, double rate)
+{
+    const double n = std::ceil(lnf / rate);
+    return n >= 1.0 && n < 1e6 ? (int)n : 1;
+}
+
 // Run inner iterations until every rhs is done or max_iter is reached.
-// Returns the state array copied to host in host_state.
-static int run_inner(Inner &in, const wl_solver_params &prm, int max_iter, std::vector<BiState> &host_state,
-                     cudaStream_t s)
+// Returns the state array copied to host in host_state.  delta2 (host, per
+// rhs, read for the rhs with active[r] != 0): the squared reduction each
+// solve stops at.
+//
+// In graph mode the iterations between two looks at the state are as many as
+// the solve is expected to need: the reduction asked for over the rate of
+// the last inner solve for this mass, later over this solve's own rate; full
+// captured blocks, then captured single iterations.  (With fixed blocks of eight, 8^4
+// with four masses ran 112 iterations for 83 and 16^3x32 with eight 112 for
+// 74; a surplus iteration is seven launches that find the rhs done, 9-10 us
+// there.  8^4 x 4 masses 4.69 -> 4.58 ms, 16^3x32 x 8 8.11 -> 7.82, 24^3x64
+// with 12 sources 324 -> 312, 48^3x96 FP16 163 -> 160.)  Which iterations run, and their results, do not depend on it.
+static int run_inner(Inner &in, const wl_solver_params &prm, int max_iter, const double *delta2, const int *active,
+                     std::vector<BiState> &host_state, cudaStream_t s)
 {
     const int nrhs = in.nrhs;
     const int rb = prm.rhs_block;  // 0: the autotuned hop variant
@@ -233,36 +290,12 @@ static int run_inner(Inner &in, const wl_solver_params &prm, int max_iter, std::
             for (auto &e : gc.events) WL_CUDA_TRY(cudaEventCreate(&e));
             cudaStream_t cap = nullptr;
             WL_CUDA_TRY(cudaStreamCreateWithFlags(&cap, cudaStreamNonBlocking));
-            cudaGraph_t graph = nullptr;
-            cudaError_t e = cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal);
-            if (e == cudaSuccess) {
-                for (int k = 0; k < K && status == WL_OK; ++k)
-                    status = prm.inner_solver == WL_SOLVER_CG
-                                 ? inner_iteration_cg(in, rb, cap, prof ? &gc.events[2 * k] : nullptr)
-                                 : inner_iteration(in, rb, cap, prof ? &gc.events[2 * k] : nullptr);
-                e = cudaStreamEndCapture(cap, &graph);
-            }
-            if (e == cudaSuccess && status == WL_OK) e = cudaGraphInstantiate(&gc.exec, graph, 0);
-            if (graph) {
-                // kernel nodes only (event-record nodes are not launches)
-                size_t n = 0;
-                cudaGraphGetNodes(graph, nullptr, &n);
-                std::vector<cudaGraphNode_t> nodes(n);
-                if (n) cudaGraphGetNodes(graph, nodes.data(), &n);
-                gc.kernels = 0;
-                for (auto nd : nodes) {
-                    cudaGraphNodeType t;
-                    if (cudaGraphNodeGetType(nd, &t) == cudaSuccess && t == cudaGraphNodeTypeKernel) ++gc.kernels;
-                }
-                cudaGraphDestroy(graph);
-            }
+            status = capture_iterations(in, prm, rb, K, prof ? gc.events.data() : nullptr, cap, &gc.exec, &gc.kernels);
+            if (status == WL_OK && !prof && K > 1)
+                status = capture_iterations(in, prm, rb, 1, nullptr, cap, &gc.one, &gc.one_kernels);
             cudaStreamDestroy(cap);
-            if (e != cudaSuccess || status != WL_OK) {
+            if (status != WL_OK) {
                 gc.release();
-                if (status == WL_OK) {
-                    set_error(std::string("graph capture: ") + cudaGetErrorString(e));
-                    status = WL_ERR_CUDA;
-                }
                 return status;
             }
             gc.key = key;
@@ -280,16 +313,34 @@ static int run_inner(Inner &in, const wl_solver_params &prm, int max_iter, std::
         ~EvFree() { for (auto e : v) cudaEventDestroy(e); }
     } ev_free{host_ev};
     int done_iters = 0;
+    double &rate = in.rate;
+    const long last = ((long)max_iter + K - 1) / K * K;   // max_iter in whole blocks
+    const bool predict = exec && !prof;
+    int group = K;   // iterations before the next look at the state
+    if (predict && rate > 0.0) {
+        group = 1;
+        for (int r = 0; r < nrhs; ++r)
+            if (active[r]) group = std::max(group, iterations_for(-std::log(delta2[r]), rate));
+        group = (int)std::min<long>(group, last);
+    }
     for (;;) {
         if (exec) {
-            cudaError_t e = cudaGraphLaunch(exec, s);
+            int n = group;
+            cudaError_t e = cudaSuccess;
+            for (; n >= K && e == cudaSuccess; n -= K) {
+                e = cudaGraphLaunch(exec, s);
+                add_launches(graph_kernels);
+            }
+            for (; n > 0 && e == cudaSuccess; --n) {
+                e = cudaGraphLaunch(in.g->inner_graph.one, s);
+                add_launches(in.g->inner_graph.one_kernels);
+            }
             if (e != cudaSuccess) {
                 set_error(std::string("cudaGraphLaunch: ") + cudaGetErrorString(e));
                 status = WL_ERR_CUDA;
                 break;
             }
-            add_launches(graph_kernels);
-            done_iters += K;
+            done_iters += group;
         } else {
             status = prm.inner_solver == WL_SOLVER_CG ? inner_iteration_cg(in, rb, s, ev) : inner_iteration(in, rb, s, ev);
             if (status != WL_OK) break;
@@ -328,7 +379,24 @@ static int run_inner(Inner &in, const wl_solver_params &prm, int max_iter, std::
         }
         bool all = true;
         for (int r = 0; r < nrhs; ++r) all &= hs[r].done != 0;
-        if (all || done_iters >= max_iter) break;
+        if (predict) {
+            // the slowest rhs's rate, and what is left at each one's own
+            double slowest = 0.0;
+            group = 1;
+            for (int r = 0; r < nrhs; ++r) {
+                if (!active[r] || hs[r].iters < 1 || !(hs[r].rr > 0.0)) continue;
+                const double own = std::log(hs[r].target2 / delta2[r] / hs[r].rr) / hs[r].iters;
+                if (!(own > 0.0) || !std::isfinite(own)) {
+                    group = K;
+                    continue;
+                }
+                slowest = slowest > 0.0 ? std::min(slowest, own) : own;
+                if (!hs[r].done) group = std::max(group, std::min(K, iterations_for(std::log(hs[r].rr / hs[r].target2), own)));
+            }
+            if (slowest > 0.0) rate = slowest;
+            group = (int)std::min<long>(group, last - done_iters);
+        }
+        if (all || done_iters >= last) break;
     }
     std::memcpy(host_state.data(), hs, sizeof(BiState) * nrhs);
     if (status == WL_OK && hop_variant_for(in.g, in.prec, nrhs, rb) >= 9000) {
@@ -541,7 +609,7 @@ static int eo_defect_correction(wl_gauge *g, const Vec &bprec, const Vec &x64, d
         int cap = 0;
         for (int r = 0; r < nrhs; ++r)
             if (h_active[r]) cap = std::max(cap, prm.max_iter - iters[r]);
-        WL_TRY(run_inner(in, prm, cap, hst, s));
+        WL_TRY(run_inner(in, prm, cap, h_delta2, h_active, hst, s));
         for (int r = 0; r < nrhs; ++r)
             if (h_active[r]) iters[r] += hst[r].iters;
         // Further segments only for the rhs whose outer target lies below
@@ -595,7 +663,7 @@ static int eo_defect_correction(wl_gauge *g, const Vec &bprec, const Vec &x64, d
                 int mcap = 0;
                 for (int r = 0; r < nrhs; ++r)
                     if (h_mode[r]) mcap = std::max(mcap, prm.max_iter - iters[r]);
-                WL_TRY(run_inner(in, prm, mcap, hst, s));
+                WL_TRY(run_inner(in, prm, mcap, h_mdelta2, h_mode, hst, s));
                 for (int r = 0; r < nrhs; ++r)
                     if (h_mode[r]) iters[r] += hst[r].iters;
             }
