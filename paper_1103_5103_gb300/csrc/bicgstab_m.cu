@@ -26,6 +26,7 @@
 #include <string>
 #include <vector>
 
+#include "hop_fix.cuh"
 #include "internal.h"
 
 namespace wl {
@@ -201,20 +202,170 @@ __global__ void __launch_bounds__(kBlock) k_m_s(Geom g, int nsb, Vec r, Vec v, V
     for (int c = 0; c < 12; ++c) C::st(s.rhs(h), str, c, i, C::ld(r.rhs(h), str, c, i) - al * C::ld(v.rhs(h), str, c, i));
 }
 
+// The FP64 shift updates in fixed point.  Six complex products per component
+// and shift are 24 FP64 multiply-adds, and at 1.7 per clock and SM the update
+// was bound by the FP64 pipe and more than half of a multi-shift solve; as
+// 64-bit integers they are 72 multiply-adds at 53-62 per clock.  Each complex
+// number has its own scale:
+//  - a component with largest biased exponent e is an integer in units of
+//    2^(e-1081), below 2^59 (fix_conv: kFixFrac = 58); a coefficient one in
+//    units of 2^(e-1084), below 2^62;
+//  - their product (hi*hi and the two cross terms of balanced 32-bit limbs,
+//    as in the FP64 hop) has scale S = e + e', units of 2^(S-2101), and is
+//    below 2^58 (complex: below 2^59 with the second term).  A component
+//    with exponent e is the same integer at scale e + 1020;
+//  - a sum is formed at the largest scale of its terms, whose rounding unit
+//    is 2^-55 of the term that sets it where FP64's is 2^-53, and is rounded
+//    to FP64 once, at the store.  Error against exact arithmetic (random
+//    complex values, relative l2): x^s 4.8-6.9e-17, FP64 products 7.4-9.6e-17;
+//    q^s 4.8-5.3e-17 and 6.7-10.2e-17, for residuals of 1 to 1e-10 of x and
+//    for exponents that differ by up to 300.
+// A component outside 2^(-423..478), or a coefficient outside 2^(-200..201)
+// (zeros are inside), takes the FP64 products.
+//
+// 16^3x32, seven shifts: the multi-shift solve 30.2 -> 23.2 ms.  Bound by
+// instruction latency and the ALU pipe (49% busy at 15.6 warps per SM, issue
+// 48%, DRAM 32%): most of the instructions convert, align and round.
+// Measured on the solve: without the prefetch 25.0, 4 to 7 blocks per SM and
+// FP64 operands reloaded instead of kept all within 2%, one thread for all 12
+// components 23.8.
+constexpr int kShiftMinExp = 600, kShiftMaxExp = 1500;
+constexpr int kShiftCoefMin = 823, kShiftCoefMax = 1223;
+constexpr int kShiftUnit = 1020;   // scale of a component: exponent + this
+
+struct FixShift {
+    int4 u[6];   // cxp, cxs, cqr, cqs, cpr, bs as limbs re.lo, re.hi, im.lo, im.hi
+    int e[6];
+    int fp;      // a coefficient outside the range
+};
+
+// Largest biased exponent of v, zero as the smallest one; special: outside the range.
+__device__ __forceinline__ int shift_exp(cx<double> v, int lo, int hi, bool &special)
+{
+    const int A = fix_absmax(0, make_double2(v.re, v.im)), e = A >> 20;
+    special = special || e > hi || (e < lo && (A | fix_lobits(make_double2(v.re, v.im))) != 0);
+    return max(e, lo);
+}
+__device__ __forceinline__ i64 shift_conv(double x, int e)
+{
+    int neg = 0;
+    const i64 q = fix_conv(x, e, 0, neg);
+    return q - neg;
+}
+
+__device__ __forceinline__ void shift_coef(FixShift &q, int j, cx<double> v)
+{
+    bool special = false;
+    const int e = shift_exp(v, kShiftCoefMin, kShiftCoefMax, special);
+    const i64 re = shift_conv(v.re, e) << 3, im = shift_conv(v.im, e) << 3;
+    q.u[j] = make_int4((int)re, fix_hi(re), (int)im, fix_hi(im));
+    q.e[j] = e;
+    if (special) q.fp = 1;
+}
+
+// A component as limbs of re, im and -im, with its exponent.
+struct FixComp {
+    int rh, rl, ih, il, nh, nl, e;
+    __device__ __forceinline__ void set(i64 re, i64 im, int exp)
+    {
+        rl = (int)re;
+        rh = fix_hi(re);
+        il = (int)im;
+        ih = fix_hi(im);
+        nl = (int)-im;
+        nh = fix_hi(-im);
+        e = exp;
+    }
+};
+
+struct FixSum {
+    i64 re, im;
+};
+// coefficient times component, moved down by sh: rounded down, or with NEAREST
+// (x^s, which adds up all iterations) to nearest, so that no drift builds up
+template <bool NEAREST = false>
+__device__ __forceinline__ FixSum shift_mul(const int4 u, const FixComp &x, int sh)
+{
+    i64 h0 = (i64)u.y * x.rh, h1 = (i64)u.y * x.ih, x0 = 1ll << 31, x1 = 1ll << 31;
+    x0 += (i64)u.y * x.rl;
+    x0 += (i64)u.x * x.rh;
+    x1 += (i64)u.y * x.il;
+    x1 += (i64)u.x * x.ih;
+    h0 += (i64)u.w * x.nh;
+    x0 += (i64)u.w * x.nl;
+    x0 += (i64)u.z * x.nh;
+    h1 += (i64)u.w * x.rh;
+    x1 += (i64)u.w * x.rl;
+    x1 += (i64)u.z * x.rh;
+    const i64 half = NEAREST ? (1ll << min(sh, 62)) >> 1 : 0;
+    return {fix_sar(h0 + (x0 >> 32) + half, sh), fix_sar(h1 + (x1 >> 32) + half, sh)};
+}
+
+// v 2^(S-2101), rounded to FP64 (|v| < 2^62; never subnormal within the ranges).
+__device__ __forceinline__ double shift_out(i64 v, int S)
+{
+    const i64 m = v >> 63;
+    const u64 a = (u64)((v ^ m) - m);
+    const int n = __clzll((i64)a) - 1;
+    const u64 mant = ((a << n) + (1ull << 9)) >> 10;
+    const u64 bits = mant + ((u64)(unsigned)(S - kShiftUnit + 3 - n) << 52);
+    return a ? __longlong_as_double((i64)(bits | ((u64)m & (1ull << 63)))) : 0.0;
+}
+
+// x^s and q^s of one component: p^s = cpr r + beta^s q^s, then x^s += cxp p^s
+// + cxs s and q^s = p^s + cqr r + cqs s.  rs_special: r or s outside the range.
+__device__ __forceinline__ void shift_update(const FixShift &q, const cx<double> *c, const FixComp &r, const FixComp &s,
+                                             bool rs_special, cx<double> rc, cx<double> sc, cx<double> &x, cx<double> &p)
+{
+    bool special = rs_special || q.fp;
+    const int ex = shift_exp(x, kShiftMinExp, kShiftMaxExp, special);
+    const int ep = shift_exp(p, kShiftMinExp, kShiftMaxExp, special);
+    if (special) {
+        const cx<double> pc = cmad(c[4], rc, c[5] * p);
+        x = cmad(c[0], pc, cmad(c[1], sc, x));
+        p = cmad(c[2], rc, cmad(c[3], sc, pc));
+        return;
+    }
+    // p^s, at the larger of its terms' scales
+    const int S4 = r.e + q.e[4], Sp = max(S4, ep + q.e[5]);
+    FixComp t;
+    t.set(shift_conv(p.re, Sp - q.e[5]), shift_conv(p.im, Sp - q.e[5]), 0);
+    const FixSum a = shift_mul(q.u[4], r, Sp - S4), b = shift_mul(q.u[5], t, 0);
+    const i64 pre = a.re + b.re, pim = a.im + b.im;
+    t.set(pre, pim, Sp - kShiftUnit);
+    // x^s
+    const int S0 = t.e + q.e[0], S1 = s.e + q.e[1], Sx = max(max(S0, S1), ex + kShiftUnit);
+    const FixSum d = shift_mul<true>(q.u[0], t, Sx - S0), f = shift_mul<true>(q.u[1], s, Sx - S1);
+    x.re = shift_out(shift_conv(x.re, Sx - kShiftUnit) + d.re + f.re, Sx);
+    x.im = shift_out(shift_conv(x.im, Sx - kShiftUnit) + d.im + f.im, Sx);
+    // q^s
+    const int S2 = r.e + q.e[2], S3 = s.e + q.e[3], Sq = max(max(S2, S3), Sp);
+    const FixSum g = shift_mul(q.u[2], r, Sq - S2), h = shift_mul(q.u[3], s, Sq - S3);
+    p.re = shift_out(fix_sar(pre, Sq - Sp) + g.re + h.re, Sq);
+    p.im = shift_out(fix_sar(pim, Sq - Sp) + g.im + h.im, Sq);
+}
+
+// Sites of a k_m_update block: in FP64, two threads take a site's components
+// (twice the blocks: 1024 blocks of 16^3x32 are 1.35 waves).
+constexpr int update_sites(int P) { return P == WL_F64 ? kBlock / 2 : kBlock; }
+
 // Shift updates, p^s = cpr r + beta^s q^s (previous iteration's
 // coefficients; cpr = 1, beta^s = 0 at the start), then x^s and q^s;
 // unshifted x += alpha p + omega s, r = s - omega t with <rhat, r> and
 // ||r||^2 -> beta (last block).
 template <int P>
-__global__ void __launch_bounds__(kBlock) k_m_update(Geom g, int nsb, Vec x, Vec p, Vec s, Vec t, Vec r, Vec rhat,
-                                                     ShiftVecs sv, const ShiftState *sh, int ns, BiState *st,
-                                                     double *partials)
+__global__ void __launch_bounds__(kBlock, P == WL_F64 ? 5 : 8)
+k_m_update(Geom g, int nsb, Vec x, Vec p, Vec s, Vec t, Vec r, Vec rhat, ShiftVecs sv, const ShiftState *sh, int ns,
+           BiState *st, double *partials)
 {
     using C = CompIO<P>;
     using R = typename PrecTraits<P>::R;
     static_assert(sizeof(cx<R>) == 16, "coefficient staging assumes 16-byte complex scalars");
     st += chain_begin();
-    const FullIdx f = full_idx(nsb);
+    constexpr int kSites = update_sites(P), kComps = 12 * kSites / kBlock;
+    FullIdx f = full_idx(nsb);
+    f.i = f.sb * kSites + threadIdx.x % kSites;
+    const int c0 = threadIdx.x / kSites * kComps;
     BiState &S = *st;
     if (__ldcg(&S.done)) return;
     // the active shifts and their six coefficients, staged once per block
@@ -222,6 +373,7 @@ __global__ void __launch_bounds__(kBlock) k_m_update(Geom g, int nsb, Vec x, Vec
     __shared__ int sact[32];
     __shared__ int snact;
     cx<R> *sc = reinterpret_cast<cx<R> *>(sraw);
+    __shared__ FixShift sfix[P == WL_F64 ? 32 : 1];
     if (threadIdx.x < ns) {
         const ShiftState &Q = sh[threadIdx.x];
         cx<R> *q = sc + 6 * threadIdx.x;
@@ -231,6 +383,12 @@ __global__ void __launch_bounds__(kBlock) k_m_update(Geom g, int nsb, Vec x, Vec
         q[3] = cs<R>(Q.cqs_re, Q.cqs_im);
         q[4] = cs<R>(Q.cpr_re, Q.cpr_im);
         q[5] = cs<R>(Q.bs_re, Q.bs_im);
+        if constexpr (P == WL_F64) {
+            FixShift &F = sfix[threadIdx.x];
+            F.fp = 0;
+#pragma unroll
+            for (int j = 0; j < 6; ++j) shift_coef(F, j, q[j]);
+        }
     }
     if (threadIdx.x == 0) {
         int n = 0;
@@ -246,18 +404,51 @@ __global__ void __launch_bounds__(kBlock) k_m_update(Geom g, int nsb, Vec x, Vec
         const cx<R> om = cs<R>(__ldcg(&S.omega_re), __ldcg(&S.omega_im));
         cx<R> d = {R(0), R(0)};
         R n = R(0);
-#pragma unroll 2
-        for (int c = 0; c < 12; ++c) {
+        constexpr int kUnroll = P == WL_F64 ? 1 : 2;
+#pragma unroll kUnroll
+        for (int c = c0; c < c0 + kComps; ++c) {
             const cx<R> sc_ = C::ld(s.rhs(h), str, c, i), rc = C::ld(r.rhs(h), str, c, i);
-            for (int j = 0; j < nact; ++j) {
-                const int k = sact[j];
-                const cx<R> *q = sc + 6 * k;
-                cx<R> xs = C::ld(sv.x[h][k], str, c, i);
-                const cx<R> ps = C::ld(sv.p[h][k], str, c, i);
-                const cx<R> pc = cmad(q[4], rc, q[5] * ps);
-                xs = cmad(q[0], pc, cmad(q[1], sc_, xs));
-                C::st(sv.x[h][k], str, c, i, xs);
-                C::st(sv.p[h][k], str, c, i, cmad(q[2], rc, cmad(q[3], sc_, pc)));
+            if constexpr (P == WL_F64) {
+                bool special = false;
+                FixComp rf, sf;
+                const int er = shift_exp(rc, kShiftMinExp, kShiftMaxExp, special);
+                const int es = shift_exp(sc_, kShiftMinExp, kShiftMaxExp, special);
+                rf.set(shift_conv(rc.re, er), shift_conv(rc.im, er), er);
+                sf.set(shift_conv(sc_.re, es), shift_conv(sc_.im, es), es);
+                // the next shift's vectors are requested before this one's arithmetic
+                int k = sact[0];
+                cx<R> xs, ps;
+                if (nact) {
+                    xs = C::ld(sv.x[h][k], str, c, i);
+                    ps = C::ld(sv.p[h][k], str, c, i);
+                }
+#pragma unroll 1
+                for (int j = 0; j < nact; ++j) {
+                    cx<R> xn, pn;
+                    int kn = k;
+                    if (j + 1 < nact) {
+                        kn = sact[j + 1];
+                        xn = C::ld(sv.x[h][kn], str, c, i);
+                        pn = C::ld(sv.p[h][kn], str, c, i);
+                    }
+                    shift_update(sfix[k], sc + 6 * k, rf, sf, special, rc, sc_, xs, ps);
+                    C::st(sv.x[h][k], str, c, i, xs);
+                    C::st(sv.p[h][k], str, c, i, ps);
+                    k = kn;
+                    xs = xn;
+                    ps = pn;
+                }
+            } else {
+                for (int j = 0; j < nact; ++j) {
+                    const int k = sact[j];
+                    const cx<R> *q = sc + 6 * k;
+                    cx<R> xs = C::ld(sv.x[h][k], str, c, i);
+                    const cx<R> ps = C::ld(sv.p[h][k], str, c, i);
+                    const cx<R> pc = cmad(q[4], rc, q[5] * ps);
+                    xs = cmad(q[0], pc, cmad(q[1], sc_, xs));
+                    C::st(sv.x[h][k], str, c, i, xs);
+                    C::st(sv.p[h][k], str, c, i, cmad(q[2], rc, cmad(q[3], sc_, pc)));
+                }
             }
             C::st(x.rhs(h), str, c, i, cmad(al, C::ld(p.rhs(h), str, c, i), cmad(om, sc_, C::ld(x.rhs(h), str, c, i))));
             const cx<R> rn = sc_ - om * C::ld(t.rhs(h), str, c, i);
@@ -390,7 +581,7 @@ extern "C" int bicgstab_m_solve(wl_gauge *g, const void *b, void *const *x, cons
     std::unique_lock<std::mutex> lock(g->mu);
     cudaStream_t s = as_stream(stream);
     const Geom &geo = g->lat->geom;
-    const int nsb = site_blocks(geo);
+    const int nsb = site_blocks(geo), nsu = (geo.Vh + update_sites(P) - 1) / update_sites(P);
     int is = 0;
     for (int i = 1; i < n_mass; ++i)
         if (m0[i] < m0[is]) is = i;
@@ -518,9 +709,9 @@ extern "C" int bicgstab_m_solve(wl_gauge *g, const void *b, void *const *x, cons
             note_launch(q);
         }
         if (P == WL_DF)
-            launch_chained(k_m_update<WL_DF>, 2 * nsb, kBlock, q, geo, nsb, xv, pv, sv, t, r, rhat, shv, sh, ns, st, partials);
+            launch_chained(k_m_update<WL_DF>, 2 * nsu, kBlock, q, geo, nsu, xv, pv, sv, t, r, rhat, shv, sh, ns, st, partials);
         else
-            launch_chained(k_m_update<WL_F64>, 2 * nsb, kBlock, q, geo, nsb, xv, pv, sv, t, r, rhat, shv, sh, ns, st, partials);
+            launch_chained(k_m_update<WL_F64>, 2 * nsu, kBlock, q, geo, nsu, xv, pv, sv, t, r, rhat, shv, sh, ns, st, partials);
         launch_chained(k_shift_b, 1, 32, q, sh, ns, st, mst);
         if (P == WL_DF) launch_chained(k_m_p<WL_DF>, 2 * nsb, kBlock, q, geo, nsb, r, pv, v, st);
         else launch_chained(k_m_p<WL_F64>, 2 * nsb, kBlock, q, geo, nsb, r, pv, v, st);
