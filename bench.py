@@ -8,8 +8,8 @@ BiCGstab, Lagrange initial guesses, masses heaviest first) for every source
 of the workload, the sources batched into multimass_solve calls.  The line
 also carries the end-to-end time through the public API with host inputs
 and outputs, a roofline entry for each hop class that takes a large share
-of the step (the inner hop against HBM, the FP64 residual hop against the
-FP64 pipe), the FP64 oracle's time on the host cores, the solution error
+of the step (the inner hop against HBM, the FP64 residual hop beside the
+FP64 pipe's rate), the FP64 oracle's time on the host cores, the solution error
 against stored oracle solutions per mass, and the multi-shift BiCGstab-M
 baseline (FP64 and double-float) on the same GPU.
 
@@ -80,10 +80,13 @@ FLOP_SITE = 1320   # per hop output site and rhs
 # lattice sites of the captured case, bytes).  Traffic scales with sites.
 # An entry is valid only for the kernel as it was when captured; remove it
 # when that kernel changes.
-HOP_TRAFFIC = {("f16", 105, 3): (1048576, 617.48e6), ("f16", 106, 3): (1048576, 617.32e6),
+HOP_TRAFFIC = {("f16", 105, 3): (1048576, 617.61e6), ("f16", 106, 3): (1048576, 617.19e6),
+               ("f16", 8105, 3): (1048576, 617.64e6), ("f64", 6000, 3): (442368, 1012.35e6),
                ("f64", 101, 3): (442368, 1013.01e6), ("f64", 103, 3): (442368, 1024.87e6)}
-# FP64 pipe utilisation of the FP64 hop in the same captures
-FP64_PIPE = {(101, 3): "92.6% busy in an ncu capture of this variant on 24^3x64, 3 rhs",
+# pipe utilisation of the FP64 hop in the same captures
+FP64_PIPE = {(6000, 3): "29% busy, integer multiply-add pipe 70%, ALU 52%, issue 57% in an ncu capture of this "
+                        "variant on 24^3x64, 3 rhs",
+             (101, 3): "92.6% busy in an ncu capture of this variant on 24^3x64, 3 rhs",
              (103, 3): "92.6% busy in an ncu capture of this variant on 24^3x64, 3 rhs"}
 # FP64 FMA rate of one GB300 (TFLOP/s, 2 flops per FMA): 152 SMs x 2 FP64
 # FMA per clock x 2.07 GHz, the unit count and clock of the part
@@ -318,8 +321,10 @@ def roofline_entries(prof, inner, outer, V, peak, peak_kind, nb, hop_variant, ou
     """One entry per hop class from the solve's live CUDA-event timings: the
     inner hop (D_oe p, the first hop of every inner BiCGstab iteration) is
     bound by HBM bandwidth; the FP64 residual hop (D_oe x, the first hop of
-    every outer check) by the FP64 pipe, whose FMA rate GB300 cuts to 1/57
-    of FP32.  Each entry also gives the class's estimated share of the step:
+    every outer check) by arithmetic.  That hop runs in block fixed point on
+    the integer pipes (variants 6000 and up), for which no flop peak is
+    defined: its entry gives the rate, the rate over that of the FP64 pipe,
+    which GB300 cuts to 1/57 of FP32, and the fraction of HBM.  Each entry also gives the class's estimated share of the step:
     its mean launch time times its launches per step (four hops per inner
     iteration, two per outer check)."""
     out = {}
@@ -353,13 +358,18 @@ def roofline_entries(prof, inner, outer, V, peak, peak_kind, nb, hop_variant, ou
             if ("f64", outer_variant, nb) in HOP_TRAFFIC:
                 sites_cap, bytes_cap = HOP_TRAFFIC[("f64", outer_variant, nb)]
                 otraffic = bytes_cap * (V // 2) / sites_cap
-            out["outer"] = {"bound": "alu", "achieved": tf, "peak": FP64_PEAK_TFLOPS, "unit": "TFLOP/s",
-                            "frac": tf / FP64_PEAK_TFLOPS, "traffic": otraffic,
-                            "fp64_pipe": FP64_PIPE.get((outer_variant, nb)),
-                            "kernel": f"k_hop<f64> (D_oe x, first hop of each outer FP64 residual check), "
+            fix = 6000 <= outer_variant < 7000
+            obytes = po["sites"] / po["launches"] * 8 * LINK_B["f64"] + site_rhs * 2 * SPINOR_B["f64"]
+            out["outer"] = {"bound": "alu", "achieved": tf, "peak": None if fix else FP64_PEAK_TFLOPS, "unit": "TFLOP/s",
+                            "frac": None if fix else tf / FP64_PEAK_TFLOPS, "traffic": otraffic,
+                            "over_fp64_pipe_rate": tf / FP64_PEAK_TFLOPS, "hbm_frac": obytes / avg / 1e9 / peak,
+                            "bytes_per_launch": obytes, "fp64_pipe": FP64_PIPE.get((outer_variant, nb)),
+                            "kernel": f"{'k_hop_fix' if fix else 'k_hop<f64>'} (D_oe x, first hop of each outer FP64 residual check), "
                                       f"variant {outer_variant}, {site_rhs / (po['sites'] / po['launches']):.2f} "
                                       f"rhs per launch on average",
-                            "peak_kind": "FP64 FMA rate from the unit count and clock (152 SMs x 2 FMA/clk "
+                            "peak_kind": "none: 64-bit integer arithmetic (FP64 FMA rate from the unit count and "
+                                         "clock: 152 SMs x 2 FMA/clk x 2.07 GHz)" if fix else
+                                         "FP64 FMA rate from the unit count and clock (152 SMs x 2 FMA/clk "
                                          "x 2.07 GHz)",
                             "flops_per_site": FLOP_SITE, "avg_launch_us": avg * 1e6,
                             "timed_launches": po["launches"]}
@@ -538,7 +548,9 @@ def run_ours(args, cfg):
     for gw in gs:
         api.profile_enable(gw, False)
     hop_variant = api.autotune(g, inner, nb)[0]   # the cached choices the solves used
-    outer_variant = (7000 + 100 * min(nb, 2) + ob) if (ob and outer == "f64") else api.autotune(g, outer, nb)[0]
+    outer_variant = api.autotune(g, outer, nb)[0]
+    if ob and outer == "f64":   # the looping grid of the same arithmetic
+        outer_variant = 6000 + ob if outer_variant >= 6000 else 7000 + 100 * min(nb, 2) + ob
     barrier(ws)
     t_step = max_over_ranks(float(np.mean(step_ms)) / 1e3, ws)
 

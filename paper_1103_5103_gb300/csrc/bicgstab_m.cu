@@ -212,8 +212,8 @@ __global__ void __launch_bounds__(kBlock) k_m_s(Geom g, int nsb, Vec r, Vec v, V
 //    units of 2^(e-1084), below 2^62;
 //  - their product (hi*hi and the two cross terms of balanced 32-bit limbs,
 //    as in the FP64 hop) has scale S = e + e', units of 2^(S-2101), and is
-//    below 2^58 (complex: below 2^59 with the second term).  A component
-//    with exponent e is the same integer at scale e + 1020;
+//    below 2^58.  A component with exponent e is the same integer at scale
+//    e + 1020;
 //  - a sum is formed at the largest scale of its terms, whose rounding unit
 //    is 2^-55 of the term that sets it where FP64's is 2^-53, and is rounded
 //    to FP64 once, at the store.  Error against exact arithmetic (random
@@ -224,8 +224,9 @@ __global__ void __launch_bounds__(kBlock) k_m_s(Geom g, int nsb, Vec r, Vec v, V
 // (zeros are inside), takes the FP64 products.
 //
 // 16^3x32, seven shifts: the multi-shift solve 30.2 -> 23.2 ms.  Bound by
-// instruction latency and the ALU pipe (49% busy at 15.6 warps per SM, issue
-// 48%, DRAM 32%): most of the instructions convert, align and round.
+// the integer pipes' issue and latency at 18 warps per SM (ALU 57%,
+// multiply-add pipe 52%, FP64 pipe 20% busy, issue 56%): most of the
+// instructions convert, align and round.
 // Measured on the solve: without the prefetch 25.0, 4 to 7 blocks per SM and
 // FP64 operands reloaded instead of kept all within 2%, one thread for all 12
 // components 23.8.

@@ -585,10 +585,11 @@ __device__ __forceinline__ void reconstruct_row2(cx<R> (&u)[9])
     u[8] = {c.re, -c.im};
 }
 
-// FP64 links keep all three rows as given (18 reals): the FP64 hop is bound
-// by the FP64 pipe (1/57 of the FP32 rate on GB300), where rebuilding row 2
-// costs about 10% of its instructions, and not by memory, where the extra
-// 48 B per link are cheap.
+// FP64 links keep all three rows as given (18 reals): the FP64 transporters
+// (handles without integer links, sites outside the integers' range, the
+// persistent kernel) are bound by the FP64 pipe (1/57 of the FP32 rate on
+// GB300), where rebuilding row 2 costs about 10% of their instructions, and
+// not by memory, where the extra 48 B per link are cheap.
 template <> struct LinkIO<WL_F64> {
     using R = double;
     static constexpr int chunks = 9;

@@ -732,7 +732,8 @@ __global__ void __launch_bounds__(128, MINB) k_hop(HopArgs a, EpiStore epi)
 
 // Grid-stride form of k_hop: a fixed grid of blocks_per_sm x SM-count
 // blocks, each looping over the (site block, rhs group) tiles.  Meant for
-// the FP64 hop, which is bound by the FP64 pipe (1/57 of the FP32 rate on
+// the FP64 hop of handles without integer links (k_hop_fix has a looping grid
+// of its own), which is bound by the FP64 pipe (1/57 of the FP32 rate on
 // GB300) and needs only a few warps per SM to keep it busy: with a small
 // grid it leaves most warp slots and issue cycles to kernels of another
 // stream running at the same time (another batch's FP32/FP16 inner solve),
