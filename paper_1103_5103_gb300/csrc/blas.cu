@@ -121,30 +121,30 @@ __global__ void __launch_bounds__(kBlock) k_xr_update(Geom g, Vec x, Vec p, Vec 
         red[2] = n;
     }
     double tot[3];
-    if (site_sum<3>(red, g, partials, q.r, &S.ticket[2], q.sb, q.nsb, tot) &&
-        threadIdx.x == 0) {
-        const double r1re = tot[0], r1im = tot[1], rr = tot[2];
+    if (site_sum<3>(red, g, partials, q.r, &S.ticket[2], q.sb, q.nsb, tot) && threadIdx.x < 32) {
+        const double r1re = lane_get(tot[0], 0), r1im = lane_get(tot[1], 0), rr = lane_get(tot[2], 0);
+        const double ore = S.omega_re, oim = S.omega_im, pre = S.rho_re, pim = S.rho_im;
+        const double are = S.alpha_re, aim = S.alpha_im;
+        const double rho2 = pre * pre + pim * pim, om2 = ore * ore + oim * oim;
+        // beta = (rho1 / rho) * (alpha / omega): the four quotients by four lanes
+        const int l = threadIdx.x & 3;
+        const double nr = l < 2 ? r1re : are, ni = l < 2 ? r1im : aim;
+        const double dr = l < 2 ? pre : ore, di = l < 2 ? pim : oim;
+        const double quo = ((l & 1) ? ni * dr - nr * di : nr * dr + ni * di) / (l < 2 ? rho2 : om2);
+        const double qre = lane_get(quo, 0), qim = lane_get(quo, 1), wre = lane_get(quo, 2), wim = lane_get(quo, 3);
+        if (threadIdx.x != 0) return;
         S.iters += 1;
         S.rr = rr;
-        const double ore = S.omega_re, oim = S.omega_im;
         if (!isfinite(rr) || !isfinite(r1re) || !isfinite(r1im)) {
             S.breakdown = 1;
             S.done = 1;
         } else if (rr <= S.target2) {
             S.done = 1;
         } else {
-            const double rho2 = S.rho_re * S.rho_re + S.rho_im * S.rho_im;
-            const double om2 = ore * ore + oim * oim;
             if (!(rho2 > 0.0) || !(om2 > 0.0) || !(r1re * r1re + r1im * r1im > S.brk2 * S.rhat2 * rr)) {
                 S.breakdown = 1;
                 S.done = 1;
             } else {
-                // beta = (rho1 / rho) * (alpha / omega)
-                const double qre = (r1re * S.rho_re + r1im * S.rho_im) / rho2;
-                const double qim = (r1im * S.rho_re - r1re * S.rho_im) / rho2;
-                const double are = S.alpha_re, aim = S.alpha_im;
-                const double wre = (are * ore + aim * oim) / om2;
-                const double wim = (aim * ore - are * oim) / om2;
                 S.beta_re = qre * wre - qim * wim;
                 S.beta_im = qre * wim + qim * wre;
                 S.rho_re = r1re;

@@ -998,7 +998,20 @@ __device__ __forceinline__ void hop_reduce_finish(const Geom &g, const EpiReduce
     constexpr int NV = EpiReduce<KIND>::NV;
     double tot[NV];
     if (site_sum<NV>(red, g, e.partials, r, &st.ticket[KIND], e.blk_off + sb, e.blk_total, tot) &&
-        threadIdx.x == 0) {
+        threadIdx.x < 32) {
+        double quo_re = 0.0, quo_im = 0.0;   // two lanes divide
+        if constexpr (KIND == 0 || KIND == 1) {
+            const double t0 = lane_get(tot[0], 0), t1 = lane_get(tot[1], 0), t2 = lane_get(tot[NV - 1], 0);
+            double num = threadIdx.x & 1 ? t1 : t0, den = t2;
+            if constexpr (KIND == 0) {   // rho / <rhat, v>
+                num = threadIdx.x & 1 ? st.rho_im * t0 - st.rho_re * t1 : st.rho_re * t0 + st.rho_im * t1;
+                den = t0 * t0 + t1 * t1;
+            }
+            const double quo = num / den;
+            quo_re = lane_get(quo, 0);
+            quo_im = lane_get(quo, 1);
+        }
+        if (threadIdx.x != 0) return;
         if constexpr (KIND == 0) {
             const double dr = tot[0], di = tot[1];
             const double den = dr * dr + di * di;
@@ -1006,14 +1019,14 @@ __device__ __forceinline__ void hop_reduce_finish(const Geom &g, const EpiReduce
                 st.breakdown = 1;
                 st.done = 1;
             } else {  // alpha = rho / <rhat, v>
-                st.alpha_re = (st.rho_re * dr + st.rho_im * di) / den;
-                st.alpha_im = (st.rho_im * dr - st.rho_re * di) / den;
+                st.alpha_re = quo_re;
+                st.alpha_im = quo_im;
             }
         } else if constexpr (KIND == 1) {
             const double tt = tot[2];
             if (tt > 0.0 && isfinite(tt)) {
-                st.omega_re = tot[0] / tt;
-                st.omega_im = tot[1] / tt;
+                st.omega_re = quo_re;
+                st.omega_im = quo_im;
             } else {
                 st.omega_re = 0.0;
                 st.omega_im = 0.0;
