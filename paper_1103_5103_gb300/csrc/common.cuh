@@ -792,6 +792,18 @@ __device__ __forceinline__ T red_cast(R x)
     else return to_double(x);
 }
 
+// The next ticket.  Release: the caller's partial sums are visible before it
+// is counted; acquire: the caller, and after a block barrier its block, sees
+// those of every earlier ticket.  (Two full fences around a relaxed atomic
+// cost more: 8^4 with four masses 4.23 -> 4.13 ms, the gradient on 16^4 15.0 ->
+// 14.8.)
+__device__ __forceinline__ unsigned take_ticket(unsigned *ticket)
+{
+    unsigned t;
+    asm volatile("atom.add.acq_rel.gpu.u32 %0, [%1], 1;" : "=r"(t) : "l"(ticket) : "memory");
+    return t;
+}
+
 // Grid-wide deterministic reduction without a second launch ("last block"
 // pattern): every block deposits its NV partial sums in partials[blk][NV];
 // the block that arrives last (atomic ticket) adds the partials in block
@@ -828,13 +840,10 @@ __device__ __forceinline__ bool grid_finish(double (&v)[NV], double *partials, u
     if (threadIdx.x == 0) {
 #pragma unroll
         for (int k = 0; k < NV; ++k) partials[(size_t)blk * NV + k] = v[k];
-        __threadfence();
-        unsigned t = atomicAdd(ticket, 1u);
-        is_last = (t == (unsigned)nblk - 1);
+        is_last = take_ticket(ticket) == (unsigned)nblk - 1;
     }
     __syncthreads();
     if (!is_last) return false;
-    __threadfence();
     double acc[NV];
 #pragma unroll
     for (int k = 0; k < NV; ++k) acc[k] = 0.0;
@@ -896,12 +905,10 @@ __device__ __forceinline__ bool site_sum(T (&red)[NV], const Geom &g, double *pa
     if (threadIdx.x == 0) {
 #pragma unroll
         for (int k = 0; k < NV; ++k) part[(size_t)blk * NV + k] = v[k];
-        __threadfence();
-        last_blk = atomicAdd(gt, 1u) == (unsigned)in_grp - 1;
+        last_blk = take_ticket(gt) == (unsigned)in_grp - 1;
     }
     __syncthreads();
     if (!last_blk) return false;
-    __threadfence();
 #pragma unroll
     for (int k = 0; k < NV; ++k)
         v[k] = (int)threadIdx.x < in_grp ? __ldcg(part + (size_t)(first + threadIdx.x) * NV + k) : 0.0;
@@ -910,12 +917,10 @@ __device__ __forceinline__ bool site_sum(T (&red)[NV], const Geom &g, double *pa
         *gt = 0u;
 #pragma unroll
         for (int k = 0; k < NV; ++k) gsum[(size_t)grp * NV + k] = v[k];
-        __threadfence();
-        last_grp = atomicAdd(ticket, 1u) == (unsigned)ngrp - 1;
+        last_grp = take_ticket(ticket) == (unsigned)ngrp - 1;
     }
     __syncthreads();
     if (!last_grp) return false;
-    __threadfence();
 #pragma unroll
     for (int k = 0; k < NV; ++k) v[k] = 0.0;
     for (int b = threadIdx.x; b < ngrp; b += blockDim.x)
