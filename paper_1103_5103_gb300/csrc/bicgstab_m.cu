@@ -26,7 +26,7 @@
 #include <string>
 #include <vector>
 
-#include "hop_fix.cuh"
+#include "fix_scalar.cuh"
 #include "internal.h"
 
 namespace wl {
@@ -230,29 +230,11 @@ __global__ void __launch_bounds__(kBlock) k_m_s(Geom g, int nsb, Vec r, Vec v, V
 // Measured on the solve: without the prefetch 25.0, 4 to 7 blocks per SM and
 // FP64 operands reloaded instead of kept all within 2%, one thread for all 12
 // components 23.8.
-constexpr int kShiftMinExp = 600, kShiftMaxExp = 1500;
-constexpr int kShiftCoefMin = 823, kShiftCoefMax = 1223;
-constexpr int kShiftUnit = 1020;   // scale of a component: exponent + this
-
 struct FixShift {
     int4 u[6];   // cxp, cxs, cqr, cqs, cpr, bs as limbs re.lo, re.hi, im.lo, im.hi
     int e[6];
     int fp;      // a coefficient outside the range
 };
-
-// Largest biased exponent of v, zero as the smallest one; special: outside the range.
-__device__ __forceinline__ int shift_exp(cx<double> v, int lo, int hi, bool &special)
-{
-    const int A = fix_absmax(0, make_double2(v.re, v.im)), e = A >> 20;
-    special = special || e > hi || (e < lo && (A | fix_lobits(make_double2(v.re, v.im))) != 0);
-    return max(e, lo);
-}
-__device__ __forceinline__ i64 shift_conv(double x, int e)
-{
-    int neg = 0;
-    const i64 q = fix_conv(x, e, 0, neg);
-    return q - neg;
-}
 
 __device__ __forceinline__ void shift_coef(FixShift &q, int j, cx<double> v)
 {
@@ -300,17 +282,6 @@ __device__ __forceinline__ FixSum shift_mul(const int4 u, const FixComp &x, int 
     x1 += (i64)u.z * x.rh;
     const i64 half = NEAREST ? (1ll << min(sh, 62)) >> 1 : 0;
     return {fix_sar(h0 + (x0 >> 32) + half, sh), fix_sar(h1 + (x1 >> 32) + half, sh)};
-}
-
-// v 2^(S-2101), rounded to FP64 (|v| < 2^62; never subnormal within the ranges).
-__device__ __forceinline__ double shift_out(i64 v, int S)
-{
-    const i64 m = v >> 63;
-    const u64 a = (u64)((v ^ m) - m);
-    const int n = __clzll((i64)a) - 1;
-    const u64 mant = ((a << n) + (1ull << 9)) >> 10;
-    const u64 bits = mant + ((u64)(unsigned)(S - kShiftUnit + 3 - n) << 52);
-    return a ? __longlong_as_double((i64)(bits | ((u64)m & (1ull << 63)))) : 0.0;
 }
 
 // x^s and q^s of one component: p^s = cpr r + beta^s q^s, then x^s += cxp p^s
