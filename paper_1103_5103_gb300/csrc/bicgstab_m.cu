@@ -205,23 +205,13 @@ __global__ void __launch_bounds__(kBlock) k_m_s(Geom g, int nsb, Vec r, Vec v, V
 // The FP64 shift updates in fixed point.  Six complex products per component
 // and shift are 24 FP64 multiply-adds, and at 1.7 per clock and SM the update
 // was bound by the FP64 pipe and more than half of a multi-shift solve; as
-// 64-bit integers they are 72 multiply-adds at 53-62 per clock.  Each complex
-// number has its own scale:
-//  - a component with largest biased exponent e is an integer in units of
-//    2^(e-1081), below 2^59 (fix_conv: kFixFrac = 58); a coefficient one in
-//    units of 2^(e-1084), below 2^62;
-//  - their product (hi*hi and the two cross terms of balanced 32-bit limbs,
-//    as in the FP64 hop) has scale S = e + e', units of 2^(S-2101), and is
-//    below 2^58.  A component with exponent e is the same integer at scale
-//    e + 1020;
-//  - a sum is formed at the largest scale of its terms, whose rounding unit
-//    is 2^-55 of the term that sets it where FP64's is 2^-53, and is rounded
-//    to FP64 once, at the store.  Error against exact arithmetic (random
-//    complex values, relative l2): x^s 4.8-6.9e-17, FP64 products 7.4-9.6e-17;
-//    q^s 4.8-5.3e-17 and 6.7-10.2e-17, for residuals of 1 to 1e-10 of x and
-//    for exponents that differ by up to 300.
-// A component outside 2^(-423..478), or a coefficient outside 2^(-200..201)
-// (zeros are inside), takes the FP64 products.
+// 64-bit integers (fix_scalar.cuh) they are 72 multiply-adds at 53-62 per
+// clock.  A sum is formed at the largest scale of its terms, whose rounding
+// unit is 2^-55 of the term that sets it where FP64's is 2^-53, and is rounded
+// to FP64 once, at the store.  Error against exact arithmetic (random complex
+// values, relative l2): x^s 4.8-6.9e-17, FP64 products 7.4-9.6e-17; q^s
+// 4.8-5.3e-17 and 6.7-10.2e-17, for residuals of 1 to 1e-10 of x and for
+// exponents that differ by up to 300.
 //
 // 16^3x32, seven shifts: the multi-shift solve 30.2 -> 23.2 ms.  Bound by
 // the integer pipes' issue and latency at 18 warps per SM (ALU 57%,
