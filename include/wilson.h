@@ -220,6 +220,15 @@ int wl_gauge_create(wl_lattice *lat, const void *U_canon_c128, unsigned prec_mas
                     wl_gauge **out);
 int wl_gauge_destroy(wl_gauge *g);
 
+/* FP64 links are held twice: as given (144 B per link), and as integers for
+ * the fixed-point FP64 hop (144 B more; see wilson_hop_multi).  A handle for
+ * whose integer links there is no memory at creation does without them: its
+ * FP64 hops run on the FP64 pipe, about three times slower.  This call
+ * releases them for the rest of the handle's life, for callers that need the
+ * memory more (no effect on a handle without them); the variants 6000 to
+ * 6002 are then refused.  Synchronises the device. */
+int wl_gauge_release_integer_links(wl_gauge *g);
+
 /* ---------------------------------------------------------------- dslash */
 
 /* One parity hop on internal spinors (Section 2, Eq. 4; Algorithm 1 without

@@ -89,6 +89,7 @@ _sig("wl_spinor_import", [_vp, _vp, _vp, _int, _int, _vp])
 _sig("wl_spinor_export", [_vp, _vp, _vp, _int, _int, _vp])
 _sig("wl_gauge_create", [_vp, _vp, ctypes.c_uint, _vp, ctypes.POINTER(_vp)])
 _sig("wl_gauge_destroy", [_vp])
+_sig("wl_gauge_release_integer_links", [_vp])
 _sig("wilson_hop", [_vp, _vp, _vp, _vp, _dbl, _int, _int, _int, _vp])
 _sig("wilson_hop_multi", [_vp, _vp, _vp, _vp, _dbl, _int, _int, _int, _int, ctypes.c_size_t, _int, _vp])
 _sig("wilson_dslash", [_vp, _vp, _vp, _dbl, _int, _int, _vp])
@@ -232,6 +233,10 @@ class Gauge:
         _check(_lib.wl_gauge_create(lat.handle, _ptr(U), mask, _stream(stream), ctypes.byref(h)))
         self.handle = h
         self.lat = lat
+
+    def release_integer_links(self):
+        """Free the integer copy of the FP64 links; FP64 hops then run on the FP64 pipe."""
+        _check(_lib.wl_gauge_release_integer_links(self.handle))
 
     def close(self):
         if getattr(self, "handle", None):

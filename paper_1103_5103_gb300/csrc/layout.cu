@@ -108,6 +108,19 @@ void Workspace::release()
     bufs.clear();
 }
 
+bool release_integer_links(wl_gauge *g)
+{
+    if (!g->fix_links[0]) return false;
+    cudaDeviceSynchronize();
+    g->inner_graph.release();
+    for (int par = 0; par < 2; ++par) {
+        cudaFree(g->fix_links[par]);
+        g->fix_links[par] = nullptr;
+    }
+    for (auto it = g->tune.begin(); it != g->tune.end();) it = it->first.first == WL_F64 ? g->tune.erase(it) : std::next(it);
+    return true;
+}
+
 int make_vec(wl_gauge *g, const std::string &name, int prec, int nrhs, Vec *v)
 {
     v->prec = prec;
@@ -678,6 +691,15 @@ extern "C" int wl_gauge_create(wl_lattice *lat, const void *U, unsigned prec_mas
         return WL_ERR_CUDA;
     }
     *out = g;
+    return WL_OK;
+}
+
+extern "C" int wl_gauge_release_integer_links(wl_gauge *g)
+{
+    if (!g) { set_error("wl_gauge_release_integer_links: NULL"); return WL_ERR_ARG; }
+    std::lock_guard<std::mutex> lock(g->mu);
+    release_integer_links(g);
+    WL_CUDA_TRY(cudaGetLastError());
     return WL_OK;
 }
 

@@ -55,12 +55,13 @@ int hop_variant_for(wl_gauge *g, int prec, int nrhs, int rhs_block)
 static const std::vector<int> &tune_candidates(const wl_gauge *g, int prec)
 {
     static const std::vector<int> f32 = {8104, 105, 106, 205}, f16 = {105, 106, 8105}, fix = {6000},
-                                  dfv = {101, 103, 104};
+                                  pipe = {101, 103, 201, 7101, 7102, 7201, 7202}, dfv = {101, 103, 104};
     switch (prec) {
     case WL_F32: return f32;
     case WL_F16: return f16;
     case WL_DF: return dfv;
-    default: return g->fix_links[0] ? fix : hop_variants(prec);   // (hop_variant_for)
+    case WL_F64: return g->fix_links[0] ? fix : pipe;   // (hop_variant_for)
+    default: return hop_variants(prec);
     }
 }
 
