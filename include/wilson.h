@@ -222,12 +222,18 @@ int wl_gauge_destroy(wl_gauge *g);
 
 /* FP64 links are held twice: as given (144 B per link), and as integers for
  * the fixed-point FP64 hop (144 B more; see wilson_hop_multi).  A handle for
- * whose integer links there is no memory at creation does without them: its
- * FP64 hops run on the FP64 pipe, about three times slower.  This call
- * releases them for the rest of the handle's life, for callers that need the
- * memory more (no effect on a handle without them); the variants 6000 to
- * 6002 are then refused.  Synchronises the device. */
+ * whose integer links there is no memory at creation, or no longer when a
+ * call allocates workspace, does without them: its FP64 hops run on the FP64
+ * pipe, about three times slower.  This call releases them for the rest of
+ * the handle's life, for callers that need the memory elsewhere (no effect on
+ * a handle without them); the variants 6000 to 6002 are then refused.
+ * Synchronises the device. */
 int wl_gauge_release_integer_links(wl_gauge *g);
+
+/* Test hook: of the handle's further workspace allocations, the one after
+ * `after` successful ones fails once as if device memory had run out
+ * (after < 0: none). */
+int wl_gauge_fail_allocation(wl_gauge *g, int after);
 
 /* ---------------------------------------------------------------- dslash */
 

@@ -90,6 +90,7 @@ _sig("wl_spinor_export", [_vp, _vp, _vp, _int, _int, _vp])
 _sig("wl_gauge_create", [_vp, _vp, ctypes.c_uint, _vp, ctypes.POINTER(_vp)])
 _sig("wl_gauge_destroy", [_vp])
 _sig("wl_gauge_release_integer_links", [_vp])
+_sig("wl_gauge_fail_allocation", [_vp, _int])
 _sig("wilson_hop", [_vp, _vp, _vp, _vp, _dbl, _int, _int, _int, _vp])
 _sig("wilson_hop_multi", [_vp, _vp, _vp, _vp, _dbl, _int, _int, _int, _int, ctypes.c_size_t, _int, _vp])
 _sig("wilson_dslash", [_vp, _vp, _vp, _dbl, _int, _int, _vp])
@@ -237,6 +238,10 @@ class Gauge:
     def release_integer_links(self):
         """Free the integer copy of the FP64 links; FP64 hops then run on the FP64 pipe."""
         _check(_lib.wl_gauge_release_integer_links(self.handle))
+
+    def fail_allocation(self, after: int):
+        """Test hook: the workspace allocation after this many more fails once."""
+        _check(_lib.wl_gauge_fail_allocation(self.handle, int(after)))
 
     def close(self):
         if getattr(self, "handle", None):

@@ -188,6 +188,7 @@ extern "C" int wilson_hop(wl_gauge *g, const void *in, void *out, const void *x,
     vi.rhs_bytes = vo.rhs_bytes = vx.rhs_bytes = spinor_bytes(g->lat->geom, prec);
     vo.ptr = out;
     vx.ptr = const_cast<void *>(x);
+    std::lock_guard<std::mutex> lock(g->hop_mu);
     return dslash_checked(hop(g, vi, vo, x ? &vx : nullptr, coef, out_parity, dagger ? 1 : 0, 1, as_stream(stream)),
                           stream);
 }
@@ -212,6 +213,7 @@ extern "C" int wilson_hop_multi(wl_gauge *g, const void *in, void *out, const vo
     vi.prec = vo.prec = vx.prec = prec;
     vi.nrhs = vo.nrhs = vx.nrhs = n_rhs;
     vi.rhs_bytes = vo.rhs_bytes = vx.rhs_bytes = rhs_stride;
+    std::lock_guard<std::mutex> lock(g->hop_mu);
     return dslash_checked(hop(g, vi, vo, x ? &vx : nullptr, coef, out_parity, dagger ? 1 : 0, rhs_block,
                               as_stream(stream)), stream);
 }
@@ -260,12 +262,10 @@ static int dslash_common(wl_gauge *g, const void *in, void *out, double kappa, i
     std::lock_guard<std::mutex> lock(g->mu);
     cudaStream_t s = as_stream(stream);
     const Geom &geo = g->lat->geom;
-    if (dslash_direct(g, in, out, prec)) {
-        Vec tmp;
-        if (op == WL_OP_MPREC) WL_TRY(make_vec(g, "dslash_oo", prec, 1, &tmp));
-        return dslash_fix(g, in, out, kappa, op, dagger, tmp.ptr, s);
-    }
     Vec ie, io, oe, oo;
+    // (an allocation may release the integer links: it comes before the choice)
+    if (op == WL_OP_MPREC) WL_TRY(make_vec(g, "dslash_oo", prec, 1, &oo));
+    if (dslash_direct(g, in, out, prec)) return dslash_fix(g, in, out, kappa, op, dagger, oo.ptr, s);
     WL_TRY(make_vec(g, "dslash_ie", prec, 1, &ie));
     WL_TRY(make_vec(g, "dslash_io", prec, 1, &io));
     WL_TRY(make_vec(g, "dslash_oe", prec, 1, &oe));

@@ -3,6 +3,7 @@
 
 #include <cuda_runtime.h>
 
+#include <functional>
 #include <map>
 #include <utility>
 #include <mutex>
@@ -38,6 +39,8 @@ struct Vec {
 // across calls, freed with the handle.
 struct Workspace {
     std::map<std::string, DevBuf> bufs;
+    std::function<bool()> reclaim;   // frees other memory of the handle when an allocation fails; false: nothing to free
+    int fail_after = -1;             // >= 0: the allocation after this many more fails once (wl_gauge_fail_allocation)
     int get(const std::string &name, size_t bytes, void **out);
     void release();
 };
@@ -86,6 +89,7 @@ struct wl_gauge {
     wl::Workspace ws;
     wl::HostPinned pinned;
     std::mutex mu;      // one solve at a time per handle (shared workspace)
+    std::mutex hop_mu;  // the single hops, which run beside a solve, against changes of fix_links and tune; taken after mu
     int profiling = 0;
     wl_kernel_profile prof[4] = {};   // inner hop per precision index (F64, F32, F16); [3] outer residual hop
 };

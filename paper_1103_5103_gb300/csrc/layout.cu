@@ -89,8 +89,14 @@ int Workspace::get(const std::string &name, size_t bytes, void **out)
         if (b.ptr) cudaFree(b.ptr);
         b.ptr = nullptr;
         b.bytes = 0;
-        cudaError_t e = cudaMalloc(&b.ptr, bytes);
+        cudaError_t e = fail_after == 0 ? cudaErrorMemoryAllocation : cudaMalloc(&b.ptr, bytes);
+        if (fail_after >= 0) --fail_after;
+        if (e == cudaErrorMemoryAllocation && reclaim && reclaim()) {
+            (void)cudaGetLastError();
+            e = cudaMalloc(&b.ptr, bytes);
+        }
         if (e != cudaSuccess) {
+            (void)cudaGetLastError();   // reported here; not by the next launch
             set_error("workspace '" + name + "' cudaMalloc(" + std::to_string(bytes) + "): " + cudaGetErrorString(e));
             b.ptr = nullptr;
             return e == cudaErrorMemoryAllocation ? WL_ERR_OOM : WL_ERR_CUDA;
@@ -111,6 +117,7 @@ void Workspace::release()
 bool release_integer_links(wl_gauge *g)
 {
     if (!g->fix_links[0]) return false;
+    std::lock_guard<std::mutex> lock(g->hop_mu);
     cudaDeviceSynchronize();
     g->inner_graph.release();
     for (int par = 0; par < 2; ++par) {
@@ -635,6 +642,7 @@ extern "C" int wl_gauge_create(wl_lattice *lat, const void *U, unsigned prec_mas
         }
     }
     wl_gauge *g = new wl_gauge;
+    g->ws.reclaim = [g] { return release_integer_links(g); };
     g->lat = lat;
     g->prec_mask = prec_mask;
     std::memset(g->links, 0, sizeof(g->links));
@@ -700,6 +708,14 @@ extern "C" int wl_gauge_release_integer_links(wl_gauge *g)
     std::lock_guard<std::mutex> lock(g->mu);
     release_integer_links(g);
     WL_CUDA_TRY(cudaGetLastError());
+    return WL_OK;
+}
+
+extern "C" int wl_gauge_fail_allocation(wl_gauge *g, int after)
+{
+    if (!g) { set_error("wl_gauge_fail_allocation: NULL"); return WL_ERR_ARG; }
+    std::lock_guard<std::mutex> lock(g->mu);
+    g->ws.fail_after = after;
     return WL_OK;
 }
 

@@ -282,7 +282,7 @@ static int run_inner(Inner &in, const wl_solver_params &prm, int max_iter, const
             (uintptr_t)in.rhat.ptr, (uintptr_t)in.s.ptr, (uintptr_t)in.t.ptr, (uintptr_t)in.e.ptr,
             (uintptr_t)in.sc.state, (uintptr_t)in.sc.partials, (uintptr_t)in.sc.kappa2, (uintptr_t)nrhs,
             (uintptr_t)in.prec, (uintptr_t)in.xprec, (uintptr_t)K, (uintptr_t)rb, (uintptr_t)prof,
-            (uintptr_t)prm.inner_solver,
+            (uintptr_t)prm.inner_solver, (uintptr_t)in.g->fix_links[0],
             (uintptr_t)in.g->lat->geom.Vh};
         if (gc.exec == nullptr || gc.key != key) {
             gc.release();
@@ -477,10 +477,13 @@ static int eo_defect_correction(wl_gauge *g, const Vec &bprec, const Vec &x64, d
     WL_CUDA_TRY(cudaMemsetAsync(in.sc.outer_done, 0, sizeof(int) * nrhs, s));
     int total_restarts = 0;
     bool lincomb_check = r0_given;
-    // outer residual hops: full grid, or the FP64 grid-stride form
-    const int ohop = (prm.outer_blocks_per_sm > 0 && x64.prec == WL_F64)
-                         ? -((g->fix_links[0] ? 6000 : 7000 + 100 * (nrhs >= 2 ? 2 : 1)) + prm.outer_blocks_per_sm)
-                         : 0;
+    // outer residual hops: full grid, or the FP64 grid-stride form (chosen at
+    // each check: an allocation may have released the integer links)
+    auto outer_hop = [&] {
+        return (prm.outer_blocks_per_sm > 0 && x64.prec == WL_F64)
+                   ? -((g->fix_links[0] ? 6000 : 7000 + 100 * (nrhs >= 2 ? 2 : 1)) + prm.outer_blocks_per_sm)
+                   : 0;
+    };
     // Three levels for FP16 inner solves (prm.inner_refine): an FP16 BiCGstab
     // stops near 3e-4 of its starting residual, where the FP16 rounding of its
     // first iterations leaves the true residual; so one outer step runs FP16
@@ -525,6 +528,7 @@ static int eo_defect_correction(wl_gauge *g, const Vec &bprec, const Vec &x64, d
         // D_oe x stays in tmp64 (the reconstruction uses the last one)
         int n_hop = 0;  // rhs the residual hops process
         if (!lincomb_check) {
+            const int ohop = outer_hop();
             for (int r = 0; r < nrhs; ++r) n_hop += outer_done[r] ? 0 : 1;
             if (ev.e[0]) WL_CUDA_TRY(cudaEventRecord(ev.e[0], s));
             WL_TRY(hop_ex(g, x64, tmp64, nullptr, 0.0, nullptr, 0.0, 1.0, WL_ODD, 0, ohop, in.sc.outer_done, 1, s));

@@ -86,12 +86,12 @@ int autotune_hop(wl_gauge *g, int prec, int nrhs, cudaStream_t s, TuneResult *ou
         if (out) *out = it->second;
         return WL_OK;
     }
-    const std::vector<int> &vs = tune_candidates(g, prec);
-    if (vs.empty()) { set_error("autotune: bad precision"); return WL_ERR_ARG; }
+    if (tune_candidates(g, prec).empty()) { set_error("autotune: bad precision"); return WL_ERR_ARG; }
     TuneResult best;
     const char *path = std::getenv("WL_AUTOTUNE_CACHE");
     const std::string fkey = tune_key(g, prec, nrhs);
     if (path && *path) {
+        const std::vector<int> &vs = tune_candidates(g, prec);
         std::ifstream f(path);
         std::string line;
         while (std::getline(f, line)) {
@@ -102,6 +102,7 @@ int autotune_hop(wl_gauge *g, int prec, int nrhs, cudaStream_t s, TuneResult *ou
             }
         }
         if (best.variant > 0) {
+            std::lock_guard<std::mutex> lock(g->hop_mu);
             g->tune[key] = best;
             if (out) *out = best;
             return WL_OK;
@@ -110,6 +111,8 @@ int autotune_hop(wl_gauge *g, int prec, int nrhs, cudaStream_t s, TuneResult *ou
     Vec in, o;
     WL_TRY(make_vec(g, "tune_in", prec, nrhs, &in));
     WL_TRY(make_vec(g, "tune_out", prec, nrhs, &o));
+    // (after the allocations, which may have released the integer links)
+    const std::vector<int> &vs = tune_candidates(g, prec);
     WL_CUDA_TRY(cudaMemsetAsync(in.ptr, 0, in.rhs_bytes * nrhs, s));
     cudaEvent_t e0, e1;
     WL_CUDA_TRY(cudaEventCreate(&e0));
@@ -148,7 +151,10 @@ int autotune_hop(wl_gauge *g, int prec, int nrhs, cudaStream_t s, TuneResult *ou
         return WL_ERR_TIMEOUT;
     }
     if (out) best.table = out->table;
-    g->tune[key] = best;
+    {
+        std::lock_guard<std::mutex> lock(g->hop_mu);
+        g->tune[key] = best;
+    }
     if (out) *out = best;
     if (path && *path) {
         std::ofstream f(path, std::ios::app);

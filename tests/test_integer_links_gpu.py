@@ -80,3 +80,69 @@ def test_multishift_and_gradient(api):
         out.append([torch.stack(xs), dU, torch.tensor(dm)])
     for a, c in zip(*out):
         assert float((a - c).norm() / a.norm()) <= 1e-8
+
+
+def _holds(api, g):
+    n = g.lat.spinor_bytes("f64")
+    a, b = (torch.zeros(n, dtype=torch.uint8, device="cuda") for _ in range(2))
+    try:
+        api.hop_batch(g, a, b, 1, (n + 255) // 256 * 256, 1.0, "f64", api.ODD, -6000)
+    except api.WilsonError:
+        return False
+    return True
+
+
+def _calls(api, b):
+    """Calls with their results, for handles that hold all precisions."""
+    def mm(**kw):
+        def f(g):
+            xs, st = api.multimass_solve(g, [b], [0.5, 0.3, 0.2], api.params(**kw))
+            assert max(s["true_relres"] for s in st[0]) <= 1e-10
+            return torch.stack(xs[0])
+        return f
+
+    def mprec(g):
+        x = torch.empty_like(b)
+        api.wilson_dslash(g, b, x, 0.13, "f64", api.OP_MPREC)
+        return x
+
+    def shifts(g):
+        xs = [torch.empty_like(b) for _ in range(2)]
+        api.bicgstab_m_solve(g, b, xs, [0.2, 0.4], api.params(outer_prec="f64"))
+        return torch.stack(xs)
+
+    def gradient(g):
+        return api.solve_backward(g, b, [b], [0.3], None, api.params(inner_prec="f64"))[0]
+
+    return dict(refined=mm(inner_prec="f16", inner_refine=1, outer_blocks_per_sm=2), ssm=mm(inner_prec="f64", guess=2),
+                mprec=mprec, shifts=shifts, gradient=gradient)
+
+
+@pytest.mark.parametrize("name", ["refined", "ssm", "mprec", "shifts", "gradient"])
+def test_out_of_memory_gives_the_integer_links_up(api, name):
+    """Whichever allocation of a call fails: the integer links are released and
+    the call goes on without them, as on a handle that never had them."""
+    from paper_1103_5103_gb300 import synth
+    U = torch.from_numpy(synth.gauge_field(DIMS, 0.4, seed=85)).cuda()
+    lat = api.Lattice(DIMS)
+    b = torch.from_numpy(synth.gaussian_source(DIMS, seed=86)).cuda()
+    call = _calls(api, b)[name]
+    ref = call(api.Gauge(lat, U))
+    after = 0
+    while True:
+        g = api.Gauge(lat, U)
+        g.fail_allocation(after)
+        x = call(g)
+        assert float((x - ref).norm() / ref.norm()) <= 1e-8, after
+        if _holds(api, g):   # fewer allocations than that
+            break
+        after += 1
+    assert after >= (1 if name == "mprec" else 10)
+    # nothing left to release: reported, and the next call finds a clean state
+    g = api.Gauge(lat, U)
+    g.release_integer_links()
+    g.fail_allocation(0)
+    with pytest.raises(api.WilsonError) as e:
+        call(g)
+    assert e.value.status == api.WL_ERR_OOM
+    assert float((call(g) - ref).norm() / ref.norm()) <= 1e-8
