@@ -226,8 +226,11 @@ int wl_gauge_destroy(wl_gauge *g);
  * call allocates workspace, does without them: its FP64 hops run on the FP64
  * pipe, about three times slower.  This call releases them for the rest of
  * the handle's life, for callers that need the memory elsewhere (no effect on
- * a handle without them); the variants 6000 to 6002 are then refused.
- * Synchronises the device. */
+ * a handle without them); the variants 6000 to 6002 are then refused.  Once
+ * an FP64 operator of the handle has been queued on a capturing stream its
+ * graph may read the integer links at any time: they stay, this call answers
+ * WL_ERR_ARG, and workspace that does not fit WL_ERR_OOM.  Synchronises the
+ * device. */
 int wl_gauge_release_integer_links(wl_gauge *g);
 
 /* Test hook: of the handle's further workspace allocations, the one after

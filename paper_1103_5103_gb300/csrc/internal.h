@@ -86,6 +86,7 @@ struct wl_gauge {
     unsigned prec_mask;
     void *links[4][2];  // [prec index][parity] -> 4 directions of 12-real links
     void *fix_links[2] = {nullptr, nullptr};  // [parity] FP64 links as integers (hop_fix.cuh); null: FP64 hops run on the FP64 pipe
+    bool captured = false;   // a caller's stream capture holds the addresses of fix_links: they stay (hop_mu)
     wl::Workspace ws;
     wl::HostPinned pinned;
     std::mutex mu;      // one solve at a time per handle (shared workspace)
@@ -107,8 +108,11 @@ int make_vec(wl_gauge *g, const std::string &name, int prec, int nrhs, Vec *v);
 
 // ---- layout.cu
 // Frees the handle's integer links and what was chosen or captured with them
-// (the caller holds g->mu); false if it holds none.
+// (the caller holds g->mu); false if it holds none, or if a caller's captured
+// graph may read them.
 bool release_integer_links(wl_gauge *g);
+// An FP64 operator is about to be queued on s for a caller (hop_mu held).
+void note_link_use(wl_gauge *g, int prec, cudaStream_t s);
 int import_spinors(const Geom &g, const void *const *canon, const Vec &out, int parity, cudaStream_t s);
 int export_spinors(const Geom &g, const Vec &in, void *const *canon, int parity, cudaStream_t s);
 // Both parities in one pass, with whole-line canonical accesses.

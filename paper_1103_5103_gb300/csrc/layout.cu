@@ -114,10 +114,18 @@ void Workspace::release()
     bufs.clear();
 }
 
+void note_link_use(wl_gauge *g, int prec, cudaStream_t s)
+{
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    if (prec == WL_F64 && !g->captured && cudaStreamIsCapturing(s, &cs) == cudaSuccess &&
+        cs == cudaStreamCaptureStatusActive)
+        g->captured = true;
+}
+
 bool release_integer_links(wl_gauge *g)
 {
-    if (!g->fix_links[0]) return false;
     std::lock_guard<std::mutex> lock(g->hop_mu);
+    if (!g->fix_links[0] || g->captured) return false;
     cudaDeviceSynchronize();
     g->inner_graph.release();
     for (int par = 0; par < 2; ++par) {
@@ -706,7 +714,10 @@ extern "C" int wl_gauge_release_integer_links(wl_gauge *g)
 {
     if (!g) { set_error("wl_gauge_release_integer_links: NULL"); return WL_ERR_ARG; }
     std::lock_guard<std::mutex> lock(g->mu);
-    release_integer_links(g);
+    if (!release_integer_links(g) && g->fix_links[0]) {
+        set_error("wl_gauge_release_integer_links: a stream capture has used them");
+        return WL_ERR_ARG;
+    }
     WL_CUDA_TRY(cudaGetLastError());
     return WL_OK;
 }

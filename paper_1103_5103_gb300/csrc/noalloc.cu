@@ -83,6 +83,10 @@ extern "C" int wilson_dslash_noalloc(wl_gauge *g, const void *in, void *out, dou
     // wl_autotune may be filling from another thread
     std::lock_guard<std::mutex> lock(g->mu);
     cudaStream_t s = as_stream(stream);
+    {
+        std::lock_guard<std::mutex> hop_lock(g->hop_mu);
+        note_link_use(g, prec, s);
+    }
     Vec ie, io, oe, oo;
     Vec *v[4] = {&ie, &io, &oe, &oo};
     for (int k = 0; k < 4; ++k) {

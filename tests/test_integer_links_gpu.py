@@ -146,3 +146,41 @@ def test_out_of_memory_gives_the_integer_links_up(api, name):
         call(g)
     assert e.value.status == api.WL_ERR_OOM
     assert float((call(g) - ref).norm() / ref.norm()) <= 1e-8
+
+
+@pytest.mark.parametrize("call", ["dslash", "noalloc", "batch"])
+def test_captured_operators_keep_the_integer_links(api, call):
+    """A caller's graph reads the links when it is replayed: neither a failed
+    allocation nor the release call takes them away."""
+    from paper_1103_5103_gb300 import synth
+    U = torch.from_numpy(synth.gauge_field(DIMS, 0.4, seed=87)).cuda()
+    lat = api.Lattice(DIMS)
+    g = api.Gauge(lat, U)
+    b = torch.from_numpy(synth.gaussian_source(DIMS, seed=88)).cuda()
+    n = (lat.spinor_bytes("f64") + 255) // 256 * 256
+    a = torch.zeros(n, dtype=torch.uint8, device="cuda")
+    lat.spinor_import(b, a, "f64", api.EVEN)
+    x = torch.empty_like(b) if call != "batch" else torch.zeros_like(a)
+
+    def run():
+        if call == "batch":
+            api.hop_batch(g, a, x, 1, n, 1.0, "f64", api.ODD)
+        else:
+            (api.wilson_dslash if call == "dslash" else api.wilson_dslash_noalloc)(g, b, x, 0.13, "f64", api.OP_MPREC)
+
+    run()   # workspace and addresses before the capture
+    torch.cuda.synchronize()
+    want = x.clone()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        run()
+    with pytest.raises(api.WilsonError):
+        g.release_integer_links()
+    g.fail_allocation(0)
+    with pytest.raises(api.WilsonError) as e:
+        api.multimass_solve(g, [b], [0.5], api.params(inner_prec="f64"))
+    assert e.value.status == api.WL_ERR_OOM and _holds(api, g)
+    x.zero_()
+    graph.replay()
+    torch.cuda.synchronize()
+    assert torch.equal(x, want)
