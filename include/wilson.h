@@ -258,9 +258,18 @@ int wilson_hop(wl_gauge *g, const void *in, void *out, const void *x, double coe
  * loads each link into registers once for all of them; rhs_block = 0 uses
  * the variant chosen by wl_autotune for (prec, n_rhs), or 1 if untuned; a
  * negative rhs_block selects the autotuner variant -rhs_block directly.
- * FP64 hops run in block fixed point on the integer pipes (64-bit integers
- * scaled per site, closer to the exact sum than FP64 arithmetic) for every
- * rhs_block >= 0; the FP64-pipe hops stay selectable as variants. */
+ * FP64 hops run in block fixed point on the integer pipes for every
+ * rhs_block >= 0, here and in every other call: the components of a site's
+ * eight neighbours are 64-bit integers on one scale, and a component of the
+ * result is off by a few 2^-56 of the LARGEST of them (below 2^-51), plus its
+ * rounding to FP64.  In norm that is closer to the exact sum than FP64
+ * arithmetic (2^-53 per operation); a component that is much smaller than
+ * its neighbourhood has fewer good bits than FP64 arithmetic leaves it where
+ * it is a sum of small terms alone.  Links that keep colours apart (one with
+ * an entry below 2^-30, such as unit or diagonal links), where whole colours
+ * can be so, therefore run on the FP64 pipe.  The FP64-pipe hops (variants
+ * 101, 103, 201, 7101 to 7202) and the fixed-point ones (6000 to 6002) can
+ * be named on every handle. */
 int wilson_hop_multi(wl_gauge *g, const void *in, void *out, const void *x, double coef, int prec,
                      int out_parity, int dagger, int n_rhs, size_t rhs_stride, int rhs_block, void *stream);
 
@@ -268,8 +277,9 @@ int wilson_hop_multi(wl_gauge *g, const void *in, void *out, const void *x, doub
  *   WL_OP_HOP   out = D in
  *   WL_OP_M     out = in - kappa D in                        (Eq. 3, kappa form)
  *   WL_OP_MPREC out_e = in_e - kappa^2 D_eo D_oe in_e, out_o = 0   (Eq. eo4)
- * computed in precision prec through the internal layout.  Scratch comes
- * from the gauge handle's workspace.  in and out must not alias. */
+ * computed in precision prec (FP64: see wilson_hop_multi for the error of its
+ * small components).  Scratch comes from the gauge handle's workspace.  in
+ * and out must not alias. */
 int wilson_dslash(wl_gauge *g, const void *in, void *out, double kappa, int prec, int op,
                   void *stream);
 /* The adjoint of the same operator: D^dag = gamma5 D gamma5. */

@@ -100,7 +100,7 @@ int hop(wl_gauge *g, const Vec &in, const Vec &out, const Vec *x, double coef, i
 static int reduce_blocks(const wl_gauge *g, int prec)
 {
     const Geom &geo = g->lat->geom;
-    return prec == WL_F64 && g->fix_links[0] ? (geo.Vh + 63) / 64 : site_blocks(geo);
+    return prec == WL_F64 && g->fixed_point() ? (geo.Vh + 63) / 64 : site_blocks(geo);
 }
 
 template <int KIND>
@@ -110,6 +110,7 @@ static int hop_reduce_k(wl_gauge *g, const Vec &tmp, const Vec &xin, double a1, 
 {
     WL_TRY(check_links(g, tmp.prec));
     HopArgs a = hop_args(g, tmp, out_parity);
+    if (!g->fixed_point()) a.fix_out = a.fix_in = nullptr;   // (hop_reduce_launch_prec)
     a.skip = &state[0].done;
     a.skip_stride = sizeof(BiState) / sizeof(int);
     EpiReduce<KIND> e;
@@ -229,7 +230,7 @@ static bool device_fields(const void *in, const void *out);
 // keep the layout passes, which read each site over the host link once.
 bool dslash_direct(const wl_gauge *g, const void *in, const void *out, int prec)
 {
-    return prec == WL_F64 && g->fix_links[0] && device_fields(in, out);
+    return prec == WL_F64 && g->fixed_point() && device_fields(in, out);
 }
 
 static bool device_fields(const void *in, const void *out)

@@ -17,9 +17,14 @@
 //  - Range: |q| < 2^59, the shrink doubles it, and a row of a link has unit
 //    norm: a transported component is below 2.45 * 2^60 / 4 units of
 //    2^(E-56), the sum of eight below 2^62.3.  Nothing overflows 63 bits.
-//  - Error: a few units of 2^(E-56) per output component, where one FP64
-//    rounding of a value of the neighbours' size is 2^(E-53): the result is
-//    closer to the exact sum than that of eight FP64 transporters.
+//  - Error: a few units of 2^(E-56) per output component (below 2^(E-51)),
+//    where one FP64 rounding of a value of the neighbours' size is 2^(E-53):
+//    in norm the result is closer to the exact sum than that of eight FP64
+//    transporters.  It is relative to the largest neighbour component, not to
+//    each one: an input 2^-k of it counts with 58 - k bits, a result of that
+//    size with about 53 - k.  Handles whose links keep colours apart, where
+//    results of one colour can be small throughout, don't come here
+//    (kMixingExp in layout.cu).
 //  - A site with a neighbour component that is not finite, of 2^878 or more,
 //    or whose components are not all zero and all below 2^-823 goes through
 //    the FP64 transporters (the exponent range of the scale; infinities, NaN).

@@ -86,6 +86,9 @@ struct wl_gauge {
     unsigned prec_mask;
     void *links[4][2];  // [prec index][parity] -> 4 directions of 12-real links
     void *fix_links[2] = {nullptr, nullptr};  // [parity] FP64 links as integers (hop_fix.cuh); null: FP64 hops run on the FP64 pipe
+    bool mixes_colours = true;   // no link keeps colours apart (smallest entry, wl_gauge_create)
+    // FP64 hops run in fixed point unless their variant is named
+    bool fixed_point() const { return fix_links[0] && mixes_colours; }
     bool captured = false;   // a caller's stream capture holds the addresses of fix_links: they stay (hop_mu)
     wl::Workspace ws;
     wl::HostPinned pinned;

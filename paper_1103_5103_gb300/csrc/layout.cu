@@ -565,20 +565,24 @@ extern "C" int wl_spinor_export(const wl_lattice *lat, const void *internal, voi
 // the entries of |U U^dag - 1| and of |det U - 1| (each as max(|re|, |im|)).
 // A NaN counts as +inf.  Blocks combine with an atomic max on the bit
 // pattern, which orders non-negative doubles (and +inf) like their values.
+// Beside it the smallest entry of any link, as the high word of max(|re|, |im|).
 static __device__ __forceinline__ void dev_max(double &m, double v)
 {
     if (!(v <= m)) m = (v != v) ? INFINITY : v;
 }
 
-static __global__ void k_su3_deviation(const double2 *__restrict__ U, size_t nlinks, unsigned long long *out)
+static __global__ void k_su3_deviation(const double2 *__restrict__ U, size_t nlinks, unsigned long long *out,
+                                        int *smallest)
 {
     double m = 0.0;
+    int e = 0x7fffffff;
     for (size_t l = (size_t)blockIdx.x * blockDim.x + threadIdx.x; l < nlinks; l += (size_t)gridDim.x * blockDim.x) {
         cx<double> u[9];
 #pragma unroll
         for (int k = 0; k < 9; ++k) {
             const double2 t = U[l * 9 + k];
             u[k] = {t.x, t.y};
+            e = min(e, max(__double2hiint(t.x) & 0x7fffffff, __double2hiint(t.y) & 0x7fffffff));
         }
 #pragma unroll
         for (int a = 0; a < 3; ++a)
@@ -596,8 +600,14 @@ static __global__ void k_su3_deviation(const double2 *__restrict__ U, size_t nli
         dev_max(m, fabs(det.im));
     }
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) dev_max(m, __shfl_xor_sync(0xffffffffu, m, o));
-    if ((threadIdx.x & 31) == 0) atomicMax(out, (unsigned long long)__double_as_longlong(m));
+    for (int o = 16; o > 0; o >>= 1) {
+        dev_max(m, __shfl_xor_sync(0xffffffffu, m, o));
+        e = min(e, __shfl_xor_sync(0xffffffffu, e, o));
+    }
+    if ((threadIdx.x & 31) == 0) {
+        atomicMax(out, (unsigned long long)__double_as_longlong(m));
+        atomicMin(smallest, e);
+    }
 }
 
 // Links further than this from SU(3) are rejected: the 12-real formats
@@ -605,18 +615,32 @@ static __global__ void k_su3_deviation(const double2 *__restrict__ U, size_t nli
 // SU(3) matrices.
 constexpr double kSU3Tol = 1e-6;
 
-static int su3_deviation(const Geom &geo, const void *U, double *dev, cudaStream_t s)
+// A link with an entry below 2^-30 keeps two colours (all but) apart: unit,
+// diagonal and block-diagonal links.  The fixed-point hop is off by a few
+// 2^-56 of the largest component of a site's neighbours, whichever colour
+// that is in; where links mix the colours every component of the result is
+// of that size, but where they don't a small colour beside a large one would
+// lose the bits that the FP64 transporters keep (a colour 2^60 below another:
+// all of them).  A handle that has such a link runs its FP64 hops on the FP64
+// pipe.  In a random SU(3) link an entry is that small with probability
+// 2 (2^-30)^2: 7e-10 for one in all links of 48^3x96.
+constexpr int kMixingExp = 1023 - 30;
+
+static int su3_deviation(const Geom &geo, const void *U, double *dev, bool *mixes_colours, cudaStream_t s)
 {
-    unsigned long long *d = nullptr, h = 0;
+    struct {
+        unsigned long long dev;
+        int smallest, pad;
+    } h = {0, 0x7fffffff, 0}, *d = nullptr;
     int dev_id = 0, nsm = 0;
     WL_CUDA_TRY(cudaGetDevice(&dev_id));
     WL_CUDA_TRY(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev_id));
-    WL_CUDA_TRY(cudaMalloc(&d, sizeof(unsigned long long)));
-    cudaError_t e = cudaMemsetAsync(d, 0, sizeof(unsigned long long), s);
+    WL_CUDA_TRY(cudaMalloc(&d, sizeof(h)));
+    cudaError_t e = cudaMemcpyAsync(d, &h, sizeof(h), cudaMemcpyHostToDevice, s);
     if (e == cudaSuccess) {
         const size_t nlinks = (size_t)4 * geo.Vh * 2;
         const unsigned grid = (unsigned)std::min<size_t>((nlinks + 255) / 256, (size_t)nsm * 8);
-        k_su3_deviation<<<grid, 256, 0, s>>>(static_cast<const double2 *>(U), nlinks, d);
+        k_su3_deviation<<<grid, 256, 0, s>>>(static_cast<const double2 *>(U), nlinks, &d->dev, &d->smallest);
         note_launch(s);
         e = cudaGetLastError();
     }
@@ -627,7 +651,8 @@ static int su3_deviation(const Geom &geo, const void *U, double *dev, cudaStream
         set_error(std::string("wl_gauge_create: ") + cudaGetErrorString(e));
         return WL_ERR_CUDA;
     }
-    std::memcpy(dev, &h, sizeof(double));
+    std::memcpy(dev, &h.dev, sizeof(double));
+    *mixes_colours = (h.smallest >> 20) >= kMixingExp;
     return WL_OK;
 }
 
@@ -638,9 +663,10 @@ extern "C" int wl_gauge_create(wl_lattice *lat, const void *U, unsigned prec_mas
         return WL_ERR_ARG;
     }
     cudaStream_t s = as_stream(stream);
+    bool mixes_colours = true;
     {
         double dev = 0.0;
-        WL_TRY(su3_deviation(lat->geom, U, &dev, s));
+        WL_TRY(su3_deviation(lat->geom, U, &dev, &mixes_colours, s));
         if (!(dev <= kSU3Tol)) {
             char msg[160];
             std::snprintf(msg, sizeof(msg), "wl_gauge_create: links are not SU(3) (largest deviation %.3g > %.0e)",
@@ -653,6 +679,7 @@ extern "C" int wl_gauge_create(wl_lattice *lat, const void *U, unsigned prec_mas
     g->ws.reclaim = [g] { return release_integer_links(g); };
     g->lat = lat;
     g->prec_mask = prec_mask;
+    g->mixes_colours = mixes_colours;
     std::memset(g->links, 0, sizeof(g->links));
     const Geom &geo = lat->geom;
     const int precs[4] = {WL_F64, WL_F32, WL_F16, WL_DF};

@@ -481,7 +481,7 @@ static int eo_defect_correction(wl_gauge *g, const Vec &bprec, const Vec &x64, d
     // each check: an allocation may have released the integer links)
     auto outer_hop = [&] {
         return (prm.outer_blocks_per_sm > 0 && x64.prec == WL_F64)
-                   ? -((g->fix_links[0] ? 6000 : 7000 + 100 * (nrhs >= 2 ? 2 : 1)) + prm.outer_blocks_per_sm)
+                   ? -((g->fixed_point() ? 6000 : 7000 + 100 * (nrhs >= 2 ? 2 : 1)) + prm.outer_blocks_per_sm)
                    : 0;
     };
     // Three levels for FP16 inner solves (prm.inner_refine): an FP16 BiCGstab

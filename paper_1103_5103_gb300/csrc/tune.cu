@@ -40,8 +40,9 @@ int hop_variant_for(wl_gauge *g, int prec, int nrhs, int rhs_block)
     if (rhs_block < 0) return -rhs_block;
     // FP64: the fixed-point hop at every size (8^4 14 against 35 us, 24^3x64
     // with three rhs 0.70 against 2.0 ms of the FP64-pipe hops); it shares the
-    // links of several rhs through L1 and has no rhs-per-thread form
-    if (prec == WL_F64 && g->fix_links[0]) return 6000;
+    // links of several rhs through L1 and has no rhs-per-thread form.  Not for
+    // links that keep colours apart (kMixingExp)
+    if (prec == WL_F64 && g->fixed_point()) return 6000;
     if (rhs_block > 0) return rhs_block * 100 + 1;
     auto it = g->tune.find(std::make_pair(prec, nrhs));
     return it == g->tune.end() ? 101 : it->second.variant;
@@ -60,7 +61,7 @@ static const std::vector<int> &tune_candidates(const wl_gauge *g, int prec)
     case WL_F32: return f32;
     case WL_F16: return f16;
     case WL_DF: return dfv;
-    case WL_F64: return g->fix_links[0] ? fix : pipe;   // (hop_variant_for)
+    case WL_F64: return g->fixed_point() ? fix : pipe;   // (hop_variant_for)
     default: return hop_variants(prec);
     }
 }

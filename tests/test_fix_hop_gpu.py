@@ -202,3 +202,75 @@ def test_canonical_application_is_the_internal_one(api, dims, kind):
             assert np.abs(a[ok] - b[ok]).max() <= 2.0 ** -50 * big
             if op == api.OP_MPREC:
                 assert np.all(a[synth.parity(dims) == 1] == 0)
+
+
+def _separating_links(dims, kind):
+    """Links that keep colours apart: unit, diagonal, or SU(2) on colours 0, 1."""
+    U = synth.unit_gauge_field(dims)
+    rng = np.random.default_rng(5)
+    if kind == "diagonal":
+        a = rng.uniform(-np.pi, np.pi, U.shape[:2] + (2,))
+        for c, p in enumerate((a[..., 0], a[..., 1], -a[..., 0] - a[..., 1])):
+            U[..., c, c] = np.exp(1j * p)
+    elif kind == "block":
+        q = rng.standard_normal(U.shape[:2] + (4,))
+        q /= np.linalg.norm(q, axis=-1, keepdims=True)
+        a, b = q[..., 0] + 1j * q[..., 1], q[..., 2] + 1j * q[..., 3]
+        U[..., 0, 0], U[..., 0, 1], U[..., 1, 0], U[..., 1, 1] = a, b, -b.conj(), a.conj()
+    return U
+
+
+@pytest.mark.parametrize("kind", ["unit", "diagonal", "block"])
+def test_colours_that_do_not_mix_keep_their_precision(api, kind):
+    """Colours 2^-30 and 2^-60 of another (block: only colour 2 stands apart):
+    each comes out to FP64 rounding of its own size, through every FP64
+    operator.  Bound per colour: 8 transporters and the epilogue, some 20
+    roundings each of at most the colour's own norm, twice for M_prec."""
+    dims = (4, 6, 2, 8)
+    U = _separating_links(dims, kind)
+    lat = api.Lattice(dims)
+    g = api.Gauge(lat, torch.from_numpy(U).cuda(), precs=("f64",))
+    psi = synth.gaussian_source(dims, seed=12) * (2.0 ** np.array([0, 0 if kind == "block" else -30, -60]))
+    odd = synth.parity(dims) == 1
+    dev, k = torch.from_numpy(psi).cuda(), 0.13
+    even_in = psi.copy()
+    even_in[odd] = 0
+
+    def close(got, want):
+        for c in range(3):
+            e = np.sqrt((np.abs(got[..., c].astype(CLD) - want[..., c]) ** 2).sum())
+            assert e <= 2.0 ** -48 * np.sqrt((np.abs(want[..., c]) ** 2).sum()), (c, float(e))
+
+    for dagger, f in ((False, api.wilson_dslash), (True, api.wilson_dslash_dag)):
+        D = _reference(U, dims, psi, dagger)[0]
+        Doe = _reference(U, dims, even_in, dagger)[0]
+        DD = _reference(U, dims, Doe, dagger)[0]
+        mprec = even_in - LD(k) ** 2 * DD
+        mprec[odd] = 0
+        for op, want in ((api.OP_HOP, D), (api.OP_M, psi - LD(k) * D), (api.OP_MPREC, mprec)):
+            a, b = torch.empty_like(dev), torch.empty_like(dev)
+            f(g, dev, a, k, "f64", op)
+            api.wilson_dslash_noalloc(g, dev, b, k, "f64", op, dagger=dagger)
+            close(a.cpu().numpy(), want)
+            close(b.cpu().numpy(), want)
+        Doe[~odd] = 0
+        close(_hop(api, lat, g, even_in, 0, dagger), Doe)             # rhs_block 1
+        close(_hop(api, lat, g, even_in, 0, dagger, nrhs=3), Doe)
+
+
+@pytest.mark.parametrize("exponent,fixed", [(-29, True), (-31, False)])
+def test_where_colours_count_as_mixed(api, exponent, fixed):
+    """The line at entries of 2^-30: rotations by 2^exponent in all three planes."""
+    dims = (2, 2, 2, 2)
+    th = 2.0 ** exponent
+    R = np.eye(3)
+    for i, j in ((0, 1), (0, 2), (1, 2)):
+        P = np.eye(3)
+        P[i, i] = P[j, j] = np.cos(th)
+        P[i, j], P[j, i] = np.sin(th), -np.sin(th)
+        R = R @ P
+    # random links but for one
+    U = synth.gauge_field(dims, 0.5, seed=33)
+    U[2, 5] = R
+    g = api.Gauge(api.Lattice(dims), torch.from_numpy(U).cuda(), precs=("f64",))
+    assert (api.autotune(g, "f64", 1)[0] == 6000) == fixed
