@@ -486,6 +486,38 @@ __global__ void __launch_bounds__(kBlock) k_norm2(Geom g, Vec a, double *out, do
         out[q.r] = tot[0];
 }
 
+__device__ __forceinline__ bool is_zero(double x) { return x == 0.0; }
+__device__ __forceinline__ bool is_zero(df x) { return x.hi == 0.f && x.lo == 0.f; }
+
+// Whether a has an entry that is not zero, exactly: flags[r] (zeroed by the
+// caller) gets its bits.  A norm cannot tell: squares of entries below 2.2e-162
+// (FP64) or 2.6e-23 (double-float norms are summed in FP32) underflow.
+template <int P>
+__global__ void __launch_bounds__(kBlock) k_nonzero(Geom g, Vec a, int *flags)
+{
+    using R = typename PrecTraits<P>::R;
+    const SiteIdx q = site_idx(a.nrhs);
+    int any = 0;
+    if (q.i < g.Vh) {
+        cx<R> v[12];
+        SpinorIO<P>::load(a.rhs(q.r), g.stride, q.i, v);
+#pragma unroll
+        for (int c = 0; c < 12; ++c) any |= !is_zero(v[c].re) || !is_zero(v[c].im);
+    }
+    if (__syncthreads_or(any) && threadIdx.x == 0) flags[q.r] = 1;
+}
+
+int blas_nonzero(const Geom &g, const Vec &a, int *flags_dev, cudaStream_t s)
+{
+    const int gr = grid_of(g, a.nrhs);
+    if (a.prec == WL_DF) launch_chained(k_nonzero<WL_DF>, gr, kBlock, s, g, a, flags_dev);
+    else if (a.prec == WL_F64) launch_chained(k_nonzero<WL_F64>, gr, kBlock, s, g, a, flags_dev);
+    else { set_error("blas_nonzero: outer precision only"); return WL_ERR_ARG; }
+    WL_CUDA_TRY(cudaGetLastError());
+    note_launch(s);
+    return WL_OK;
+}
+
 int blas_norm2(const Geom &g, const Vec &a, double *out_dev, double *partials, unsigned *tickets, cudaStream_t s)
 {
     const int gr = grid_of(g, a.nrhs);

@@ -173,6 +173,8 @@ int blas_restart(const Geom &g, const Vec &r64, const Vec &r, const Vec &rhat, c
                  BiState *state, double *partials, const int *active, const double *delta2, cudaStream_t s);
 int blas_accum(const Geom &g, const Vec &e, const Vec &x64, const int *active, cudaStream_t s);
 int blas_norm2(const Geom &g, const Vec &a, double *out_dev, double *partials, unsigned *tickets, cudaStream_t s);
+// flags[r] = 1 where rhs r has an entry that is not zero (zeroed by the caller)
+int blas_nonzero(const Geom &g, const Vec &a, int *flags_dev, cudaStream_t s);
 // out = sum_j c_j in_j, 1 <= k <= 32 inputs, real coefficients per rhs
 // c[r * k + j] (cim_dev is ignored)
 int blas_lincomb(const Geom &g, const double *cre_dev, const double *cim_dev, const Vec *const *in, int k,

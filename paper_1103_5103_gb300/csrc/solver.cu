@@ -1109,27 +1109,30 @@ extern "C" int multimass_solve(wl_gauge *g, const void *const *b, void *const *x
     Scratch sc;
     WL_TRY(get_scratch(g, n_rhs, &sc, s));
     std::vector<double> ne, no, bn2(n_rhs);
+    // which sources have an odd part, read with the norms
+    WL_CUDA_TRY(cudaMemsetAsync(sc.active, 0, sizeof(int) * n_rhs, s));
+    WL_TRY(blas_nonzero(geo, bo, sc.active, s));
+    void *pp = nullptr;
+    WL_TRY(g->pinned.get("mm_skip", sizeof(int) * 2 * n_rhs, &pp));
+    int *has_odd = static_cast<int *>(pp), *h_zero = has_odd + n_rhs;
+    WL_CUDA_TRY(cudaMemcpyAsync(has_odd, sc.active, sizeof(int) * n_rhs, cudaMemcpyDeviceToHost, s));
     WL_TRY(norms2_host(g, be, sc, ne, s));
     WL_TRY(norms2_host(g, bo, sc, no, s));
     for (int r = 0; r < n_rhs; ++r) bn2[r] = ne[r] + no[r];
     // D_eo b_o once for all masses; b_prec(m) = b_e + kappa(m) D_eo b_o.  A
     // source without an odd part (a point source on an even site) needs no
-    // hop: its D_eo b_o is zero.  ||b_o||^2 is exactly zero only if every odd
-    // entry is below 2.2e-162, whose hop would be as negligible.  If no source
-    // of the call has one, b_prec is b_e for every mass.
+    // hop: its D_eo b_o is zero.  If no source of the call has one, b_prec is
+    // b_e for every mass.
     bool odd_zero = true;
-    for (int r = 0; r < n_rhs; ++r) odd_zero &= no[r] == 0.0;
+    for (int r = 0; r < n_rhs; ++r) odd_zero &= !has_odd[r];
     if (odd_zero) {
         bprec = be;
     } else {
         WL_TRY(make_vec(g, "mm_Dbo", PO, n_rhs, &dbo));
         WL_TRY(make_vec(g, "mm_bprec", PO, n_rhs, &bprec));
-        void *pp = nullptr;
-        WL_TRY(g->pinned.get("mm_skip", sizeof(int) * n_rhs, &pp));
-        int *h_zero = static_cast<int *>(pp);
         int n_zero = 0;
         for (int r = 0; r < n_rhs; ++r) {
-            h_zero[r] = no[r] == 0.0 ? 1 : 0;
+            h_zero[r] = has_odd[r] ? 0 : 1;
             n_zero += h_zero[r];
             if (h_zero[r]) WL_CUDA_TRY(cudaMemsetAsync(dbo.rhs(r), 0, dbo.rhs_bytes, s));
         }
