@@ -23,6 +23,7 @@
 #include <vector>
 
 #include "internal.h"
+#include "iteration_group.h"
 
 namespace wl {
 
@@ -96,7 +97,7 @@ struct Inner {
     double kappa;
     Vec r, rhat, p, v, s, t, tmp, e;
     Scratch sc;
-    double rate = 0.0;   // ln of ||r||^2 lost per iteration in the last inner solve (0: none yet)
+    InnerPace pace;   // of the last inner solve for this mass
 };
 
 static int make_inner(wl_gauge *g, int prec, int nrhs, double kappa, Inner *in, cudaStream_t s)
@@ -226,23 +227,15 @@ static int capture_iterations(Inner &in, const wl_solver_params &prm, int rhs_bl
     return status;
 }
 
-// Iterations that an rhs still needs to take its residual (squared) down by
-// the factor exp(-lnf), at `rate` per iteration.
-static int iterations_for(double lnf, double rate)
-{
-    const double n = std::ceil(lnf / rate);
-    return n >= 1.0 && n < 1e6 ? (int)n : 1;
-}
-
 // Run inner iterations until every rhs is done or max_iter is reached.
 // Returns the state array copied to host in host_state.  delta2 (host, per
 // rhs, read for the rhs with active[r] != 0): the squared reduction each
 // solve stops at.
 //
 // In graph mode the iterations between two looks at the state are as many as
-// the solve is expected to need: the reduction asked for over the rate of
-// the last inner solve for this mass, later over this solve's own rate; full
-// captured blocks, then captured single iterations.  (With fixed blocks of eight, 8^4
+// the solve is expected to need (iteration_group.h): the reduction asked for
+// over the rate of the last inner solve for this mass, later over this solve's
+// own rate; full captured blocks, then captured single iterations.  (With fixed blocks of eight, 8^4
 // with four masses ran 112 iterations for 83 and 16^3x32 with eight 112 for
 // 74; a surplus iteration is seven launches that find the rhs done, 9-10 us
 // there.  8^4 x 4 masses 4.69 -> 4.58 ms, 16^3x32 x 8 8.11 -> 7.82, 24^3x64
@@ -313,16 +306,11 @@ static int run_inner(Inner &in, const wl_solver_params &prm, int max_iter, const
         ~EvFree() { for (auto e : v) cudaEventDestroy(e); }
     } ev_free{host_ev};
     int done_iters = 0;
-    double &rate = in.rate;
     const long last = ((long)max_iter + K - 1) / K * K;   // max_iter in whole blocks
     const bool predict = exec && !prof;
-    int group = K;   // iterations before the next look at the state
-    if (predict && rate > 0.0) {
-        group = 1;
-        for (int r = 0; r < nrhs; ++r)
-            if (active[r]) group = std::max(group, iterations_for(-std::log(delta2[r]), rate));
-        group = (int)std::min<long>(group, last);
-    }
+    // iterations before the next look at the state
+    int group = predict ? first_group(in.pace, K, last, delta2, active, nrhs) : K;
+    std::vector<RhsProgress> prog(nrhs);
     for (;;) {
         if (exec) {
             int n = group;
@@ -380,24 +368,14 @@ static int run_inner(Inner &in, const wl_solver_params &prm, int max_iter, const
         bool all = true;
         for (int r = 0; r < nrhs; ++r) all &= hs[r].done != 0;
         if (predict) {
-            // the slowest rhs's rate, and what is left at each one's own
-            double slowest = 0.0;
-            group = 1;
-            for (int r = 0; r < nrhs; ++r) {
-                if (!active[r] || hs[r].iters < 1 || !(hs[r].rr > 0.0)) continue;
-                const double own = std::log(hs[r].target2 / delta2[r] / hs[r].rr) / hs[r].iters;
-                if (!(own > 0.0) || !std::isfinite(own)) {
-                    group = K;
-                    continue;
-                }
-                slowest = slowest > 0.0 ? std::min(slowest, own) : own;
-                if (!hs[r].done) group = std::max(group, std::min(K, iterations_for(std::log(hs[r].rr / hs[r].target2), own)));
-            }
-            if (slowest > 0.0) rate = slowest;
-            group = (int)std::min<long>(group, last - done_iters);
+            for (int r = 0; r < nrhs; ++r)
+                prog[r] = {active[r] != 0, hs[r].done != 0, hs[r].breakdown != 0, hs[r].iters, hs[r].rr, hs[r].target2,
+                           delta2[r]};
+            group = next_group(prog.data(), nrhs, K, last - done_iters);
         }
         if (all || done_iters >= last) break;
     }
+    if (predict && status == WL_OK) in.pace = learn_pace(prog.data(), nrhs);
     std::memcpy(host_state.data(), hs, sizeof(BiState) * nrhs);
     if (status == WL_OK && hop_variant_for(in.g, in.prec, nrhs, rb) >= 9000) {
         // a TMA-staged hop that stopped waiting leaves its tile unwritten
