@@ -107,6 +107,9 @@ __device__ __forceinline__ int chain_begin()
 
 constexpr unsigned kChainBlocks = 8 * 152, kChainCaptured = 128;
 
+// Whether this thread's last launch_chained went into a stream capture.
+extern thread_local bool launch_captured;
+
 template <typename... K, typename... A>
 cudaError_t launch_chained(void (*kernel)(K...), unsigned grid, unsigned block, cudaStream_t s, const A &...args)
 {
@@ -119,8 +122,8 @@ cudaError_t launch_chained(void (*kernel)(K...), unsigned grid, unsigned block, 
     at[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = at;
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-    const bool captured = cudaStreamIsCapturing(s, &cs) == cudaSuccess && cs == cudaStreamCaptureStatusActive;
-    cfg.numAttrs = grid <= (captured ? kChainCaptured : kChainBlocks) ? 1 : 0;
+    launch_captured = cudaStreamIsCapturing(s, &cs) == cudaSuccess && cs == cudaStreamCaptureStatusActive;
+    cfg.numAttrs = grid <= (launch_captured ? kChainCaptured : kChainBlocks) ? 1 : 0;
     return cudaLaunchKernelEx(&cfg, kernel, static_cast<K>(args)...);
 }
 

@@ -190,9 +190,9 @@ extern "C" int wilson_hop(wl_gauge *g, const void *in, void *out, const void *x,
     vo.ptr = out;
     vx.ptr = const_cast<void *>(x);
     std::lock_guard<std::mutex> lock(g->hop_mu);
-    note_link_use(g, prec, as_stream(stream));
-    return dslash_checked(hop(g, vi, vo, x ? &vx : nullptr, coef, out_parity, dagger ? 1 : 0, 1, as_stream(stream)),
-                          stream);
+    const int st = hop(g, vi, vo, x ? &vx : nullptr, coef, out_parity, dagger ? 1 : 0, 1, as_stream(stream));
+    note_link_use(g, prec);
+    return dslash_checked(st, stream);
 }
 
 extern "C" int wilson_hop_multi(wl_gauge *g, const void *in, void *out, const void *x, double coef, int prec,
@@ -216,9 +216,9 @@ extern "C" int wilson_hop_multi(wl_gauge *g, const void *in, void *out, const vo
     vi.nrhs = vo.nrhs = vx.nrhs = n_rhs;
     vi.rhs_bytes = vo.rhs_bytes = vx.rhs_bytes = rhs_stride;
     std::lock_guard<std::mutex> lock(g->hop_mu);
-    note_link_use(g, prec, as_stream(stream));
-    return dslash_checked(hop(g, vi, vo, x ? &vx : nullptr, coef, out_parity, dagger ? 1 : 0, rhs_block,
-                              as_stream(stream)), stream);
+    const int st = hop(g, vi, vo, x ? &vx : nullptr, coef, out_parity, dagger ? 1 : 0, rhs_block, as_stream(stream));
+    note_link_use(g, prec);
+    return dslash_checked(st, stream);
 }
 
 namespace wl {
@@ -268,11 +268,11 @@ static int dslash_common(wl_gauge *g, const void *in, void *out, double kappa, i
     Vec ie, io, oe, oo;
     // (an allocation may release the integer links: it comes before the choice)
     if (op == WL_OP_MPREC) WL_TRY(make_vec(g, "dslash_oo", prec, 1, &oo));
-    {
-        std::lock_guard<std::mutex> hop_lock(g->hop_mu);
-        note_link_use(g, prec, s);
+    if (dslash_direct(g, in, out, prec)) {
+        const int st = dslash_fix(g, in, out, kappa, op, dagger, oo.ptr, s);
+        note_link_use(g, prec);
+        return st;
     }
-    if (dslash_direct(g, in, out, prec)) return dslash_fix(g, in, out, kappa, op, dagger, oo.ptr, s);
     WL_TRY(make_vec(g, "dslash_ie", prec, 1, &ie));
     WL_TRY(make_vec(g, "dslash_io", prec, 1, &io));
     WL_TRY(make_vec(g, "dslash_oe", prec, 1, &oe));
@@ -311,6 +311,7 @@ static int dslash_common(wl_gauge *g, const void *in, void *out, double kappa, i
         WL_CUDA_TRY(cudaMemsetAsync(oo.ptr, 0, spinor_bytes(geo, prec), s));
     }
     WL_TRY(export_full(geo, oe, oo, cout, s));
+    note_link_use(g, prec);
     return WL_OK;
 }
 

@@ -3,6 +3,7 @@
 
 #include <cuda_runtime.h>
 
+#include <atomic>
 #include <functional>
 #include <map>
 #include <utility>
@@ -89,7 +90,7 @@ struct wl_gauge {
     bool mixes_colours = true;   // no link keeps colours apart (smallest entry, wl_gauge_create)
     // FP64 hops run in fixed point unless their variant is named
     bool fixed_point() const { return fix_links[0] && mixes_colours; }
-    bool captured = false;   // a caller's stream capture holds the addresses of fix_links: they stay (hop_mu)
+    std::atomic<bool> captured{false};   // a caller's stream capture holds the addresses of fix_links: they stay
     wl::Workspace ws;
     wl::HostPinned pinned;
     std::mutex mu;      // one solve at a time per handle (shared workspace)
@@ -114,8 +115,11 @@ int make_vec(wl_gauge *g, const std::string &name, int prec, int nrhs, Vec *v);
 // (the caller holds g->mu); false if it holds none, or if a caller's captured
 // graph may read them.
 bool release_integer_links(wl_gauge *g);
-// An FP64 operator is about to be queued on s for a caller (hop_mu held).
-void note_link_use(wl_gauge *g, int prec, cudaStream_t s);
+// This thread has just queued an operator for a caller (mu or hop_mu held).
+inline void note_link_use(wl_gauge *g, int prec)
+{
+    if (prec == WL_F64 && launch_captured) g->captured = true;
+}
 int import_spinors(const Geom &g, const void *const *canon, const Vec &out, int parity, cudaStream_t s);
 int export_spinors(const Geom &g, const Vec &in, void *const *canon, int parity, cudaStream_t s);
 // Both parities in one pass, with whole-line canonical accesses.

@@ -114,13 +114,7 @@ void Workspace::release()
     bufs.clear();
 }
 
-void note_link_use(wl_gauge *g, int prec, cudaStream_t s)
-{
-    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-    if (prec == WL_F64 && !g->captured && cudaStreamIsCapturing(s, &cs) == cudaSuccess &&
-        cs == cudaStreamCaptureStatusActive)
-        g->captured = true;
-}
+thread_local bool launch_captured = false;
 
 bool release_integer_links(wl_gauge *g)
 {

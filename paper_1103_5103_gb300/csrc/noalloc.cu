@@ -83,10 +83,6 @@ extern "C" int wilson_dslash_noalloc(wl_gauge *g, const void *in, void *out, dou
     // wl_autotune may be filling from another thread
     std::lock_guard<std::mutex> lock(g->mu);
     cudaStream_t s = as_stream(stream);
-    {
-        std::lock_guard<std::mutex> hop_lock(g->hop_mu);
-        note_link_use(g, prec, s);
-    }
     Vec ie, io, oe, oo;
     Vec *v[4] = {&ie, &io, &oe, &oo};
     for (int k = 0; k < 4; ++k) {
@@ -98,7 +94,11 @@ extern "C" int wilson_dslash_noalloc(wl_gauge *g, const void *in, void *out, dou
     const int dag = dagger ? 1 : 0;
     const void *cin[1] = {in};
     void *cout[1] = {out};
-    if (dslash_direct(g, in, out, prec)) return dslash_fix(g, in, out, kappa, op, dag, base, s);
+    if (dslash_direct(g, in, out, prec)) {
+        const int st = dslash_fix(g, in, out, kappa, op, dag, base, s);
+        note_link_use(g, prec);
+        return st;
+    }
     // every scratch buffer is fully written below before it is read, except
     // the odd output of M_prec, which is defined as zero
     WL_TRY(import_full(geo, cin, ie, io, s));
@@ -114,5 +114,6 @@ extern "C" int wilson_dslash_noalloc(wl_gauge *g, const void *in, void *out, dou
         WL_CUDA_TRY(cudaMemsetAsync(oo.ptr, 0, spinor_bytes(geo, prec), s));
     }
     WL_TRY(export_full(geo, oe, oo, cout, s));
+    note_link_use(g, prec);
     return WL_OK;
 }
