@@ -442,12 +442,18 @@ int wl_wait_faults(unsigned *count, int reset, void *stream);
  *                 dots[3 r ..]: <rhat, r> (re, im) and ||r||^2 of the new r
  *   WL_VEC_P      p = r + beta (p - omega v)               vecs r, p, v
  *   WL_VEC_NORM2  dots[r] = ||a||^2                        vecs a
+ *   WL_VEC_GUESS + k   x = sum_j c_j x_j,  r = b - x + sum_j d_j y_j over
+ *                 j < k <= 15: the initial guess and first residual of
+ *                 multimass_solve; WL_F64 only; scal[2 k r ..] = c_0 ..
+ *                 c_{k-1}, d_0 .. d_{k-1} of rhs r
+ *                                     vecs x_0 .. x_{k-1}, y_0 .. y_{k-1}, b, x, r
  * Inner products: FP32 per site, FP32 within a warp, FP64 across warps and
  * blocks.  Synchronises the stream. */
 #define WL_VEC_S     0
 #define WL_VEC_XR    1
 #define WL_VEC_P     2
 #define WL_VEC_NORM2 3
+#define WL_VEC_GUESS 4
 int wl_vector_op(wl_gauge *g, int kind, int prec, int n_rhs, size_t rhs_stride, void *const *vecs,
                  const double *scal, double *dots, void *stream);
 

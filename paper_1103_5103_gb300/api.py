@@ -360,21 +360,21 @@ def wait_faults(reset: bool = True, stream=None) -> int:
     return n.value
 
 
-VEC_S, VEC_XR, VEC_P, VEC_NORM2 = 0, 1, 2, 3
+VEC_S, VEC_XR, VEC_P, VEC_NORM2, VEC_GUESS = 0, 1, 2, 3, 4
 
 
 def vector_op(g: Gauge, kind: int, prec, n_rhs: int, rhs_stride: int, vecs, scal=None, stream=None):
     """wl_vector_op on internal vectors (uint8 CUDA tensors holding n_rhs
     vectors rhs_stride bytes apart); scal: per-rhs (alpha, omega, beta)
-    complex triples.  Returns the dots (list) for VEC_XR / VEC_NORM2."""
+    complex triples, or for VEC_GUESS + k per rhs the k real c_j and then the
+    k real d_j.  Returns the dots (list) for VEC_XR / VEC_NORM2."""
     vp = (_vp * len(vecs))(*[_ptr(v).value for v in vecs])
     sc = None
     if scal is not None:
         flat = []
-        for a, o, b in scal:
-            flat += [complex(a).real, complex(a).imag, complex(o).real, complex(o).imag,
-                     complex(b).real, complex(b).imag]
-        sc = (_dbl * len(flat))(*flat)
+        for row in scal:
+            flat += [float(v) for v in row] if kind >= VEC_GUESS else [w for v in row for w in (complex(v).real, complex(v).imag)]
+        sc = (_dbl * max(1, len(flat)))(*flat)
     nd = 3 * n_rhs if kind == VEC_XR else n_rhs
     d = (_dbl * nd)()
     _check(_lib.wl_vector_op(g.handle, int(kind), _prec(prec), int(n_rhs), int(rhs_stride), vp, sc, d,

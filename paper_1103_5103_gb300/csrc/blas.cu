@@ -669,9 +669,14 @@ __global__ void __launch_bounds__(kBlock) k_guess_residual(Geom g, LinIn in, int
 // by the FP64 pipe.  Each complex number's sum has a running scale: a term of
 // a larger one moves the sum down, others are converted at the sum's.  x is
 // rounded to FP64 before it is subtracted, as above.  At most 15 terms: x
-// below 15 2^57, r below 2 2^59 + 15 2^57, both below 2^62.  Error against
-// exact sums (2 to 15 Lagrange terms, relative l2): x 4.8e-17 to 1.7e-16, in
-// FP64 5.7e-17 to 5.1e-16; r 0.8-9.2e-17 of |b|, in FP64 3.3e-17 to 2.3e-16.
+// below 15 2^57, r below 2 2^59 + 15 2^57, both below 2^62.  Error: per term
+// at most four units of 2^-55 of the largest term of its complex number
+// (conversion, the dropped lo*lo, the rounded low word, a move to a larger
+// scale), and the rounding to FP64.  Measured against exact sums (2 to 15
+// Lagrange terms, relative l2): x 4.8e-17 to 1.7e-16, in FP64 5.7e-17 to
+// 5.1e-16; r 0.8-9.2e-17 of |b|, in FP64 3.3e-17 to 2.3e-16.  The smaller of
+// re and im has the error of the larger one; the checks of the solve, which
+// recompute the residual, don't build on these values.
 //
 // 32^3x64, three sources and 16 masses, FP16 inner: 210.6 -> 208.9 ms (with
 // 2, 4 and 6 components in flight 211.0, 209.5 and 217.1).
@@ -721,8 +726,8 @@ __global__ void __launch_bounds__(kBlock) k_guess_residual_fix(Geom g, LinIn in,
         sc[t] = {(int)w, fix_hi(w), e, special ? 1 : 0};
     }
     __syncthreads();
-    if (q.i >= g.Vh) return;
-    const size_t off = (size_t)q.r * rhs_bytes + (size_t)q.i * sizeof(double2);
+    if (q.i >= g.Vh || !WL_STORE_OK(q.i, g.stride, 2)) return;
+    const size_t off = (size_t)q.r * rhs_bytes + (size_t)WL_LOAD_IDX(q.i, g.stride, 1) * sizeof(double2);
     bool cfp = false;
     for (int j = 0; j < 2 * k; ++j) cfp = cfp || sc[j].fp;
     double2 *xp = static_cast<double2 *>(xo.rhs(q.r)) + q.i, *rp = static_cast<double2 *>(ro.rhs(q.r)) + q.i;

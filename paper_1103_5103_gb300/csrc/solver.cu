@@ -885,8 +885,11 @@ extern "C" int wl_persistent_selftest(wl_gauge *g, int prec, int inject_missing_
 extern "C" int wl_vector_op(wl_gauge *g, int kind, int prec, int n_rhs, size_t rhs_stride, void *const *vecs,
                             const double *scal, double *dots, void *stream)
 {
-    const int nv = kind == WL_VEC_S ? 3 : kind == WL_VEC_XR ? 6 : kind == WL_VEC_P ? 3 : kind == WL_VEC_NORM2 ? 1 : 0;
-    if (!g || nv == 0 || !vecs || n_rhs < 1 || n_rhs > 64 || !valid_prec(prec) || prec == WL_DF ||
+    // WL_VEC_GUESS + k: a guess through k solutions
+    const int terms = kind >= WL_VEC_GUESS && kind <= WL_VEC_GUESS + 15 ? kind - WL_VEC_GUESS : -1;
+    const int nv = kind == WL_VEC_S ? 3 : kind == WL_VEC_XR ? 6 : kind == WL_VEC_P ? 3 : kind == WL_VEC_NORM2 ? 1
+                 : terms >= 0 ? 2 * terms + 3 : 0;
+    if (!g || nv == 0 || (terms >= 0 && prec != WL_F64) || !vecs || n_rhs < 1 || n_rhs > 64 || !valid_prec(prec) || prec == WL_DF ||
         (kind != WL_VEC_NORM2 && !scal) || ((kind == WL_VEC_XR || kind == WL_VEC_NORM2) && !dots)) {
         set_error("wl_vector_op: bad argument");
         return WL_ERR_ARG;
@@ -902,7 +905,7 @@ extern "C" int wl_vector_op(wl_gauge *g, int kind, int prec, int n_rhs, size_t r
         if (!vecs[k]) { set_error("wl_vector_op: NULL vector"); return WL_ERR_ARG; }
     std::lock_guard<std::mutex> lock(g->mu);
     cudaStream_t s = as_stream(stream);
-    Vec v[6];
+    Vec v[33];
     for (int k = 0; k < nv; ++k) {
         v[k].ptr = vecs[k];
         v[k].prec = prec;
@@ -911,6 +914,20 @@ extern "C" int wl_vector_op(wl_gauge *g, int kind, int prec, int n_rhs, size_t r
     }
     Scratch sc;
     WL_TRY(get_scratch(g, n_rhs, &sc, s));
+    if (terms >= 0) {
+        std::vector<double> c(64 * (size_t)n_rhs);
+        for (int r = 0; r < n_rhs; ++r)
+            for (int j = 0; j < terms; ++j) {
+                c[r * terms + j] = scal[2 * terms * r + j];
+                c[32 * n_rhs + r * terms + j] = scal[2 * terms * r + terms + j];
+            }
+        WL_CUDA_TRY(cudaMemcpyAsync(sc.coef, c.data(), sizeof(double) * c.size(), cudaMemcpyHostToDevice, s));
+        const Vec *in[31];
+        for (int j = 0; j < 2 * terms + 1; ++j) in[j] = &v[j];
+        WL_TRY(blas_guess_residual(geo, sc.coef, sc.coef + 32 * n_rhs, in, terms, v[nv - 2], v[nv - 1], s, false));
+        WL_CUDA_TRY(cudaStreamSynchronize(s));
+        return checked_result(WL_OK);
+    }
     std::vector<BiState> hs(n_rhs);
     for (int r = 0; r < n_rhs && kind != WL_VEC_NORM2; ++r) {
         BiState &b = hs[r];
