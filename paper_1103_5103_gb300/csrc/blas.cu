@@ -88,10 +88,14 @@ __global__ void __launch_bounds__(kBlock) k_xr_update(Geom g, Vec x, Vec p, Vec 
     if (q.i < g.Vh) {
         const double are = __ldcg(&S.alpha_re), aim = __ldcg(&S.alpha_im);
         const double ore = __ldcg(&S.omega_re), oim = __ldcg(&S.omega_im);
-        cx<R> pv[12], sv_[12], tv[12];
+        // FP32: rhat's loads ahead of the stores, which coherent loads do not
+        // pass (12 rhs on 24^3x64 433 -> 427 us); FP16 is slower so (3 rhs on
+        // 32^3x64 163 -> 198 us), FP64 has no registers for it
+        cx<R> pv[12], sv_[12], tv[12], rh[12];
         ld<P>(p, q.r, g.stride, q.i, pv);
         ld<P>(sv, q.r, g.stride, q.i, sv_);
         ld<P>(t, q.r, g.stride, q.i, tv);
+        if constexpr (P == WL_F32) ld<P>(rhat, q.r, g.stride, q.i, rh);
         {
             cx<RX> xv[12];
             SpinorIO<PX>::load(x.rhs(q.r), g.stride, q.i, xv);
@@ -108,8 +112,7 @@ __global__ void __launch_bounds__(kBlock) k_xr_update(Geom g, Vec x, Vec p, Vec 
 #pragma unroll
         for (int k = 0; k < 12; ++k) rv[k] = sv_[k] - om * tv[k];
         SpinorIO<P>::store_rounded(r.rhs(q.r), g.stride, q.i, rv);
-        cx<R> rh[12];
-        ld<P>(rhat, q.r, g.stride, q.i, rh);
+        if constexpr (P != WL_F32) ld<P>(rhat, q.r, g.stride, q.i, rh);
         cx<R> d = {R(0), R(0)};
         R n = R(0);
 #pragma unroll

@@ -89,7 +89,8 @@ void add_launches(long long n);
 // then waits until the predecessor has completed and its writes are visible.
 // Every such kernel calls chain_begin() first, in every block, and adds its
 // result (0) to the site index: the addresses of its loads then depend on
-// the wait, and none can be moved ahead of it.
+// the wait, and none can be moved ahead of it.  Fields are read with coherent
+// loads (ld_field): the kernel is resident while they are still written.
 //
 // Which launches: those of at most kChainBlocks blocks (about a wave) outside
 // stream capture, and of at most kChainCaptured inside.  wilson_dslash FP64
@@ -323,16 +324,46 @@ __device__ __forceinline__ void norm_acc(double &n, double x) { n = fma(x, x, n)
 template <typename R> struct NormT { using T = float; };
 template <> struct NormT<double> { using T = double; };
 
-// Vector loads: the read-only path (__ldg) for data that no block of the
-// running kernel writes; ordinary loads for data that other blocks of the
-// same (persistent) kernel rewrite between grid barriers -- after the
-// barrier's release/acquire fences those are coherent, the non-coherent
-// read-only path is not.
+// Loads of field data are coherent ones (ld.global).  The read-only path
+// (__ldg, ld.global.nc) is for data that nothing writes while the kernel is
+// resident: the links.  A field may still be written by the predecessor of a
+// chained kernel (launch_chained) after this one has started; what follows
+// griddepcontrol.wait sees it through coherent loads only.  Written as asm
+// without side effects, so that the compiler still batches loads ahead of
+// stores to other fields, as it does with __ldg.
+__device__ __forceinline__ float ld_field(const float *p)
+{
+    float v;
+    asm("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ uint4 ld_field(const uint4 *p)
+{
+    uint4 v;
+    asm("ld.global.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ float4 ld_field(const float4 *p)
+{
+    float4 v;
+    asm("ld.global.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ double2 ld_field(const double2 *p)
+{
+    double2 v;
+    asm("ld.global.v2.f64 {%0, %1}, [%2];" : "=d"(v.x), "=d"(v.y) : "l"(p));
+    return v;
+}
+
+// Vector loads: as above for data that no block of the running kernel
+// writes; ordinary ones, in program order, for data that other blocks of the
+// same (persistent) kernel rewrite between grid barriers.
 template <bool CG, typename T>
 __device__ __forceinline__ T ldx(const T *p)
 {
     if constexpr (CG) return *p;
-    else return __ldg(p);
+    else return ld_field(p);
 }
 
 template <typename To, typename From>

@@ -16,25 +16,39 @@
 
 namespace wl {
 
-__device__ __forceinline__ float4 ldv4(const void *p)
+// Links through the read-only path, fields through coherent loads (ld_field in
+// common.cuh says why).
+__device__ __forceinline__ float4 ldv4_link(const void *p)
 {
     float4 v;
     asm volatile("ld.global.nc.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p));
     return v;
 }
-__device__ __forceinline__ uint4 ldvu4(const void *p)
+__device__ __forceinline__ float4 ldv4_field(const void *p)
 {
-    uint4 v;
-    asm volatile("ld.global.nc.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
+    float4 v;
+    asm volatile("ld.global.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p));
     return v;
 }
-__device__ __forceinline__ uint2 ldvu2(const void *p)
+__device__ __forceinline__ uint4 ldvu4_field(const void *p)
+{
+    uint4 v;
+    asm volatile("ld.global.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ unsigned ldvu_field(const void *p)
+{
+    unsigned v;
+    asm volatile("ld.global.u32 %0, [%1];" : "=r"(v) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ uint2 ldvu2_link(const void *p)
 {
     uint2 v;
     asm volatile("ld.global.nc.v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "l"(p));
     return v;
 }
-__device__ __forceinline__ unsigned ldvu(const void *p)
+__device__ __forceinline__ unsigned ldvu_link(const void *p)
 {
     unsigned v;
     asm volatile("ld.global.nc.u32 %0, [%1];" : "=r"(v) : "l"(p));
@@ -51,9 +65,9 @@ template <> struct RawDir<WL_F32> {
         const float4 *l = reinterpret_cast<const float4 *>(lk) + WL_LOAD_IDX(li, stride, 3);
         const float4 *q = reinterpret_cast<const float4 *>(sp) + WL_LOAD_IDX(j, stride, 1);
 #pragma unroll
-        for (int k = 0; k < 3; ++k) u[k] = ldv4(l + (size_t)k * stride);
+        for (int k = 0; k < 3; ++k) u[k] = ldv4_link(l + (size_t)k * stride);
 #pragma unroll
-        for (int k = 0; k < 6; ++k) s[k] = ldv4(q + (size_t)k * stride);
+        for (int k = 0; k < 6; ++k) s[k] = ldv4_field(q + (size_t)k * stride);
     }
     __device__ __forceinline__ float get(cx<float> (&U)[9], cx<float> (&psi)[12]) const
     {
@@ -83,11 +97,11 @@ template <> struct RawDir<WL_F16> {
         const uint2 *l = reinterpret_cast<const uint2 *>(lk) + li;
         const uint4 *q = reinterpret_cast<const uint4 *>(sp) + j;
 #pragma unroll
-        for (int k = 0; k < 4; ++k) u[k] = ldvu2(l + (size_t)k * stride);
-        u8 = ldvu(reinterpret_cast<const unsigned *>(reinterpret_cast<const uint2 *>(lk) + (size_t)4 * stride) + li);
+        for (int k = 0; k < 4; ++k) u[k] = ldvu2_link(l + (size_t)k * stride);
+        u8 = ldvu_link(reinterpret_cast<const unsigned *>(reinterpret_cast<const uint2 *>(lk) + (size_t)4 * stride) + li);
 #pragma unroll
-        for (int k = 0; k < 3; ++k) s[k] = ldvu4(q + (size_t)k * stride);
-        n = ldvu(SpinorIO<WL_F16>::norms(sp, stride) + j);
+        for (int k = 0; k < 3; ++k) s[k] = ldvu4_field(q + (size_t)k * stride);
+        n = ldvu_field(SpinorIO<WL_F16>::norms(sp, stride) + j);
     }
     __device__ __forceinline__ float get(cx<float> (&U)[9], cx<float> (&psi)[12]) const
     {

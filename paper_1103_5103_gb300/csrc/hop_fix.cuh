@@ -73,8 +73,9 @@ __device__ __forceinline__ i64 fix_sar(i64 v, int s)
     return r;
 }
 
-// Loads that stay where they are written, ahead of the arithmetic.
-__device__ __forceinline__ int4 fix_ld(const int4 *p)
+// Loads that stay where they are written, ahead of the arithmetic: of links
+// through the read-only path, of fields coherent (ld_field).
+__device__ __forceinline__ int4 fix_ld_link(const int4 *p)
 {
     int4 v;
     asm volatile("ld.global.nc.v4.s32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
@@ -83,7 +84,7 @@ __device__ __forceinline__ int4 fix_ld(const int4 *p)
 __device__ __forceinline__ double2 fix_ld(const double2 *p)
 {
     double2 v;
-    asm volatile("ld.global.nc.v2.f64 {%0, %1}, [%2];" : "=d"(v.x), "=d"(v.y) : "l"(p));
+    asm volatile("ld.global.v2.f64 {%0, %1}, [%2];" : "=d"(v.x), "=d"(v.y) : "l"(p));
     return v;
 }
 
@@ -142,7 +143,7 @@ __device__ __forceinline__ void fix_load_link(int4 (&u)[9], const int4 *p, int c
 #pragma unroll
     for (int r = 0; r < 3; ++r)
 #pragma unroll
-        for (int k = 0; k < 3; ++k) u[3 * r + k] = fix_ld(p + (r * row + k * col));
+        for (int k = 0; k < 3; ++k) u[3 * r + k] = fix_ld_link(p + (r * row + k * col));
 }
 
 // One transporter of one colour vector: adds L psi (1 -/+ gamma_mu) for the
@@ -367,7 +368,7 @@ __device__ __forceinline__ void half_load(const void *base, int stride, int s, i
     const double2 *p = static_cast<const double2 *>(base) + i;
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
-        const double2 x = __ldg(p + (size_t)(3 * s + k) * stride), y = __ldg(p + (size_t)(3 * (3 - s) + k) * stride);
+        const double2 x = ld_field(p + (size_t)(3 * s + k) * stride), y = ld_field(p + (size_t)(3 * (3 - s) + k) * stride);
         v[k] = {x.x, x.y};
         v[3 + k] = {y.x, y.y};
     }

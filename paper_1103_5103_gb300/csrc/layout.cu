@@ -141,7 +141,7 @@ int make_vec(wl_gauge *g, const std::string &name, int prec, int nrhs, Vec *v)
 // ------------------------------------------------------------ layout kernels
 
 template <int P>
-__global__ void k_import(Geom g, const double2 *__restrict__ canon, void *out, int parity)
+__global__ void k_import(Geom g, const double2 *canon, void *out, int parity)
 {
     const int i = blockIdx.x * blockDim.x + threadIdx.x + chain_begin();
     if (i >= g.Vh) return;
@@ -242,7 +242,7 @@ __global__ void __launch_bounds__(kFullSites) k_export_full(Geom g, const void *
 }
 
 template <int P>
-__global__ void __launch_bounds__(kFullSites) k_import_full(Geom g, const double2 *__restrict__ canon, void *even,
+__global__ void __launch_bounds__(kFullSites) k_import_full(Geom g, const double2 *canon, void *even,
                                                             void *odd)
 {
     __shared__ double2 sm[12 * (kFullSites + 1)];
