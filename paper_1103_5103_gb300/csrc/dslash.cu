@@ -275,12 +275,15 @@ static int dslash_common(wl_gauge *g, const void *in, void *out, double kappa, i
     }
     WL_TRY(make_vec(g, "dslash_ie", prec, 1, &ie));
     WL_TRY(make_vec(g, "dslash_io", prec, 1, &io));
-    WL_TRY(make_vec(g, "dslash_oe", prec, 1, &oe));
-    WL_TRY(make_vec(g, "dslash_oo", prec, 1, &oo));
+    const bool canon = prec != WL_F64 && (op != WL_OP_MPREC || geo.Vh <= kCanonPrecSites) && device_fields(in, out);
+    if (!canon) {
+        WL_TRY(make_vec(g, "dslash_oe", prec, 1, &oe));
+        WL_TRY(make_vec(g, "dslash_oo", prec, 1, &oo));
+    }
     const void *cin[1] = {in};
     void *cout[1] = {out};
     WL_TRY(import_full(geo, cin, ie, io, s));
-    if (prec != WL_F64 && (op != WL_OP_MPREC || geo.Vh <= kCanonPrecSites) && device_fields(in, out)) {
+    if (canon) {
         CanonHop h{};
         for (int p = 0; p < 2; ++p) {
             h.a[p] = hop_args(g, op == WL_OP_MPREC ? oo : p ? ie : io, p);

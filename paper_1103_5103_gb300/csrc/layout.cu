@@ -86,6 +86,13 @@ int Workspace::get(const std::string &name, size_t bytes, void **out)
 {
     DevBuf &b = bufs[name];
     if (b.bytes < bytes) {
+        // allowed while a stream is being captured, as any allocation that the
+        // captured work does not depend on for its order
+        struct Relaxed {
+            cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+            Relaxed() { cudaThreadExchangeStreamCaptureMode(&mode); }
+            ~Relaxed() { cudaThreadExchangeStreamCaptureMode(&mode); }
+        } relaxed;
         if (b.ptr) cudaFree(b.ptr);
         b.ptr = nullptr;
         b.bytes = 0;
@@ -120,7 +127,10 @@ bool release_integer_links(wl_gauge *g)
 {
     std::lock_guard<std::mutex> lock(g->hop_mu);
     if (!g->fix_links[0] || g->captured) return false;
-    cudaDeviceSynchronize();
+    if (cudaDeviceSynchronize() != cudaSuccess) {   // (refused during a capture)
+        (void)cudaGetLastError();
+        return false;
+    }
     g->inner_graph.release();
     for (int par = 0; par < 2; ++par) {
         cudaFree(g->fix_links[par]);
