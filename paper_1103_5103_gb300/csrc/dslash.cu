@@ -250,9 +250,13 @@ static bool device_fields(const void *in, const void *out)
 // FP32, FP16 and double-float: whether the last hop stores to the canonical
 // field (device memory).  D and M, both parities in one launch, gain at every
 // size (FP32 8^4 15.2 -> 12.0 us, 16^4 28.7 -> 18.0, 24^3x64 211 -> 167; DF
-// 24^3x64 786 -> 619); M_prec, one parity after another, up to 16384 sites of
-// one (20x12x6x14 18.6 -> 16.8; 16^4 26.6 -> 29.8 us).
-constexpr int kCanonPrecSites = 16384;
+// 24^3x64 786 -> 619); M_prec, one parity after another, on lattices of up to
+// 16384 sites of one parity, in double-float 8192 (us, layout passes ->
+// canonical store, 8192 / 12288 / 16384 / 24576 / 32768 sites: FP32 16.8 ->
+// 14.7, 18.6 -> 17.4, 18.6 -> 18.3, 22.6 -> 22.1, 26.7 -> 29.2; FP16 16.8 ->
+// 13.9, 18.6 -> 16.5, 18.7 -> 17.8, 22.5 -> 19.6, 24.8 -> 30.8; DF 45.1 ->
+// 44.5, 51.3 -> 52.1, 53.3 -> 59.4, 65.9 -> 73.4, 75.8 -> 83.4).
+constexpr int canon_prec_sites(int prec) { return prec == WL_DF ? 8192 : 16384; }
 
 static int dslash_common(wl_gauge *g, const void *in, void *out, double kappa, int prec, int op, int dagger,
                          void *stream)
@@ -275,7 +279,7 @@ static int dslash_common(wl_gauge *g, const void *in, void *out, double kappa, i
     }
     WL_TRY(make_vec(g, "dslash_ie", prec, 1, &ie));
     WL_TRY(make_vec(g, "dslash_io", prec, 1, &io));
-    const bool canon = prec != WL_F64 && (op != WL_OP_MPREC || geo.Vh <= kCanonPrecSites) && device_fields(in, out);
+    const bool canon = prec != WL_F64 && (op != WL_OP_MPREC || geo.Vh <= canon_prec_sites(prec)) && device_fields(in, out);
     if (!canon) {
         WL_TRY(make_vec(g, "dslash_oe", prec, 1, &oe));
         WL_TRY(make_vec(g, "dslash_oo", prec, 1, &oo));

@@ -1,7 +1,8 @@
 """wilson_dslash in FP32, FP16 and double-float: the hop that stores to the
 canonical field against the layout passes, which page-locked host fields
-still take: the same values bit for bit, below, at and above the size where
-M_prec changes its route (16384 sites per parity: 8x16x16x16)."""
+still take: the same values bit for bit, below, at and above the sizes where
+M_prec changes its route (16384 sites per parity, 8x16x16x16; in double-float
+8192, 8x16x16x8)."""
 import numpy as np
 import pytest
 import torch
@@ -9,7 +10,8 @@ import torch
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("dims", [(2, 2, 2, 2), (6, 4, 2, 10), (8, 16, 16, 16), (8, 16, 16, 18)])
+@pytest.mark.parametrize("dims", [(2, 2, 2, 2), (6, 4, 2, 10), (8, 16, 16, 8), (8, 16, 16, 10), (8, 16, 16, 16),
+                                  (8, 16, 16, 18)])
 @pytest.mark.parametrize("prec", ["f32", "f16", "df"])
 def test_canonical_store_equals_export(dims, prec):
     from paper_1103_5103_gb300 import api, synth
