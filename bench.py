@@ -80,13 +80,13 @@ FLOP_SITE = 1320   # per hop output site and rhs
 # lattice sites of the captured case, bytes).  Traffic scales with sites.
 # An entry is valid only for the kernel as it was when captured; remove it
 # when that kernel changes.
-HOP_TRAFFIC = {("f16", 105, 3): (1048576, 617.61e6), ("f16", 106, 3): (1048576, 617.19e6),
-               ("f16", 8105, 3): (1048576, 617.64e6), ("f64", 6000, 3): (442368, 1012.35e6),
-               ("f64", 101, 3): (442368, 1013.01e6), ("f64", 103, 3): (442368, 1024.87e6)}
+HOP_TRAFFIC = {("f16", 105, 3): (1048576, 617.38e6), ("f16", 106, 3): (1048576, 617.41e6),
+               ("f16", 8105, 3): (1048576, 617.48e6), ("f64", 6000, 3): (442368, 1012.50e6),
+               ("f64", 101, 3): (442368, 1012.17e6), ("f64", 103, 3): (442368, 1021.01e6)}
 # pipe utilisation of the FP64 hop in the same captures
 FP64_PIPE = {(6000, 3): "29% busy, integer multiply-add pipe 70%, ALU 52%, issue 57% in an ncu capture of this "
                         "variant on 24^3x64, 3 rhs",
-             (101, 3): "92.6% busy in an ncu capture of this variant on 24^3x64, 3 rhs",
+             (101, 3): "92.7% busy in an ncu capture of this variant on 24^3x64, 3 rhs",
              (103, 3): "92.6% busy in an ncu capture of this variant on 24^3x64, 3 rhs"}
 # FP64 FMA rate of one GB300 (TFLOP/s, 2 flops per FMA): 152 SMs x 2 FP64
 # FMA per clock x 2.07 GHz, the unit count and clock of the part

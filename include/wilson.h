@@ -189,7 +189,7 @@ const char *wl_last_error(void);
 
 /* Create a lattice of extents dims = {X, Y, Z, T}.  Every extent must be even
  * and >= 2 (the even/odd split of Section 6.2.3 needs it) and the volume
- * below 2^31.  antiperiodic_t: 1 gives -1 on hops across the time boundary.
+ * below 2^31 / 12.  antiperiodic_t: 1 gives -1 on hops across the time boundary.
  * Host-only; no device work. */
 int wl_lattice_create(const int dims[4], int antiperiodic_t, wl_lattice **out);
 int wl_lattice_destroy(wl_lattice *lat);
@@ -257,7 +257,11 @@ int wilson_hop(wl_gauge *g, const void *in, void *out, const void *x, double coe
  * launch; rhs_block (1, 2 or 4) rhs are handled by one thread, which then
  * loads each link into registers once for all of them; rhs_block = 0 uses
  * the variant chosen by wl_autotune for (prec, n_rhs), or 1 if untuned; a
- * negative rhs_block selects the autotuner variant -rhs_block directly.
+ * negative rhs_block names a variant -rhs_block directly, one of those that
+ * tuning chooses from (FP32 8104, 105, 106, 205; FP16 105, 106, 8105;
+ * double-float 101, 103, 104) or an experiment that it does not, kept for
+ * comparison: 301 to 305 (prefetch), 401, 404 (four rhs per thread), 1104 to
+ * 1203 (cp.async staging), 5006 (paired sites), 9001 to 9104 (TMA staging).
  * FP64 hops run in block fixed point on the integer pipes for every
  * rhs_block >= 0, here and in every other call: the components of a site's
  * eight neighbours are 64-bit integers on one scale, and a component of the
@@ -291,8 +295,8 @@ int wilson_dslash_dag(wl_gauge *g, const void *in, void *out, double kappa, int 
  * running while another component owns the allocator (a caching allocator
  * with a hard cap, a pool that must not fragment, a loop that cannot take
  * cudaMalloc's implicit synchronisation).  The paper has no counterpart.
- * wilson_dslash takes four internal half-lattice spinors from the gauge
- * handle's workspace and allocates it on first use; this entry point takes
+ * wilson_dslash takes up to four internal half-lattice spinors from the gauge
+ * handle's workspace and allocates them on first use; this entry point takes
  * them from a fixed 64 MiB array compiled into the library (held by every
  * GPU that loads the library until the process exits) and calls no
  * cudaMalloc, cudaFree or allocating routine.  Lattices whose four
@@ -336,7 +340,9 @@ int bicgstab_solve(wl_gauge *g, const void *b, void *x, double m0, const wl_solv
  * a single-mass BiCGstab from x[i] (FP64 inner where the handle has FP64
  * links, else FP32 inner and outer_prec outer, which needs FP32 links: a
  * polish that finds neither returns WL_ERR_ARG in stats[i].status); its
- * extra iterations are counted in stats[i].restarts.  The shadow residual is p->shadow (NULL: b).
+ * extra iterations are counted in stats[i].restarts.  In FP64 the updates of
+ * the shifted vectors run on the integer pipes, with one scale per complex
+ * number: their error is relative to its larger part.  The shadow residual is p->shadow (NULL: b).
  * Returns WL_ERR_BREAKDOWN, with the polished solutions in x, when the
  * shifted recurrences broke down.  Masses must be distinct.  Synchronises
  * the stream. */
@@ -447,8 +453,8 @@ int wl_wait_faults(unsigned *count, int reset, void *stream);
  *                 multimass_solve; WL_F64 only; scal[2 k r ..] = c_0 ..
  *                 c_{k-1}, d_0 .. d_{k-1} of rhs r
  *                                     vecs x_0 .. x_{k-1}, y_0 .. y_{k-1}, b, x, r
- * Inner products: FP32 per site, FP32 within a warp, FP64 across warps and
- * blocks.  Synchronises the stream. */
+ * Inner products of FP32 and FP16 vectors: FP32 per site and within a block,
+ * FP64 across blocks; of FP64 vectors FP64.  Synchronises the stream. */
 #define WL_VEC_S     0
 #define WL_VEC_XR    1
 #define WL_VEC_P     2

@@ -92,13 +92,16 @@ void add_launches(long long n);
 // the wait, and none can be moved ahead of it.  Fields are read with coherent
 // loads (ld_field): the kernel is resident while they are still written.
 //
-// Which launches: those of at most kChainBlocks blocks (about a wave) outside
-// stream capture, and of at most kChainCaptured inside.  wilson_dslash FP64
-// 8^4 36.9 -> 28.4 us, FP32 20x12x6x14 28.7 -> 18.5 us (four or five kernels
-// of 4-12 us each); the captured solver iterations of 8^4 gain 3%, those of
-// 16^3x32 lose 6% (8.3 -> 8.8 ms: the programmatic edges of a graph cost more
-// than they hide), and long queues of large kernels lose most (24 exports and
-// imports with 8 hops of 24^3x64, 12 rhs: 3.9 -> 5.7 ms).
+// Which launches: those of at most kChainBlocks blocks (about a wave: eight on
+// each of the GB300's 152 SMs) outside stream capture, and of at most
+// kChainCaptured inside.  wilson_dslash FP64 8^4 36.9 -> 28.4 us, FP32
+// 20x12x6x14 28.7 -> 18.5 us (four or five kernels of 4-12 us each).  Captured
+// solver iterations (four masses, one source, by blocks per launch, ms without
+// -> with): 32 blocks 3.73 -> 3.48, 81 3.75 -> 3.66, 108 4.03 -> 3.99, 162 4.38
+// -> 4.35, 256 4.80 -> 4.85, 512 6.28 -> 6.59 (the programmatic edges of a
+// graph cost more than they hide): the line, at 128, lies on the side where
+// there is something to gain.  Long queues of large kernels lose most (24
+// exports and imports with 8 hops of 24^3x64, 12 rhs: 3.9 -> 5.7 ms).
 __device__ __forceinline__ int chain_begin()
 {
     int z;

@@ -7,6 +7,9 @@
 //    has scale S = e + e', units of 2^(S-2101), and is below 2^57 (a complex
 //    one below 2^58).  A component with exponent e is the same integer at
 //    scale e + 1020.
+// The error of a sum is relative to the modulus of its largest complex term,
+// as in complex arithmetic with complex coefficients; the smaller of re and im
+// does not keep 53 bits of its own.
 // Values outside the ranges below (zeros are inside) take FP64 arithmetic:
 // components 2^(-423..478), coefficients 2^(-200..201).
 #pragma once

@@ -5,11 +5,12 @@
 //
 // FP32 at 128 registers (four blocks per SM): 12 rhs on 24^3x64 386 -> 376 us,
 // 1 rhs 51.0 -> 49.3 us, 16^3x32 10.4 -> 9.8 us against the best of the other
-// kernels.  What bounds it on the large lattices is L2: 3.6-4.2 GB to L1 plus
-// 1.2 GB of fills and 0.5 GB of stores in 0.38 ms, 14-15 TB/s, where a plain
-// read of 64 MB out of L2 reaches 14.7 TB/s.  Sharing links between rhs in
-// neighbouring warps (L1 hits 19 -> 43%) and other depths and occupancies
-// ended within 5%.
+// kernels.  What bounds it on the large lattices is the latency of loads from
+// L2 under their own traffic: 4.5 GB from L2 to L1 in 0.38 ms, 11.8 TB/s,
+// where a plain read of 64 MB out of L2 reaches 14.5 TB/s (L2 to crossbar 43%
+// and 60% busy), with long-scoreboard stalls ahead of all others.  Sharing
+// links between rhs in neighbouring warps (L1 hits 19 -> 43%) and other depths
+// and occupancies ended within 5%.
 #pragma once
 
 #include "hop.cuh"
