@@ -431,8 +431,8 @@ int wl_autotune(wl_gauge *g, int prec, int n_rhs, void *stream, int *variant, do
  * for each tile's copies; a wait that does not complete within about a
  * second of clock cycles is counted here, and that block stops instead of
  * hanging.  Reads the counter into *count after synchronising the stream
- * and, with reset = 1, sets it back to zero.  Autotuning and the inner
- * solver check it and return WL_ERR_TIMEOUT when it is non-zero. */
+ * and, with reset = 1, sets it back to zero.  Tuning and the solvers do not
+ * run these variants; a caller that names one looks here. */
 int wl_wait_faults(unsigned *count, int reset, void *stream);
 
 /* One fused vector kernel of the BiCGstab iteration (Section 5: the vector

@@ -491,7 +491,7 @@ int hop_launch_tma(int prec, int variant, int dagger, const HopArgs &a, const Ep
     return st;
 }
 
-int wait_faults(unsigned *count, bool reset, cudaStream_t s)
+static int wait_faults(unsigned *count, bool reset, cudaStream_t s)
 {
     WL_CUDA_TRY(cudaMemcpyFromSymbolAsync(count, g_wait_faults, sizeof(unsigned), 0, cudaMemcpyDeviceToHost, s));
     WL_CUDA_TRY(cudaStreamSynchronize(s));

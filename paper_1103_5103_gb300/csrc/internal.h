@@ -214,8 +214,6 @@ int persistent_inner(wl_gauge *g, int prec, int nrhs, const Vec &r, const Vec &r
 // thread; rhs_block < 0 selects variant -rhs_block; 0 takes the tuned one.
 const std::vector<int> &hop_variants(int prec);
 int hop_variant_for(wl_gauge *g, int prec, int nrhs, int rhs_block);
-// Bounded device waits (TMA-staged hops) that gave up since the last reset.
-int wait_faults(unsigned *count, bool reset, cudaStream_t s);
 
 // Bounds-checked build: status of a synchronising C-ABI call, replaced by
 // WL_ERR_CHECKED when an out-of-range site index was recorded (the words are

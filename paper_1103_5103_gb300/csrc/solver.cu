@@ -377,15 +377,6 @@ static int run_inner(Inner &in, const wl_solver_params &prm, int max_iter, const
     }
     if (predict && status == WL_OK) in.pace = learn_pace(prog.data(), nrhs);
     std::memcpy(host_state.data(), hs, sizeof(BiState) * nrhs);
-    if (status == WL_OK && hop_variant_for(in.g, in.prec, nrhs, rb) >= 9000) {
-        // a TMA-staged hop that stopped waiting leaves its tile unwritten
-        unsigned faults = 0;
-        WL_TRY(wait_faults(&faults, true, s));
-        if (faults) {
-            set_error("inner solve: a TMA-staged hop gave up waiting for its copies");
-            return WL_ERR_TIMEOUT;
-        }
-    }
     return status;
 }
 

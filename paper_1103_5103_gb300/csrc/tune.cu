@@ -1,7 +1,7 @@
-// Project autotuner (spec batching item): for each (precision,
-// number of right-hand sides, lattice) it times the hop variants -- rhs per
-// thread and the minimum number of resident blocks requested from the
-// register allocator -- on the caller's stream with CUDA events, once, and
+// Autotuner of the hops: for each (precision, number of right-hand sides,
+// lattice) it times the candidate variants -- rhs per thread, the minimum
+// number of resident blocks requested from the register allocator, the order
+// of the loads -- on the caller's stream with CUDA events, once, and
 // caches the fastest in the gauge handle.  With WL_AUTOTUNE_CACHE set to a
 // file path the choices are also read from / appended to that file, keyed by
 // lattice extents, precision, rhs count and device name.
@@ -124,7 +124,6 @@ int autotune_hop(wl_gauge *g, int prec, int nrhs, cudaStream_t s, TuneResult *ou
         int st = WL_OK;
         for (int k = 0; k < 2 && st == WL_OK; ++k)
             st = hop_ex(g, in, o, nullptr, 0.0, nullptr, 0.0, 1.0, WL_ODD, 0, -v, nullptr, 0, s);
-        if (st == WL_ERR_ARG && v >= 9000 && v < 9300) continue;   // TMA tiles do not fit this lattice
         cudaEventRecord(e0, s);
         for (int k = 0; k < reps && st == WL_OK; ++k)
             st = hop_ex(g, in, o, nullptr, 0.0, nullptr, 0.0, 1.0, WL_ODD, 0, -v, nullptr, 0, s);
@@ -146,12 +145,6 @@ int autotune_hop(wl_gauge *g, int prec, int nrhs, cudaStream_t s, TuneResult *ou
     }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
-    unsigned faults = 0;
-    WL_TRY(wait_faults(&faults, true, s));
-    if (faults) {
-        set_error("autotune: a TMA-staged hop gave up waiting for its copies");
-        return WL_ERR_TIMEOUT;
-    }
     if (out) best.table = out->table;
     {
         std::lock_guard<std::mutex> lock(g->hop_mu);
