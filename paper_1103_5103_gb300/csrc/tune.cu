@@ -51,9 +51,11 @@ int hop_variant_for(wl_gauge *g, int prec, int nrhs, int rhs_block)
 // The variants that tuning times: those that were the fastest of
 // hop_variants() on some lattice and rhs count.  The others (cp.async and TMA
 // staging, paired sites, prefetch, four rhs per thread) are experiments that
-// callers can name: in solves they never were the fastest, some won a noisy
-// timing and then lost (TMA-staged 304 us per hop where 205 takes 247, 12 rhs
-// on 24^3x64), and each costs seven launches per handle.
+// callers can name: in solves they never were the fastest, and each costs
+// seven launches per handle.  The TMA-staged 9004 is ahead of 8104 in plain
+// FP32 hops of four rhs on some lattices (24^3x64 133 against 137 us, 16^3x64
+// 43.3 against 45.2; 32^3x64 410 against 310) but not where a solve skips
+// finished rhs: 24^3x64, four sources, eight masses 110.9 against 109.0 ms.
 static const std::vector<int> &tune_candidates(const wl_gauge *g, int prec)
 {
     static const std::vector<int> f32 = {8104, 105, 106, 205}, f16 = {105, 106, 8105}, fix = {6000},
