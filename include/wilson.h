@@ -259,9 +259,10 @@ int wilson_hop(wl_gauge *g, const void *in, void *out, const void *x, double coe
  * the variant chosen by wl_autotune for (prec, n_rhs), or 1 if untuned; a
  * negative rhs_block names a variant -rhs_block directly, one of those that
  * tuning chooses from (FP32 8104, 105, 106, 205; FP16 105, 106, 8105;
- * double-float 101, 103, 104) or an experiment that it does not, kept for
- * comparison: 301 to 305 (prefetch), 401, 404 (four rhs per thread), 1104 to
- * 1203 (cp.async staging), 5006 (paired sites), 9001 to 9104 (TMA staging).
+ * double-float 101, 103, 104), another register budget or rhs per thread of
+ * the same kernel (100 * rhs + blocks per SM), or an experiment that tuning
+ * does not run, kept for comparison: 301 to 305 (prefetch), 1104 to 1203
+ * (cp.async staging), 5006 (paired sites), 9001 to 9104 (TMA staging).
  * FP64 hops run in block fixed point on the integer pipes for every
  * rhs_block >= 0, here and in every other call: the components of a site's
  * eight neighbours are 64-bit integers on one scale, and a component of the
@@ -272,8 +273,8 @@ int wilson_hop(wl_gauge *g, const void *in, void *out, const void *x, double coe
  * it is a sum of small terms alone.  Links that keep colours apart (one with
  * an entry below 2^-30, such as unit or diagonal links), where whole colours
  * can be so, therefore run on the FP64 pipe.  The FP64-pipe hops (variants
- * 101, 103, 201, 7101 to 7202) and the fixed-point ones (6000 to 6002) can
- * be named on every handle. */
+ * 101, 103, 201, 7101 to 7202) can be named on every handle, the fixed-point
+ * ones (6000 to 6002) where it holds integer links. */
 int wilson_hop_multi(wl_gauge *g, const void *in, void *out, const void *x, double coef, int prec,
                      int out_parity, int dagger, int n_rhs, size_t rhs_stride, int rhs_block, void *stream);
 
